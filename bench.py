@@ -73,9 +73,9 @@ UPDATE_HEADER = ("gi_internal.cuh", "namespace gi {", "struct ResolveArgs {")
 NRC_ADAM_SECTION = ("gi_nrc.cu", "// ---------------------------------------------------------------- gradient scatter and Adam",
                     "// ---------------------------------------------------------------- query selection")
 NCU_TRAFFIC = {
-    # k_update, boxes-1080p (5th launch): 156.84 MB read + 31.24 MB written
-    "2:update": {"bytes_per_launch": 188079872, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
-                 "source_sha": "1af4e79846bba09c"},
+    # k_update, boxes-1080p (5th launch): 158.84 MB read + 33.20 MB written
+    "2:update": {"bytes_per_launch": 192040192, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
+                 "source_sha": "4125733ab0d02a56"},
     # k_nrc_adam_table, Cornell 1080p: 3.22 TB/s x 40.16 us
     "4:adam_table": {"bytes_per_launch": 129501000, "sources": (NRC_ADAM_SECTION,), "source_sha": "a33b80b7d73defb0"},
 }
@@ -627,9 +627,9 @@ def run_native(args, rank, world, local_rank):
         "update_atomic_floor": {
             "kernel": "k_diag_atomics (gi_diag_update_atomics)", "ms": floor_ms, "update_ms": float(pass_ms[1]),
             "update_over_floor": float(pass_ms[1]) / floor_ms, "touched_slots": floor_first,
-            "note": "the update's accumulation alone (bitmap form: one 32-byte bulk reduction of the sums and count "
-                    "plus a bitmap bit per hit) on a frame's own slot ids, nothing else, L2 flushed before each "
-                    "launch: the floor of k_update's accumulation"},
+            "note": "the accumulation of a table that accumulates by slot, alone (one 32-byte addition of the sums and "
+                    "count plus a bitmap bit per hit), on a frame's own slot ids, nothing else, L2 flushed before each "
+                    "launch; k_update adds into the shorter span of the recently touched cells' accumulators"},
         "roofline_window": {"achieved": sum(alg[n] for n in ("update", "resolve", "integrate")) /
                                         (pass_ms[1:4].sum() * 1e-3) / 1e9, "peak": peak, "unit": "GB/s"},
         "cpu_baseline": cpu,

@@ -87,14 +87,13 @@ typedef void *gi_stream_t; /* cudaStream_t */
  *   rebuild_load    fraction of slots occupied (live + stale cells) above which the
  *                   next update first compacts the table, in [0.25, 0.95]
  *   first_touch     how the update accumulates and records the slots touched since the
- *                   last resolve: GI_FIRST_TOUCH_LIST (per group of same-cell records of a warp,
- *                   three 64-bit additions and a returning count addition; the first toucher of
+ *                   last resolve: GI_FIRST_TOUCH_LIST (the record's sums and count added as one
+ *                   32-byte request, the count's addition returning; the first toucher of
  *                   a slot appends it to a list, staged per block), GI_FIRST_TOUCH_BITMAP (the
- *                   group's sums and count in one 32-byte bulk reduction from shared memory,
- *                   cp.reduce.async.bulk, and a non-returning set of the slot's bit in a bitmap
- *                   of one bit per slot that the resolve walks in slot order: fewer L2
- *                   operations per record), or GI_FIRST_TOUCH_AUTO (the bitmap).  Results are
- *                   identical.
+ *                   same without a returning addition, and a non-returning set of the slot's bit
+ *                   in a bitmap of one bit per slot that the resolve walks in slot order; tables
+ *                   of 2^22 slots and more keep the accumulators of recently touched cells side
+ *                   by side), or GI_FIRST_TOUCH_AUTO (the bitmap).  Results are identical.
  *   tiles           0: a slot holds one cell.  1: two-level cache of Section 2.2.3 ("Prefiltering
  *                   Radiance"): a slot holds a tile of 8 x 8 cells on the plane that drops the
  *                   direction code's axis (in-plane cell coordinates floor-divided by 8 form the
@@ -253,8 +252,9 @@ uint32_t gi_version(void);
 /*
  * Create a cache (Section 2.2.1): allocates the slot table (fingerprints,
  * 32-byte fixed-point accumulators, resolved radiance), a spare table for
- * compaction, the record of touched slots (a bitmap of one bit per slot, or a
- * touch list of 4 bytes per slot in the list form) and counters, on the
+ * compaction (from 2^22 slots on the second set of accumulators serves recently touched cells
+ * instead, with 4 bytes of stamp per slot and table), the record of touched slots (a bitmap of one
+ * bit per slot, or a touch list of 4 bytes per slot in the list form) and counters, on the
  * current CUDA device.  The library owns this memory until gi_cache_destroy.
  * Synchronous.
  * Errors: GI_ERR_INVALID_ARG (cfg out of range), GI_ERR_OOM, GI_ERR_CUDA.
@@ -772,11 +772,11 @@ gi_status gi_cell_means_noalloc(const gi_hits *hits, const gi_view *view, float 
  * Not a step of the path.  gi_cache_update ends, per hit record (GI_MERGE_NONE), in L2
  * operations on the cell's 32-byte accumulator (Section 2.2.1's accumulation in 64-bit fixed
  * point): in the list form (GI_FIRST_TOUCH_LIST) three 64-bit additions of the sums and one
- * returning 32-bit addition of the count, whose old value flags the first touch; in the bitmap
- * form (GI_FIRST_TOUCH_BITMAP, and AUTO) one 32-byte bulk reduction of the sums and count from
- * shared memory and a non-returning set of the slot's bit.  gi_diag_update_atomics issues exactly
+ * returning addition of the count, whose old value flags the first touch; in the bitmap
+ * form (GI_FIRST_TOUCH_BITMAP, and AUTO) the four additions as one 32-byte request and a
+ * non-returning set of the slot's bit.  gi_diag_update_atomics issues
  * those operations of the given form for n slot ids (records with slot_ids[i] >= 2^log2_slots are
- * skipped; one reduction per record, as the update without merge) and nothing else: no record
+ * skipped; one addition per record, as the update without merge) and nothing else: no record
  * stream, key, probe or slot-id store.  Timed beside gi_cache_update on the same frame's slot ids
  * it gives the floor of the update's accumulation on this GPU.
  *   slot_ids       device uint32[n] (4-byte aligned), e.g. the slot_ids_out of an update

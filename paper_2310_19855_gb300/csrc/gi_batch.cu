@@ -45,7 +45,7 @@ static DescLayout desc_layout(uint32_t n) {
     return L;
 }
 
-enum { kPassSpawn = 0, kPassUpdate, kPassResolve, kPassIntegrate, kPassInterp };
+enum { kPassSpawn = 0, kPassUpdate, kPassResolve, kPassIntegrate, kPassInterp, kDenseViews };
 
 } // namespace gi
 
@@ -151,7 +151,7 @@ static gi_status enqueue_frame(gi_batch_s *b, int set, const std::vector<uint32_
     if (s == GI_OK)
         s = launch_resolve_batched(reinterpret_cast<const ResolveArgs *>(d + L.res),
                                    reinterpret_cast<const uint32_t *>(d + L.pre[kPassResolve]), n,
-                                   blocks[kPassResolve], st);
+                                   blocks[kPassResolve], blocks[kDenseViews] != 0, st);
     // the views with a surrogate: query frame and probe pass with its answers, per view, on the
     // side streams (from the resolve on), beside one launch over the views without one (all of
     // them in the plain form; a view with a surrogate has no blocks in it)
@@ -354,7 +354,9 @@ gi_status gi_batch_frame(gi_batch_t b, const gi_batch_view *views, uint32_t use_
         reinterpret_cast<IntegrateArgs *>(h + L.integ)[v] = integrate_args(bv.cache, &bv.probes, bv.slot_ids, b->rpp, bv.env);
         reinterpret_cast<InterpArgs *>(h + L.interp)[v] = interp_args(&bv.gbuf, &bv.view, &bv.probes, bv.irradiance);
     }
-    std::vector<uint32_t> blocks(5);
+    std::vector<uint32_t> blocks(6);
+    for (uint32_t v = 0; v < n; ++v)  // views with a large table: the resolve's form is part of the graph
+        blocks[kDenseViews] += reinterpret_cast<const ResolveArgs *>(h + L.res)[v].rank ? 1u : 0u;
     for (int k = 0; k < 5; ++k) {
         blocks[k] = pre[k][n];
         pre[k][n + 1] = 0;  // the pass's work-item counter starts at zero every frame

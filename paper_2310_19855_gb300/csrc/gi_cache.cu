@@ -7,11 +7,21 @@
 //   accum    Accum[N]   {u64 sum r,g,b; u32 count; u32 stamp}, one 32-byte sector
 //   resolved float4[N]  (r, g, b, cold), or half4 with GI_RESOLVED_F16
 // plus a spare table of the same shape for compaction, a record of the slots touched
-// since the last resolve and a counter line.  The first touch of a cell (its count's
-// returning add sees 0) either sets the slot's bit in a bitmap (u32[N/32]), which the
-// resolve walks and clears in slot order, or is staged per block in shared memory and
-// appended to a touch list (u32[N]).  A cache whose accumulators exceed the L2 takes
-// the bitmap (slot-ordered resolve traffic), a smaller one the list (cheaper updates).
+// since the last resolve (a bitmap u32[N/32], which the resolve walks and clears in slot order, or
+// with GI_FIRST_TOUCH_LIST a touch list u32[N]) and a counter line.
+//
+// Large tables (bitmap form, 2^kDenseLog2Slots slots and more) spread a frame's scattered
+// accumulations over more memory than the L2 holds, and their cost follows that span (2.07 M
+// random additions of 32 bytes: 27 us over 2^20 slots, 53 us over 2^22, 80 us over 2^24, 86 us over
+// 2^25).  They therefore keep, beside `accum`:
+//   dense    Accum[N]        accumulators of the cells touched lately, side by side
+//   rank     RankWord[N/32]  which slots those are, the first one's place, the touched bits
+//   cold     u32[N/32]       the cold marks
+// and the stamps in the resolved float4's w, or with float16 storage in an array u32[N] (accum's stamp
+// field is unused).
+// Each resolve hands the cells touched since one to two aging periods (8 resolves) the next dense
+// accumulators; a cell outside them, new ones above all, accumulates in its own slot of `accum` until
+// the next resolve.  All accumulators are clear after a resolve, so nothing moves.
 //
 // A cell is the pair (home, fingerprint): probing runs are shorter than 256
 // slots, so a tag, which carries home mod 256, can only match within the run
@@ -67,32 +77,32 @@ __device__ __forceinline__ uint32_t probe_cell(const UpdateArgs &a, uint32_t hom
     return GI_SLOT_NONE;
 }
 
-// Touch list (a.bitmap NULL): three 64-bit reductions of the sums and a returning add of the
-// count, whose old value 0 marks the first touch of the cell this frame; first touches go to the
-// block's shared-memory list and then, once per block, to the touch list.
-// Bitmap: the group's sums and count in one 32-byte bulk reduction from the thread's 32-byte
-// shared-memory slot (rewritten only once its previous reduction has read it), and the slot's bit
-// set by a non-returning atomicOr.  The block's shared buffer is the first-touch list in the one
-// form and the reduction slots in the other.  The bulk reductions dominate the update's issue: at
-// 1080p it ran 60 us, 39 us without any accumulation and 44 us when only every fourth lane issued
-// its reduction (sums then wrong: bounds taken to size the cost).  A tensor-map reduction of four
-// rows per instruction (cp.reduce.async.bulk.tensor .tile::scatter4 .add.u64) compiles but wrote
-// the rows instead of adding them (every cell counted one sample), so it is not used.
+// Every hit's {r, g, b, count} waits in the thread's 32-byte shared-memory slot while its probe runs;
+// then the warp adds its 32 records four lanes a record (warp_add_accum), one coalesced request per
+// 32-byte sector.  (One 32-byte bulk reduction per hit, cp.reduce.async.bulk, costs the same at the
+// L2 but is issued lane after lane: 43 M warp instructions a frame at 1080p against 26 M, 67 us
+// against 62 us.)
+// Bitmap form: the slot's touched bit is set by a non-returning atomicOr; in a large table the rank
+// word that names the accumulator also holds the bit, and only a hit that reads it clear sets it.
+// With the dense accumulators 55 us at 1080p (2^22 slots), 281 us at 4K (2^24), against 67 and 370 us
+// with a bulk reduction by slot.  What bounds it now at 1080p is the SMs' request port to the L2
+// (69 % busy: a tag load, a rank load and an addition per record).
+// List form: the count's addition returns, and its old value 0 marks the first touch of the cell this
+// frame; first touches go to the block's shared-memory list and then, once per block, to the touch
+// list (1283 x 717 pixels, 2 rays a cell: 61 us against 71 us with three additions and a returning one
+// per lane).
 // MERGE: hits of a warp that name the same cell are merged first (__match_any_sync on the cell,
 // pointer-jumping sums), so one leader per cell probes and accumulates.  Without it every hit is
-// its own group: same-cell hits of a warp then reach the same accumulator in separate reductions,
+// its own group: same-cell hits of a warp then reach the same accumulator in separate additions,
 // whose integer sums are the same.  Probe rays of one warp belong to one probe and point in
 // different directions, so few of them share a cell: at 1080p the merge cost 9 us of the update
 // for ~5 % fewer reductions (update 72 us with it, 63 us without), and on the Cornell box at
 // 1080p 41 us against 38 us.  It stays available (GI_MERGE_WARP) for workloads whose warps do hit
 // the same cells.
-static_assert(kUpdBlockRecords * 4 == kUpdThreads * 32, "one 32-byte reduction slot per thread");
-template <int KEY_DIR, bool MERGE>
-__device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, uint32_t nblk) {
-    __shared__ __align__(32) unsigned long long s_buf[kUpdBlockRecords / 2];
-    uint32_t *s_touch = reinterpret_cast<uint32_t *>(s_buf);
-    unsigned long long *s_red = s_buf + 4 * threadIdx.x;
-    const bool bitmap = a.bitmap != nullptr;
+// s_acc: one 32-byte slot per thread; s_touch: the block's first touches (list form only, else NULL).
+template <int KEY_DIR, bool MERGE, bool BITMAP>
+__device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, uint32_t nblk,
+                                            unsigned long long *s_acc, uint32_t *s_touch) {
     __shared__ uint32_t s_n, s_base, s_clamped, s_maxp;
     if (threadIdx.x == 0) {
         s_n = 0;
@@ -101,6 +111,8 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
+    unsigned long long *s_red = s_acc + 4 * threadIdx.x;
+    const unsigned long long *s_warp = s_acc + 4 * (threadIdx.x & ~31u);
     const unsigned long long stride = (unsigned long long)nblk * kUpdThreads;
     uint32_t my_clamped = 0, my_maxp = 0;
     // far hits go to the surrogate while it is trusted (the decision of the whole launch)
@@ -129,8 +141,7 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
             r2 = __ldcs(a.rad[2] + i);
         }
         bool hit = inr && isfinite(len) && len >= 0.0f && isfinite3(px, py, pz);
-        const bool miss = inr && len == INFINITY;
-        bool far = false;
+        uint32_t code = inr && len == INFINITY ? GI_SLOT_MISS : GI_SLOT_NONE;  // slot id of a record without cell
         unsigned long long q0 = 0, q1 = 0, q2 = 0;
         uint32_t home = 0, tag = 0;
         if (hit) {
@@ -139,12 +150,21 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
             q1 = quantize(r1, bad);
             q2 = quantize(r2, bad);
             my_clamped += bad;
+            if (!MERGE) {
+                // the contribution waits in shared memory while the probe runs
+                s_red[0] = q0;
+                s_red[1] = q1;
+                s_red[2] = q2;
+                s_red[3] = 1ull;
+            }
             unsigned long long key =
                 cell_key(a.kp, px, py, pz, sx, sy, sz, len, KEY_DIR == GI_KEY_DIR_NORMAL ? 0u : 1u);
             cell_of_key(key, a.mask, home, tag);
             // the LOD sits in the descriptor's top bits
-            far = (uint32_t)(key >> 61) >= route_lod;
-            hit = !far;
+            if ((uint32_t)(key >> 61) >= route_lod) {
+                code = GI_SLOT_FAR;
+                hit = false;
+            }
         }
         uint32_t cnt = hit ? 1u : 0u;
         unsigned peers = 1u << lane;
@@ -170,41 +190,38 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
                     nxt = on;
                 }
             }
+            s_red[0] = q0;
+            s_red[1] = q1;
+            s_red[2] = q2;
+            s_red[3] = cnt;
         }
         const bool leader = hit && (peers & ((1u << lane) - 1u)) == 0u;
-        uint32_t slot = GI_SLOT_NONE;
+        uint32_t slot = GI_SLOT_NONE, loc = GI_SLOT_NONE;
         if (leader) {
             uint32_t k;
             slot = probe_cell(a, home, tag, k);
             my_maxp = max(my_maxp, k + 1u);
+            loc = slot;
             if (slot == GI_SLOT_NONE) {
                 atomicAdd(&a.ctr->dropped, (unsigned long long)cnt);
-            } else {
-                Accum *ac = a.accum + (size_t)slot * a.acc_stride;
-                if (bitmap) {
-                    bulk_wait_read();  // the previous reduction has read the slot
-                    s_red[0] = q0;
-                    s_red[1] = q1;
-                    s_red[2] = q2;
-                    s_red[3] = cnt;
-                    bulk_add_accum(ac, s_red);
-                    const uint32_t bit = 1u << (slot & 31u);
-                    atomicOr(a.bitmap + (slot >> 5), bit);
+            } else if (BITMAP) {
+                const uint32_t bit = 1u << (slot & 31u);
+                if (a.rank) {
+                    // the rank word's touched bits may be older than another block's; a bit seen set is set
+                    RankWord *rw = a.rank + (slot >> 5);
+                    const uint4 r = __ldcg(reinterpret_cast<const uint4 *>(rw));
+                    loc = accum_loc(r.x, r.y, slot);
+                    if (!(r.z & bit)) atomicOr(&rw->touched, bit);
                 } else {
-                    atomicAdd(&ac->sum[0], q0);
-                    atomicAdd(&ac->sum[1], q1);
-                    atomicAdd(&ac->sum[2], q2);
-                    // the count was cleared by the last resolve: the first adder this frame records the slot
-                    if (atomicAdd(&ac->count, cnt) == 0u) s_touch[atomicAdd(&s_n, 1u)] = slot;
+                    atomicOr(a.bitmap + (slot >> 5), bit);
                 }
             }
         }
         uint32_t my_slot = slot;
         if (MERGE) my_slot = __shfl_sync(kFull, slot, hit ? (__ffs(peers) - 1) : lane);
-        if (inr) __stcs(a.slot_ids + i, hit ? my_slot : (far ? GI_SLOT_FAR : (miss ? GI_SLOT_MISS : GI_SLOT_NONE)));
+        if (inr) __stcs(a.slot_ids + i, hit ? my_slot : code);
+        warp_add_accum<!BITMAP>(a.accum, a.dense, loc, s_warp, lane, s_touch, &s_n);
     }
-    // the bulk reductions complete (their sums visible) before the block ends
-    if (bitmap) bulk_wait_all();
     // block totals of the statistics, one global atomic each
     my_clamped = __reduce_add_sync(kFull, my_clamped);
     my_maxp = __reduce_max_sync(kFull, my_maxp);
@@ -214,30 +231,44 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (!bitmap) s_base = s_n ? atomicAdd(&a.ctr->touch_count, s_n) : 0u;
+        if (!BITMAP) s_base = s_n ? atomicAdd(&a.ctr->touch_count, s_n) : 0u;
         if (s_clamped) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamped);
         if (s_maxp) atomicMax(&a.ctr->max_probe, s_maxp);
     }
-    if (!bitmap) {
+    if (!BITMAP) {
         __syncthreads();
         for (uint32_t j = threadIdx.x; j < s_n; j += kUpdThreads) a.touch[s_base + j] = s_touch[j];
     }
 }
 
 template <int KEY_DIR, bool MERGE>
-__global__ void __launch_bounds__(kUpdThreads, 8) k_update(UpdateArgs a) {
-    update_body<KEY_DIR, MERGE>(a, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(kUpdThreads, MERGE ? 6 : 8) k_update(UpdateArgs a) {
+    __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
+    update_body<KEY_DIR, MERGE, true>(a, blockIdx.x, gridDim.x, s_acc, nullptr);
 }
 
-// the four instantiations of k_update on one stream
-static inline void launch_update(const UpdateArgs &a, uint32_t key_dir, bool merge, int blocks, cudaStream_t st) {
-    if (key_dir == GI_KEY_DIR_NORMAL) {
-        if (merge) k_update<GI_KEY_DIR_NORMAL, true><<<blocks, kUpdThreads, 0, st>>>(a);
-        else k_update<GI_KEY_DIR_NORMAL, false><<<blocks, kUpdThreads, 0, st>>>(a);
+// touch-list form: 6 blocks per SM (the returning count's path needs more than 32 registers)
+template <int KEY_DIR, bool MERGE>
+__global__ void __launch_bounds__(kUpdThreads, 6) k_update_list(UpdateArgs a) {
+    __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
+    __shared__ uint32_t s_touch[kUpdBlockRecords];
+    update_body<KEY_DIR, MERGE, false>(a, blockIdx.x, gridDim.x, s_acc, s_touch);
+}
+
+// the instantiations of k_update and k_update_list on one stream
+template <int KEY_DIR>
+static inline void launch_update_dir(const UpdateArgs &a, bool merge, int blocks, cudaStream_t st) {
+    if (a.bitmap || a.rank) {
+        if (merge) k_update<KEY_DIR, true><<<blocks, kUpdThreads, 0, st>>>(a);
+        else k_update<KEY_DIR, false><<<blocks, kUpdThreads, 0, st>>>(a);
     } else {
-        if (merge) k_update<GI_KEY_DIR_RAY, true><<<blocks, kUpdThreads, 0, st>>>(a);
-        else k_update<GI_KEY_DIR_RAY, false><<<blocks, kUpdThreads, 0, st>>>(a);
+        if (merge) k_update_list<KEY_DIR, true><<<blocks, kUpdThreads, 0, st>>>(a);
+        else k_update_list<KEY_DIR, false><<<blocks, kUpdThreads, 0, st>>>(a);
     }
+}
+static inline void launch_update(const UpdateArgs &a, uint32_t key_dir, bool merge, int blocks, cudaStream_t st) {
+    if (key_dir == GI_KEY_DIR_NORMAL) launch_update_dir<GI_KEY_DIR_NORMAL>(a, merge, blocks, st);
+    else launch_update_dir<GI_KEY_DIR_RAY>(a, merge, blocks, st);
 }
 
 // Grid of k_update: enough blocks that none takes more than kUpdBlockRecords records.
@@ -253,77 +284,82 @@ static inline int update_blocks(unsigned long long n) {
 // entries per lane and iteration, 4 blocks per SM.  (1080p: the bitmap form 34 us, against 44 us
 // when a thread walked its own word's bits 4 at a time with 3 blocks per SM: a word holds 0 to 32
 // touched slots, so those threads' chains were as uneven as their words.)
+// Large tables start at 2^22 slots (128 MB of accumulators, the size of the L2): there the frame's
+// update fell from 62 to 55 us and its resolve stayed at 34 us; at 2^24 the update fell from 370 to
+// 281 us and the resolve from 135 to 97 us (both 1 ray a cell, 1080p and 4K).  At 2^20 and 2^21 slots
+// (16 views) the rank loads cost what the shorter span gave.
+constexpr uint32_t kDenseLog2Slots = 22, kDenseAge = 8;
 constexpr int kResListUnroll = 2, kResListBlocksPerSm = 4;
 constexpr int kResBmUnroll = 2, kResBmBlocksPerSm = 4, kResBmWords = 16;
 // a table has at least 2^10 slots: its bitmap words are a whole number of chunks
 static_assert(((1u << 10) / 32u) % kResBmWords == 0, "bitmap chunk must divide the smallest table");
 
-// Resolve up to U touched slots (0xFFFFFFFF = none), their loads issued together: the
-// accumulator and, speculatively, the resolved history (a cell without history ignores it):
+// Resolve one touched slot whose accumulator (lo, hi) and resolved history (old) are loaded:
 // mean = sum / (count 2^24); a cell without history (never resolved, or evicted by an earlier
-// resolve) takes the mean, the others blend; accumulator cleared, stamp = frame + 1.
-template <int U>
-__device__ __forceinline__ void resolve_slots(const ResolveArgs &a, const uint32_t (&s)[U], uint32_t &fresh_new) {
-    uint4 lo[U], hi[U];
-    float3 old[U];
-    // accumulators leave the L2 first, resolved values last: the probe pass reads them next
-    const unsigned long long pfirst = l2_policy_evict_first(), plast = l2_policy_evict_last();
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if (s[u] != 0xFFFFFFFFu) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.accum + (size_t)s[u] * a.acc_stride);
-            lo[u] = ld_cg_hint(src, pfirst);
-            hi[u] = ld_cg_hint(src + 1, pfirst);
-            old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
-        }
+// resolve) takes the mean, the others blend.
+template <bool DENSE>
+__device__ __forceinline__ bool resolve_cell(const ResolveArgs &a, uint32_t s, uint32_t stamp, const uint4 &lo,
+                                             const uint4 &hi, const float3 &o, unsigned long long plast,
+                                             uint32_t &fresh_new) {
+    // no history: never resolved, or evicted by an earlier resolve (untouched E frames)
+    const bool fresh = stamp == 0u || (a.has_lr && (a.lr - (stamp - 1u)) >= a.evict);
+    const unsigned long long s0 = ((unsigned long long)lo.y << 32) | lo.x;
+    const unsigned long long s1 = ((unsigned long long)lo.w << 32) | lo.z;
+    const unsigned long long s2 = ((unsigned long long)hi.y << 32) | hi.x;
+    // mean = sum / (count 2^24): one reciprocal, three products (within an ulp of the quotient)
+    const float rc = __frcp_rn((float)hi.z) * 5.9604644775390625e-8f;
+    const float3 m = make_float3(__ull2float_rn(s0) * rc, __ull2float_rn(s1) * rc, __ull2float_rn(s2) * rc);
+    fresh_new += stamp == 0u ? 1u : 0u;
+    float3 v = m;
+    if (!fresh) v = make_float3(o.x + a.alpha * (m.x - o.x), o.y + a.alpha * (m.y - o.y), o.z + a.alpha * (m.z - o.z));
+    if (!a.f16) {
+        // 4th lane: the cold mark, in a large table the stamp
+        st_hint(reinterpret_cast<uint4 *>(static_cast<char *>(a.resolved) + (size_t)s * a.res_stride),
+                make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z),
+                           DENSE ? a.stamp_now : __float_as_uint(fresh ? 1.0f : 0.0f)),
+                plast);
+    } else {
+        store_resolved(a.resolved, a.res_stride, a.f16, s, v, fresh);
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if (s[u] == 0xFFFFFFFFu) continue;
-        const uint32_t stamp = hi[u].w;
-        // no history: never resolved, or evicted by an earlier resolve (untouched E frames)
-        const bool fresh = stamp == 0u || (a.has_lr && (a.lr - (stamp - 1u)) >= a.evict);
-        const unsigned long long s0 = ((unsigned long long)lo[u].y << 32) | lo[u].x;
-        const unsigned long long s1 = ((unsigned long long)lo[u].w << 32) | lo[u].z;
-        const unsigned long long s2 = ((unsigned long long)hi[u].y << 32) | hi[u].x;
-        // mean = sum / (count 2^24): one reciprocal, three products (within an ulp of the quotient)
-        const float rc = __frcp_rn((float)hi[u].z) * 5.9604644775390625e-8f;
-        const float3 m = make_float3(__ull2float_rn(s0) * rc, __ull2float_rn(s1) * rc, __ull2float_rn(s2) * rc);
-        fresh_new += stamp == 0u ? 1u : 0u;
-        float3 v = m;
-        if (!fresh) {
-            const float3 o = old[u];
-            v = make_float3(o.x + a.alpha * (m.x - o.x), o.y + a.alpha * (m.y - o.y), o.z + a.alpha * (m.z - o.z));
-        }
-        if (!a.f16) {
-            st_hint(reinterpret_cast<uint4 *>(static_cast<char *>(a.resolved) + (size_t)s[u] * a.res_stride),
-                    make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z),
-                               __float_as_uint(fresh ? 1.0f : 0.0f)),
-                    plast);
-        } else {
-            store_resolved(a.resolved, a.res_stride, a.f16, s[u], v, fresh);
-        }
-        // the cleared accumulator is next read by the next frame's update
-        uint4 *dst = reinterpret_cast<uint4 *>(a.accum + (size_t)s[u] * a.acc_stride);
-        st_hint(dst, make_uint4(0u, 0u, 0u, 0u), pfirst);
-        st_hint(dst + 1, make_uint4(0u, 0u, 0u, a.stamp_now), pfirst);
-    }
+    return fresh;
 }
 
-// touch-list form: U list entries per thread and iteration
+// touch-list form: U list entries per thread and iteration, their accumulators (which also hold the
+// stamp) and, speculatively, resolved histories loaded together; the accumulator is cleared behind
+// the loads and its stamp set to frame + 1
 template <int U>
 __device__ __forceinline__ void resolve_list_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
     const uint32_t n = __ldcg(&a.ctr->touch_count);
     const uint32_t stride = nblk * kResThreads;
     uint32_t fresh_new = 0;
+    // accumulators leave the L2 first, resolved values last: the probe pass reads them next
+    const unsigned long long pfirst = l2_policy_evict_first(), plast = l2_policy_evict_last();
     for (uint32_t i0 = blk * kResThreads + threadIdx.x; i0 < n; i0 += U * stride) {
         uint32_t s[U];
+        uint4 lo[U], hi[U];
+        float3 old[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const uint32_t i = i0 + u * stride;
             s[u] = i < n ? __ldcs(a.touch + i) : 0xFFFFFFFFu;
         }
-        resolve_slots<U>(a, s, fresh_new);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (s[u] != 0xFFFFFFFFu) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.accum + s[u]);
+                lo[u] = ld_cg_hint(src, pfirst);
+                hi[u] = ld_cg_hint(src + 1, pfirst);
+                old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (s[u] == 0xFFFFFFFFu) continue;
+            resolve_cell<false>(a, s[u], hi[u].w, lo[u], hi[u], old[u], plast, fresh_new);
+            uint4 *dst = reinterpret_cast<uint4 *>(a.accum + s[u]);
+            st_hint(dst, make_uint4(0u, 0u, 0u, 0u), pfirst);
+            st_hint(dst + 1, make_uint4(0u, 0u, 0u, a.stamp_now), pfirst);
+        }
     }
     resolve_finish(a.ctr, a.occ_out, a.stamp_now, nblk * (kResThreads / 32), fresh_new);
 }
@@ -332,47 +368,123 @@ __device__ __forceinline__ void resolve_list_body(const ResolveArgs &a, uint32_t
 // slots of their set bits in slot order to its shared list (a prefix sum of the words' bit counts
 // over the lanes gives each lane its place) and resolves the list U entries per lane at a time:
 // every lane gets the same share of the warp's touched slots whatever the words hold.
-template <int U>
+// DENSE: the accumulators of the cells in the chunk's rank words lie side by side (warp after warp in
+// the order the previous resolve handed them out), the stamps in an array of their own; the cells
+// touched lately (not since one to two aging periods) get the next dense accumulators.
+template <int U, bool DENSE>
 __device__ __forceinline__ void resolve_bm_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
-    __shared__ uint32_t s_list[kResThreads / 32][kResBmWords * 32];
+    __shared__ uint16_t s_list[kResThreads / 32][kResBmWords * 32];
+    __shared__ uint32_t s_loc[DENSE ? kResThreads / 32 : 1][DENSE ? kResBmWords * 32 : 1];
+    __shared__ uint32_t s_cold[DENSE ? kResThreads / 32 : 1][kResBmWords];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nw = nblk * (kResThreads / 32);
     const uint32_t chunks = a.words / kResBmWords;
     uint32_t fresh_new = 0;
+    // accumulators by slot leave the L2 first, resolved values last: the probe pass reads them next
+    const unsigned long long pfirst = l2_policy_evict_first(), plast = l2_policy_evict_last();
     for (uint32_t c = blk * (kResThreads / 32) + warp; c < chunks; c += nw) {
-        const uint32_t wi = c * kResBmWords + lane;
-        uint32_t bits = lane < kResBmWords ? __ldcg(a.bitmap + wi) : 0u;
-        if (bits) a.bitmap[wi] = 0u;
-        const int cnt = __popc(bits);
-        int incl = cnt;
+        const uint32_t wi = c * kResBmWords + lane, slot0 = c * (kResBmWords * 32);
+        const bool mine = lane < kResBmWords;
+        uint4 rk = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t cold = 0;
+        if (DENSE && mine) {
+            rk = __ldcg(reinterpret_cast<const uint4 *>(a.rank + wi));
+            cold = __ldcg(a.cold + wi) & ~rk.z;  // of the untouched cells
+            s_cold[warp][lane] = 0u;
+        }
+        uint32_t bits = DENSE ? rk.z : (mine ? __ldcg(a.bitmap + wi) : 0u);
+        if (!DENSE && bits) a.bitmap[wi] = 0u;
+        const uint32_t recent = rk.w | bits, keep = a.age ? recent : (rk.x | bits);
+        const int cnt = __popc(bits), kcnt = DENSE ? __popc(keep) : 0;
+        int incl = cnt | (kcnt << 16);  // both prefix sums at once (at most 512 each)
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const int t = __shfl_up_sync(kFull, incl, d);
             if (lane >= d) incl += t;
         }
-        const int total = __shfl_sync(kFull, incl, 31);
-        int pos = incl - cnt;
+        const int totals = __shfl_sync(kFull, incl, 31);
+        const int total = totals & 0xFFFF;
+        uint32_t base = 0;
+        if (DENSE && lane == 0 && (totals >> 16)) base = atomicAdd(&a.ctr->dense_next, (uint32_t)(totals >> 16));
+        int pos = (incl & 0xFFFF) - cnt;
         while (bits) {
-            s_list[warp][pos++] = wi * 32u + (uint32_t)(__ffs(bits) - 1);
+            const uint32_t b = (uint32_t)(__ffs(bits) - 1);
+            s_list[warp][pos] = (uint16_t)(32u * lane + b);
+            if (DENSE) s_loc[warp][pos] = accum_loc(rk.x, rk.y, wi * 32u + b);
+            ++pos;
             bits &= bits - 1u;
         }
         __syncwarp();
         for (int k = lane; k < total; k += 32 * U) {
-            uint32_t sl[U];
+            uint32_t s[U], loc[U], stamp[U];
+            uint4 lo[U], hi[U];
+            float3 old[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int idx = k + 32 * u;
-                sl[u] = idx < total ? s_list[warp][idx] : 0xFFFFFFFFu;
+                s[u] = 0xFFFFFFFFu;
+                if (idx < total) {
+                    s[u] = slot0 + s_list[warp][idx];
+                    if (DENSE) {
+                        loc[u] = s_loc[warp][idx];
+                        const uint4 *src = reinterpret_cast<const uint4 *>(accum_at(a.accum, a.dense, loc[u]));
+                        lo[u] = __ldcg(src);
+                        hi[u] = __ldcg(src + 1);
+                    } else {
+                        const uint4 *src = reinterpret_cast<const uint4 *>(a.accum + s[u]);
+                        lo[u] = ld_cg_hint(src, pfirst);
+                        hi[u] = ld_cg_hint(src + 1, pfirst);
+                        stamp[u] = hi[u].w;
+                    }
+                    // the history is read speculatively: a cell without one ignores it
+                    if (DENSE && !a.f16) {
+                        const float4 v = __ldcg(static_cast<const float4 *>(a.resolved) + s[u]);
+                        old[u] = make_float3(v.x, v.y, v.z);
+                        stamp[u] = __float_as_uint(v.w);
+                    } else {
+                        if (DENSE) stamp[u] = __ldcg(a.stamps + s[u]);
+                        old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
+                    }
+                }
             }
-            resolve_slots<U>(a, sl, fresh_new);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (s[u] == 0xFFFFFFFFu) continue;
+                const bool fresh = resolve_cell<DENSE>(a, s[u], stamp[u], lo[u], hi[u], old[u], plast, fresh_new);
+                if (DENSE) {
+                    if (fresh) atomicOr(&s_cold[warp][(s[u] >> 5) % kResBmWords], 1u << (s[u] & 31u));
+                    uint4 *dst = reinterpret_cast<uint4 *>(accum_at(a.accum, a.dense, loc[u]));
+                    dst[0] = make_uint4(0u, 0u, 0u, 0u);
+                    dst[1] = make_uint4(0u, 0u, 0u, 0u);
+                    if (a.f16) a.stamps[s[u]] = a.stamp_now;
+                } else {
+                    // the cleared accumulator is next read by the next frame's update
+                    uint4 *dst = reinterpret_cast<uint4 *>(a.accum + s[u]);
+                    st_hint(dst, make_uint4(0u, 0u, 0u, 0u), pfirst);
+                    st_hint(dst + 1, make_uint4(0u, 0u, 0u, a.stamp_now), pfirst);
+                }
+            }
+        }
+        if (DENSE) {
+            __syncwarp();
+            base = __shfl_sync(kFull, base, 0);
+            if (mine) {
+                *reinterpret_cast<uint4 *>(a.rank + wi) =
+                    make_uint4(keep, base + (uint32_t)((incl >> 16) - kcnt), 0u, a.age ? 0u : recent);
+                if (rk.z) a.cold[wi] = cold | s_cold[warp][lane];
+            }
         }
         __syncwarp();
     }
     resolve_finish(a.ctr, a.occ_out, a.stamp_now, nw, fresh_new);
 }
 
+// DENSE: some view of the batch has a large table (a batch without one keeps clear of that form's
+// registers, which spill beside the others').
+template <bool DENSE>
 __device__ __forceinline__ void resolve_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
-    if (a.bitmap) resolve_bm_body<kResBmUnroll>(a, blk, nblk);
+    if (DENSE && a.rank) resolve_bm_body<1, true>(a, blk, nblk);
+    else if (a.bitmap) resolve_bm_body<kResBmUnroll, false>(a, blk, nblk);
     else resolve_list_body<kResListUnroll>(a, blk, nblk);
 }
 
@@ -380,7 +492,10 @@ __global__ void __launch_bounds__(kResThreads, kResListBlocksPerSm) k_resolve(Re
     resolve_list_body<kResListUnroll>(a, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_bitmap(ResolveArgs a) {
-    resolve_bm_body<kResBmUnroll>(a, blockIdx.x, gridDim.x);
+    resolve_bm_body<kResBmUnroll, false>(a, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_dense(ResolveArgs a) {
+    resolve_bm_body<kResBmUnroll, true>(a, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------- queries
@@ -422,7 +537,7 @@ __global__ void k_query_points(UpdateArgs a, const void *resolved, uint32_t res_
                 const uint32_t t = word_tag(__ldg(a.tags + s));
                 if (t == kEmpty) break;
                 if (t == tag) {
-                    if (answers(__ldg(&a.accum[(size_t)s * a.acc_stride].stamp), rule)) {
+                    if (answers(__ldg(a.stamps + (size_t)s * a.stamp_stride), rule)) {
                         float3 v = load_resolved(resolved, res_stride, f16, s);
                         o = make_float4(v.x, v.y, v.z, 1.0f);
                     }
@@ -438,16 +553,18 @@ __global__ void k_query_points(UpdateArgs a, const void *resolved, uint32_t res_
 // ---------------------------------------------------------------- compaction
 // Re-insert every live cell of the current table into the clean spare table
 // (home recovered from the slot and the tag's low byte) and clear the current
-// table behind it, so that it is clean when it becomes the spare.
-__global__ void k_rebuild(SlotWord *old_tags, Accum *old_acc, const void *old_res, SlotWord *new_tags, Accum *new_acc,
-                          void *new_res, uint32_t res_bytes, uint32_t mask, uint32_t max_probe, LiveRule rule,
-                          Counters *ctr) {
+// table behind it, so that it is clean when it becomes the spare.  Runs right after a
+// resolve, when every accumulator is clear.  old_cold: large tables, else NULL.
+__global__ void k_rebuild(SlotWord *old_tags, uint32_t *old_stamps, const void *old_res, SlotWord *new_tags,
+                          uint32_t *new_stamps, void *new_res, uint32_t stamp_stride, uint32_t res_bytes,
+                          const uint32_t *old_cold, uint32_t *new_cold, uint32_t mask, uint32_t max_probe,
+                          LiveRule rule, Counters *ctr) {
     uint32_t live = 0, dropped = 0;
     const uint32_t N = mask + 1u;
     for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < N; s += gridDim.x * blockDim.x) {
         const uint32_t t = word_tag(old_tags[s]);
         if (t == kEmpty) continue;
-        const uint32_t stamp = old_acc[s].stamp;
+        const uint32_t stamp = old_stamps[(size_t)s * stamp_stride];
         if (answers(stamp, rule)) {
             const uint32_t home = (s - ((s - (t & 0xFFu)) & 0xFFu)) & mask;
             uint32_t ns = home, k = 0;
@@ -456,7 +573,8 @@ __global__ void k_rebuild(SlotWord *old_tags, Accum *old_acc, const void *old_re
                 ns = (ns + 1u) & mask;
             }
             if (k < max_probe) {
-                new_acc[ns].stamp = stamp;
+                new_stamps[(size_t)ns * stamp_stride] = stamp;
+                if (old_cold && ((old_cold[s >> 5] >> (s & 31u)) & 1u)) atomicOr(new_cold + (ns >> 5), 1u << (ns & 31u));
                 if (res_bytes == 8)
                     reinterpret_cast<uint2 *>(new_res)[ns] = reinterpret_cast<const uint2 *>(old_res)[s];
                 else
@@ -466,9 +584,7 @@ __global__ void k_rebuild(SlotWord *old_tags, Accum *old_acc, const void *old_re
                 ++dropped;
             }
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(old_acc + s);
-        dst[0] = make_uint4(0u, 0u, 0u, 0u);
-        dst[1] = make_uint4(0u, 0u, 0u, 0u);
+        old_stamps[(size_t)s * stamp_stride] = 0u;
         old_tags[s] = kEmpty;
     }
     live = __reduce_add_sync(kFull, live);
@@ -480,14 +596,17 @@ __global__ void k_rebuild(SlotWord *old_tags, Accum *old_acc, const void *old_re
 }
 
 // ---------------------------------------------------------------- table scan for stats
-__global__ void k_scan_stats(const SlotWord *tags, const Accum *acc, const uint32_t *bitmap, uint32_t N, LiveRule rule,
+// acc: list-form caches (a touched cell has a count); the others have the bitmap.
+__global__ void k_scan_stats(const SlotWord *tags, const Accum *acc, const uint32_t *stamps, uint32_t stamp_stride,
+                             const uint32_t *bitmap, uint32_t bitmap_stride, uint32_t N, LiveRule rule,
                              unsigned long long *out /* occupied, live, touched */) {
     unsigned long long occ = 0, live = 0, touched = 0;
     for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < N; s += gridDim.x * blockDim.x) {
-        if (bitmap && (s & 31u) == 0u) touched += __popc(bitmap[s >> 5]);
+        if (bitmap && (s & 31u) == 0u) touched += __popc(bitmap[(size_t)(s >> 5) * bitmap_stride]);
         if (word_tag(tags[s]) == kEmpty) continue;
         ++occ;
-        if (acc[s].count > 0u || answers(acc[s].stamp, rule)) ++live;
+        const bool touch = bitmap ? ((bitmap[(size_t)(s >> 5) * bitmap_stride] >> (s & 31u)) & 1u) != 0u : acc[s].count > 0u;
+        if (touch || answers(stamps[(size_t)s * stamp_stride], rule)) ++live;
     }
     for (int o = 16; o; o >>= 1) {
         occ += __shfl_xor_sync(kFull, occ, o);
@@ -509,13 +628,19 @@ template <int KEY_DIR>
 __global__ void __launch_bounds__(kUpdThreads, 6) k_update_batched(const UpdateArgs *args, const uint32_t *prefix,
                                                                    uint32_t nviews) {
     __shared__ UpdateArgs sa;
-    GI_BATCHED_ITEMS(prefix, nviews, sa, args, (update_body<KEY_DIR, false>(sa, item, items)));
+    __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
+    __shared__ uint32_t s_touch[kUpdBlockRecords];
+    GI_BATCHED_ITEMS(prefix, nviews, sa, args, {
+        if (sa.bitmap || sa.rank) update_body<KEY_DIR, false, true>(sa, item, items, s_acc, nullptr);
+        else update_body<KEY_DIR, false, false>(sa, item, items, s_acc, s_touch);
+    });
 }
 
+template <bool DENSE>
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_batched(const ResolveArgs *args, const uint32_t *prefix,
                                                                     uint32_t nviews) {
     __shared__ ResolveArgs sa;
-    GI_BATCHED_ITEMS(prefix, nviews, sa, args, resolve_body(sa, item, items));
+    GI_BATCHED_ITEMS(prefix, nviews, sa, args, resolve_body<DENSE>(sa, item, items));
 }
 
 uint32_t update_blocks_for(unsigned long long n, uint32_t records_per_block) {
@@ -537,10 +662,14 @@ gi_status launch_update_batched(const UpdateArgs *args, const uint32_t *prefix, 
 }
 
 gi_status launch_resolve_batched(const ResolveArgs *args, const uint32_t *prefix, uint32_t nviews, uint32_t blocks,
-                                 cudaStream_t st) {
+                                 bool dense, cudaStream_t st) {
     if (blocks == 0) return GI_OK;
-    k_resolve_batched<<<resident_grid(k_resolve_batched, kResThreads, blocks), kResThreads, 0, st>>>(args, prefix,
-                                                                                                    nviews);
+    if (dense)
+        k_resolve_batched<true><<<resident_grid(k_resolve_batched<true>, kResThreads, blocks), kResThreads, 0, st>>>(
+            args, prefix, nviews);
+    else
+        k_resolve_batched<false><<<resident_grid(k_resolve_batched<false>, kResThreads, blocks), kResThreads, 0, st>>>(
+            args, prefix, nviews);
     return cuda_status(cudaGetLastError(), "k_resolve_batched launch");
 }
 
@@ -560,8 +689,11 @@ struct gi_cache_s {
     int cur;
     bool tiles;                  // two-level cache: a slot holds a tile of 64 cells
     uint32_t cells;              // addressable cells: N, or 64 N for tiles
-    uint32_t *stamp[2];          // tiles: per-cell stamps, state, MIP values (gi_tiles.cu)
-    float4 *state[2];
+    uint32_t *stamp[2];          // tiles, large float16 tables: stamps (see stamps_of)
+    gi::Accum *dense;            // large tables: accumulators of the cells in `rank`
+    gi::RankWord *rank;          // large tables: touched slots and slots with a dense accumulator
+    uint32_t *cold[2];           // large tables: cells whose last resolve found no history
+    float4 *state[2];            // tiles: per-cell state, MIP values (gi_tiles.cu)
     float4 *mips[2];
     unsigned long long *omask[2];
     unsigned long long *tmask;   // tiles: cells touched since the last resolve
@@ -569,7 +701,7 @@ struct gi_cache_s {
     uint32_t *tlist;             // tiles: tile of each accumulator block
     int tres_blocks;
     uint32_t *touch;
-    uint32_t *bitmap;            // touched slots since the last resolve, one bit each
+    uint32_t *bitmap;            // touched slots since the last resolve, one bit each (large tables: in `rank`)
     gi::Counters *ctr;
     volatile uint32_t *occ_host; // mapped pinned {occupied, stamp of the resolve that wrote it}
     uint32_t *occ_dev;           // its device address
@@ -590,6 +722,7 @@ CacheView cache_view(gi_cache_t c) {
     v.resolved_stride = c->res_bytes;
     v.resolved_f16 = c->cfg.resolved_format == GI_RESOLVED_F16;
     v.slots = c->cells;
+    v.cold = c->cold[c->cur];
     return v;
 }
 
@@ -604,6 +737,19 @@ static TileArrays tile_arrays(const gi_cache_s *c, int k) {
     t.omask = c->omask[k];
     return t;
 }
+
+// The stamps of table k (slot s at s * stamp_stride): the accumulators', or in a large table the 4th
+// word of the resolved float4, or (float16 storage) an array of their own.
+static uint32_t *stamps_of(const gi_cache_s *c, int k) {
+    if (!c->rank) return &c->accum[k]->stamp;
+    return c->stamp[k] ? c->stamp[k] : static_cast<uint32_t *>(c->resolved[k]) + 3;
+}
+static uint32_t stamp_stride(const gi_cache_s *c) {
+    if (!c->rank) return (uint32_t)(sizeof(Accum) / sizeof(uint32_t));
+    return c->stamp[0] ? 1u : 4u;
+}
+// The accumulators by slot: one array for both tables where the stamps lie elsewhere.
+static Accum *accum_of(const gi_cache_s *c) { return c->accum[c->accum[1] ? c->cur : 0]; }
 
 static LiveRule live_rule(const gi_cache_s *c) {
     LiveRule r;
@@ -656,8 +802,11 @@ UpdateArgs cache_update_args(gi_cache_s *c, const gi_hits *h, const gi_view *v, 
     a.slot_ids = slot_ids;
     a.n = h->n;
     a.tags = c->tags[c->cur];
-    a.accum = c->accum[c->cur];
-    a.acc_stride = 1;
+    a.accum = accum_of(c);
+    a.dense = c->dense;
+    a.rank = c->rank;
+    a.stamps = stamps_of(c, c->cur);
+    a.stamp_stride = stamp_stride(c);
     a.touch = c->touch;
     a.bitmap = c->bitmap;
     a.ctr = c->ctr;
@@ -695,10 +844,16 @@ static gi_status maybe_rebuild(gi_cache_s *c, cudaStream_t st) {
         c->rebuilds++;
         return GI_OK;
     }
-    k_rebuild<<<c->sms * 8, 256, 0, st>>>(c->tags[c->cur], c->accum[c->cur], c->resolved[c->cur], c->tags[nxt],
-                                           c->accum[nxt], c->resolved[nxt], c->res_bytes, c->mask, c->cfg.max_probe,
-                                           live_rule(c), c->ctr);
+    if (c->rank) {
+        s = cuda_status(cudaMemsetAsync(c->cold[nxt], 0, c->N / 8, st), "rebuild memset");
+        if (s != GI_OK) return s;
+    }
+    k_rebuild<<<c->sms * 8, 256, 0, st>>>(c->tags[c->cur], stamps_of(c, c->cur), c->resolved[c->cur], c->tags[nxt],
+                                           stamps_of(c, nxt), c->resolved[nxt], stamp_stride(c), c->res_bytes, c->cold[c->cur],
+                                           c->cold[nxt], c->mask, c->cfg.max_probe, live_rule(c), c->ctr);
     s = cuda_status(cudaGetLastError(), "k_rebuild launch");
+    // the slots have moved: until the next resolve ranks them again, every cell accumulates by slot
+    if (s == GI_OK && c->rank) s = cuda_status(cudaMemsetAsync(c->rank, 0, c->N / 32 * sizeof(RankWord), st), "rebuild memset");
     if (s != GI_OK) return s;
     c->cur = nxt;
     c->rebuilds++;
@@ -710,8 +865,12 @@ ResolveArgs cache_resolve_args(gi_cache_s *c, uint32_t frame) {
     a.touch = c->touch;
     a.bitmap = c->bitmap;
     a.words = c->N / 32u;
-    a.accum = c->accum[c->cur];
-    a.acc_stride = 1;
+    a.accum = accum_of(c);
+    a.dense = c->dense;
+    a.rank = c->rank;
+    a.age = c->resolves % kDenseAge == kDenseAge - 1 ? 1u : 0u;
+    a.stamps = c->stamp[c->cur];
+    a.cold = c->cold[c->cur];
     a.resolved = c->resolved[c->cur];
     a.res_stride = c->res_bytes;
     a.ctr = c->ctr;
@@ -750,11 +909,14 @@ static void free_cache(gi_cache_s *c) {
         cudaFree(c->tags[k]);
         cudaFree(c->accum[k]);
         cudaFree(c->resolved[k]);
+        cudaFree(c->cold[k]);
         cudaFree(c->stamp[k]);
         cudaFree(c->state[k]);
         cudaFree(c->mips[k]);
         cudaFree(c->omask[k]);
     }
+    cudaFree(c->dense);
+    cudaFree(c->rank);
     cudaFree(c->tmask);
     cudaFree(c->cidx);
     cudaFree(c->tlist);
@@ -852,27 +1014,36 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
     gi_status s = cuda_status(cudaGetDevice(&c->device), "cudaGetDevice");
     if (s == GI_OK) s = cuda_status(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device), "sm count");
     const size_t N = c->N, E = c->cells;
+    // First touches: a slot bitmap walked in slot order by the resolve (the default), or a touch list.
+    const bool use_bitmap = !c->tiles && cfg->first_touch != GI_FIRST_TOUCH_LIST;
+    const bool use_dense = use_bitmap && cfg->log2_slots >= kDenseLog2Slots;
     for (int k = 0; k < 2 && s == GI_OK; ++k) {
         s = cuda_status(cudaMalloc(&c->tags[k], N * sizeof(SlotWord)), "cudaMalloc tags");
-        if (s == GI_OK) s = cuda_status(cudaMalloc(&c->accum[k], E * sizeof(Accum)), "cudaMalloc accum");
         if (s == GI_OK) s = cuda_status(cudaMalloc(&c->resolved[k], E * c->res_bytes), "cudaMalloc resolved");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->tags[k], 0, N * sizeof(SlotWord)), "memset");
-        if (s == GI_OK) s = cuda_status(cudaMemset(c->accum[k], 0, E * sizeof(Accum)), "memset");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->resolved[k], 0, E * c->res_bytes), "memset");
-        if (s == GI_OK && c->tiles) {
+        // the accumulators are clear whenever the tables change places: without stamps one array does
+        if (s == GI_OK && (k == 0 || !use_dense)) {
+            s = cuda_status(cudaMalloc(&c->accum[k], E * sizeof(Accum)), "cudaMalloc accum");
+            if (s == GI_OK) s = cuda_status(cudaMemset(c->accum[k], 0, E * sizeof(Accum)), "memset");
+        }
+        if (s == GI_OK && use_dense) {
+            s = cuda_status(cudaMalloc(&c->cold[k], N / 8), "cudaMalloc cold bits");
+            if (s == GI_OK) s = cuda_status(cudaMemset(c->cold[k], 0, N / 8), "memset");
+        }
+        if (s == GI_OK && (c->tiles || (use_dense && cfg->resolved_format == GI_RESOLVED_F16))) {
             s = cuda_status(cudaMalloc(&c->stamp[k], E * sizeof(uint32_t)), "cudaMalloc stamps");
-            if (s == GI_OK) s = cuda_status(cudaMalloc(&c->state[k], E * sizeof(float4)), "cudaMalloc state");
-            if (s == GI_OK) s = cuda_status(cudaMalloc(&c->mips[k], N * kTileMips * sizeof(float4)), "cudaMalloc mips");
             if (s == GI_OK) s = cuda_status(cudaMemset(c->stamp[k], 0, E * sizeof(uint32_t)), "memset");
+        }
+        if (s == GI_OK && c->tiles) {
+            s = cuda_status(cudaMalloc(&c->state[k], E * sizeof(float4)), "cudaMalloc state");
+            if (s == GI_OK) s = cuda_status(cudaMalloc(&c->mips[k], N * kTileMips * sizeof(float4)), "cudaMalloc mips");
             if (s == GI_OK) s = cuda_status(cudaMemset(c->state[k], 0, E * sizeof(float4)), "memset");
             if (s == GI_OK) s = cuda_status(cudaMemset(c->mips[k], 0, N * kTileMips * sizeof(float4)), "memset");
             if (s == GI_OK) s = cuda_status(cudaMalloc(&c->omask[k], N * sizeof(unsigned long long)), "cudaMalloc omask");
             if (s == GI_OK) s = cuda_status(cudaMemset(c->omask[k], 0, N * sizeof(unsigned long long)), "memset");
         }
     }
-    // First touches: a slot bitmap walked in slot order by the resolve when the accumulators
-    // exceed L2 (its ordered accesses then save DRAM traffic), else a touch list (cheaper updates).
-    const bool use_bitmap = !c->tiles && cfg->first_touch != GI_FIRST_TOUCH_LIST;
     if (s == GI_OK && c->tiles) {
         s = cuda_status(cudaMalloc(&c->tmask, N * sizeof(unsigned long long)), "cudaMalloc tile masks");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->tmask, 0, N * sizeof(unsigned long long)), "memset");
@@ -880,7 +1051,12 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
         if (s == GI_OK) s = cuda_status(cudaMemset(c->cidx, 0xFF, N * sizeof(uint32_t)), "memset");
         if (s == GI_OK) s = cuda_status(cudaMalloc(&c->tlist, N * sizeof(uint32_t)), "cudaMalloc tile list");
     }
-    if (s == GI_OK && use_bitmap) {
+    if (s == GI_OK && use_dense) {
+        s = cuda_status(cudaMalloc(&c->rank, N / 32 * sizeof(RankWord)), "cudaMalloc rank");
+        if (s == GI_OK) s = cuda_status(cudaMemset(c->rank, 0, N / 32 * sizeof(RankWord)), "memset");
+        if (s == GI_OK) s = cuda_status(cudaMalloc(&c->dense, N * sizeof(Accum)), "cudaMalloc dense accumulators");
+        if (s == GI_OK) s = cuda_status(cudaMemset(c->dense, 0, N * sizeof(Accum)), "memset");
+    } else if (s == GI_OK && use_bitmap) {
         s = cuda_status(cudaMalloc(&c->bitmap, N / 8), "cudaMalloc bitmap");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->bitmap, 0, N / 8), "memset");
     } else if (s == GI_OK && !c->tiles) {
@@ -904,7 +1080,7 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
         s = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<0, false>, kUpdThreads, 0),
                         "occupancy");
         c->upd_blocks = c->sms * std::max(per_sm, 1);
-        c->res_blocks = c->sms * (c->bitmap ? kResBmBlocksPerSm : kResListBlocksPerSm);
+        c->res_blocks = c->sms * (c->touch ? kResListBlocksPerSm : kResBmBlocksPerSm);
         c->tres_blocks = c->sms * tile_resolve_blocks_per_sm();
     }
     if (s == GI_OK) s = cuda_status(cudaDeviceSynchronize(), "create sync");
@@ -958,7 +1134,7 @@ gi_status gi_cache_update(gi_cache_t c, const gi_hits *hits, const gi_view *view
         return s;
     }
     // the bitmap form stages nothing per block: a resident grid strides over the records
-    const int blocks = c->bitmap ? (int)std::min<unsigned long long>((unsigned long long)c->upd_blocks,
+    const int blocks = !c->touch ? (int)std::min<unsigned long long>((unsigned long long)c->upd_blocks,
                                                                       (hits->n + kUpdThreads - 1) / kUpdThreads)
                                  : update_blocks(hits->n);
     launch_update(a, c->cfg.key_dir, c->cfg.merge == GI_MERGE_WARP, blocks, st);
@@ -1010,7 +1186,9 @@ gi_status gi_cache_resolve(gi_cache_t c, uint32_t frame, gi_stream_t stream) {
         s = tile_resolve_launch(ta, c->tres_blocks, st);
     } else {
         const ResolveArgs a = cache_resolve_args(c, frame);
-        if (a.bitmap)
+        if (a.rank)
+            k_resolve_dense<<<c->res_blocks, kResThreads, 0, st>>>(a);
+        else if (a.bitmap)
             k_resolve_bitmap<<<c->res_blocks, kResThreads, 0, st>>>(a);
         else
             k_resolve<<<c->res_blocks, kResThreads, 0, st>>>(a);
@@ -1074,7 +1252,9 @@ gi_status gi_cache_stats(gi_cache_t c, gi_cache_stats_t *out, gi_stream_t stream
     if (c->tiles) {
         s = tile_scan_launch(tile_arrays(c, c->cur), c->tmask, c->N, live_rule(c), c->scan, c->sms * 4, st);
     } else {
-        k_scan_stats<<<c->sms * 4, 256, 0, st>>>(c->tags[c->cur], c->accum[c->cur], c->bitmap, c->N, live_rule(c),
+        k_scan_stats<<<c->sms * 4, 256, 0, st>>>(c->tags[c->cur], accum_of(c), stamps_of(c, c->cur), stamp_stride(c),
+                                                 c->rank ? &c->rank->touched : c->bitmap,
+                                                 c->rank ? (uint32_t)(sizeof(RankWord) / 4) : 1u, c->N, live_rule(c),
                                                  c->scan);
         s = cuda_status(cudaGetLastError(), "k_scan_stats launch");
     }
@@ -1089,7 +1269,7 @@ gi_status gi_cache_stats(gi_cache_t c, gi_cache_stats_t *out, gi_stream_t stream
     out->slots = c->N;
     out->occupied = sc[0];
     out->live = sc[1];
-    out->touched = (c->bitmap || c->tiles) ? sc[2] : h.touch_count;
+    out->touched = c->touch ? h.touch_count : sc[2];
     out->dropped = h.dropped;
     out->clamped = h.clamped;
     out->rebuilds = c->rebuilds;
@@ -1146,9 +1326,27 @@ gi_status gi_cache_export(gi_cache_t c, gi_cell *out, uint64_t capacity, uint64_
     gi_status s = cuda_status(cudaStreamSynchronize(st), "export sync");
     if (s == GI_OK) s = cuda_status(cudaMemcpy(tags.data(), c->tags[c->cur], N * sizeof(SlotWord), cudaMemcpyDeviceToHost), "export");
     if (s == GI_OK)
-        s = cuda_status(cudaMemcpy(acc.data(), c->accum[c->cur], N * sizeof(Accum), cudaMemcpyDeviceToHost), "export");
+        s = cuda_status(cudaMemcpy(acc.data(), accum_of(c), N * sizeof(Accum), cudaMemcpyDeviceToHost), "export");
     if (s == GI_OK)
         s = cuda_status(cudaMemcpy(res.data(), c->resolved[c->cur], res.size(), cudaMemcpyDeviceToHost), "export");
+    if (s == GI_OK && c->rank) {
+        // large tables: a cell with a dense accumulator takes its sums from there, every cell its stamp
+        std::vector<RankWord> rank(N / 32);
+        std::vector<Accum> dense(N);
+        const uint32_t ss = stamp_stride(c);
+        std::vector<uint32_t> stamp(ss == 1u ? N : 0);
+        s = cuda_status(cudaMemcpy(rank.data(), c->rank, N / 32 * sizeof(RankWord), cudaMemcpyDeviceToHost), "export");
+        if (s == GI_OK) s = cuda_status(cudaMemcpy(dense.data(), c->dense, N * sizeof(Accum), cudaMemcpyDeviceToHost), "export");
+        if (s == GI_OK && ss == 1u)
+            s = cuda_status(cudaMemcpy(stamp.data(), c->stamp[c->cur], N * sizeof(uint32_t), cudaMemcpyDeviceToHost), "export");
+        for (size_t i = 0; i < N && s == GI_OK; ++i) {
+            const RankWord &r = rank[i / 32];
+            const uint32_t bit = 1u << (i % 32);
+            if (r.keep & bit) acc[i] = dense[r.base + (uint32_t)__builtin_popcount(r.keep & (bit - 1u))];
+            if (ss == 1u) acc[i].stamp = stamp[i];
+            else memcpy(&acc[i].stamp, res.data() + i * 16 + 12, 4);
+        }
+    }
     if (s != GI_OK) return s;
     const LiveRule r = live_rule(c);
     std::vector<gi_cell> cells;
@@ -1385,7 +1583,10 @@ extern "C" gi_status gi_cell_means_noalloc(const gi_hits *hits, const gi_view *v
     a.n = hits->n;
     a.tags = tags;
     a.accum = accum;
-    a.acc_stride = 1;
+    a.dense = nullptr;
+    a.rank = nullptr;
+    a.stamps = nullptr;
+    a.stamp_stride = 0u;
     a.touch = touch;
     a.bitmap = nullptr;
     a.ctr = ctr;

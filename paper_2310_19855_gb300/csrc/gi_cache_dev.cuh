@@ -13,28 +13,47 @@ namespace gi {
 // In the touch-list form a block of the update takes at most kUpdBlockRecords records (one
 // grid-strided chunk per iteration), so its shared-memory list of first touches can never
 // overflow and is flushed once, at the end, with one global atomic: warps never wait for one
-// another inside the loop.  The bitmap form stages nothing and runs a resident grid.
+// another inside the loop.  The bitmap form stages no touches and runs a resident grid.
 constexpr int kUpdThreads = 256;
 constexpr int kUpdBlockRecords = 2048;
 constexpr int kResThreads = 256;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// ---------------------------------------------------------------- bulk reductions
-// A cell's whole 32-byte accumulator {u64 r, g, b; u32 count; u32 stamp} in one L2 operation:
-// the thread writes {r, g, b, count} to a 32-byte shared-memory slot and the bulk-copy unit adds
-// it to global memory as four 64-bit lanes (cp.reduce.async.bulk .add.u64; the count lands in the
-// low half of the last lane, where it cannot carry into the stamp: a frame adds far fewer than
-// 2^32 to a count and every resolve clears it).  Both addresses 32-byte aligned.
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_add_accum(void *dst, const unsigned long long *src_smem) {
-    // the generic-proxy writes of the slot become visible to the bulk-copy (async) proxy
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(src_smem);
-    const unsigned long long ga = (unsigned long long)__cvta_generic_to_global(dst);
-    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.u64 [%0], [%1], 32;" ::"l"(ga), "r"(sa)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+// ---------------------------------------------------------------- quad accumulation
+// A warp's 32 accumulator contributions {u64 r, g, b; u64 count}, lane l's at s_warp[4 l .. 4 l + 3]
+// (shared memory, written by the lanes themselves), added to the cells' 32-byte sectors four lanes
+// per record: instruction j covers records 8 j .. 8 j + 7, lane l the word l & 3 of record 8 j + l / 4,
+// so that the four words of a sector leave in one coalesced L2 request.  loc: the lane's own
+// accumulator (kDense | index in `dense`, or its slot in `accum`), GI_SLOT_NONE for none.  LIST: the
+// count's addition returns, and a lane that finds it 0 (the last resolve cleared it) appends the slot
+// to s_touch.  The whole warp calls.
+constexpr uint32_t kDense = 0x80000000u;  // a table has at most 2^28 slots
+__device__ __forceinline__ Accum *accum_at(Accum *accum, Accum *dense, uint32_t loc) {
+    return (loc & kDense) ? dense + (loc & ~kDense) : accum + loc;
+}
+template <bool LIST = false>
+__device__ __forceinline__ void warp_add_accum(Accum *accum, Accum *dense, uint32_t loc,
+                                               const unsigned long long *s_warp, int lane, uint32_t *s_touch = nullptr,
+                                               uint32_t *s_n = nullptr) {
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t s = __shfl_sync(kFull, loc, 8 * j + (lane >> 2));
+        if (s != GI_SLOT_NONE) {
+            unsigned long long *w =
+                reinterpret_cast<unsigned long long *>(LIST ? accum + s : accum_at(accum, dense, s)) + (lane & 3);
+            const unsigned long long v = s_warp[32 * j + lane];
+            if (!LIST || (lane & 3) != 3) atomicAdd(w, v);
+            else if ((uint32_t)atomicAdd(w, v) == 0u) s_touch[atomicAdd(s_n, 1u)] = s;
+        }
+    }
+    __syncwarp();
+}
+
+// Accumulator of a slot: the dense one where its rank word keeps it, else the slot's own.
+__device__ __forceinline__ uint32_t accum_loc(uint32_t keep, uint32_t base, uint32_t slot) {
+    const uint32_t bit = 1u << (slot & 31u);
+    return (keep & bit) ? (kDense | (base + (uint32_t)__popc(keep & (bit - 1u)))) : slot;
 }
 
 // ---------------------------------------------------------------- L2 eviction priority
@@ -138,7 +157,8 @@ __device__ __forceinline__ float3 load_resolved(const void *r, uint32_t stride, 
 }
 
 // The 4th lane marks a cell resolved without history (its first resolve, or its first since an
-// eviction): 1 for such a cell, 0 otherwise.  The surrogate reads it to find cold cells.
+// eviction): 1 for such a cell, 0 otherwise.  The surrogate reads it to find cold cells.  (Large
+// tables keep that mark in a bitmap, and the stamp in the float4's 4th lane.)
 __device__ __forceinline__ void store_resolved(void *r, uint32_t stride, int f16, uint32_t s, float3 v, bool cold) {
     r = static_cast<char *>(r) + (size_t)s * stride;
     if (f16) {
@@ -171,6 +191,7 @@ __device__ __forceinline__ void resolve_finish(Counters *ctr, uint32_t *occ_out,
             // every warp has read the touch count: reset it for the next frame
             ctr->touch_count = 0u;
             ctr->ticket = 0u;
+            ctr->dense_next = 0u;
             // occupancy for the host's compaction decision, then the frame it belongs to
             if (occ_out) {
                 reinterpret_cast<volatile uint32_t *>(occ_out)[0] = atomicAdd(&ctr->occupied, 0u);

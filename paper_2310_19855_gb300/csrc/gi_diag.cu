@@ -2,11 +2,11 @@
 //
 // gi_cache_update ends, per hit record (the default GI_MERGE_NONE form), in L2 operations on the
 // cell's 32-byte accumulator.  List form: three 64-bit additions (the fixed-point sums) and one returning
-// 32-bit addition (the count, whose old value flags the first touch).  Bitmap form: one 32-byte
-// bulk reduction of the sums and count from shared memory and a non-returning set of the slot's
-// bit.  k_diag_atomics issues exactly those operations for a frame's slot ids, with nothing else
-// (no record stream, key, probe or slot-id store), so its time is the floor of that form on this
-// GPU.
+// addition of the count, whose old value flags the first touch.  Bitmap form: the sums and count added
+// by four lanes of the warp as one 32-byte request (warp_add_accum) and a non-returning set of the
+// slot's bit.  k_diag_atomics issues these operations for a frame's slot ids, with nothing else
+// (no record stream, key, probe or slot-id store) and by slot, so its time is the floor of the
+// accumulation of a table without dense accumulators on this GPU.
 #include "gi_cache_dev.cuh"
 
 namespace gi {
@@ -26,28 +26,24 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_diag_atomics(const uint32_t 
         const unsigned long long i = base + threadIdx.x;
         const uint32_t s = i < n ? __ldcs(slot_ids + i) : GI_SLOT_NONE;
         const bool hit = s < slots;
-        if (hit) {
-            Accum *a = acc + s;
-            if (BITMAP) {
-                bulk_wait_read();
+        if (BITMAP) {
+            if (hit) {
                 s_red[threadIdx.x][0] = 1ull;
                 s_red[threadIdx.x][1] = 2ull;
                 s_red[threadIdx.x][2] = 3ull;
                 s_red[threadIdx.x][3] = 1ull;
-                bulk_add_accum(a, s_red[threadIdx.x]);
                 atomicOr(bitmap + (s >> 5), 1u << (s & 31u));
-            } else {
-                atomicAdd(&a->sum[0], 1ull);
-                atomicAdd(&a->sum[1], 2ull);
-                atomicAdd(&a->sum[2], 3ull);
-                if (atomicAdd(&a->count, 1u) == 0u) ++first;
             }
+            warp_add_accum(acc, nullptr, hit ? s : GI_SLOT_NONE, &s_red[threadIdx.x & ~31u][0], lane);
+        } else if (hit) {
+            Accum *a = acc + s;
+            atomicAdd(&a->sum[0], 1ull);
+            atomicAdd(&a->sum[1], 2ull);
+            atomicAdd(&a->sum[2], 3ull);
+            if (atomicAdd(&a->count, 1u) == 0u) ++first;
         }
     }
-    if (BITMAP) {
-        bulk_wait_all();
-        return;
-    }
+    if (BITMAP) return;
     first = __reduce_add_sync(kFull, first);
     if (lane == 0 && first) atomicAdd(&s_first, first);
     __syncthreads();

@@ -16,10 +16,10 @@ constexpr uint32_t kQMask = (1u << kQBits) - 1u;
 
 // 32-byte per-slot accumulator: one sector.  stamp = 1 + frame of the last
 // resolve that found samples in the cell (0 = never resolved).
-struct __align__(16) Accum {
+struct __align__(32) Accum {
     unsigned long long sum[3];
     uint32_t count;
-    uint32_t stamp;
+    uint32_t stamp;  // unused in large tables (see gi_cache.cu)
 };
 static_assert(sizeof(Accum) == 32, "accumulator must fill one 32-byte sector");
 
@@ -32,7 +32,8 @@ struct __align__(128) Counters {
     unsigned long long dropped;
     unsigned long long clamped;
     uint32_t error_word;
-    uint32_t pad[23];
+    uint32_t dense_next;    // dense accumulators handed out by the resolve under way
+    uint32_t pad[22];
 };
 
 // Per-view constants of the cell descriptor (Algorithm 6 + LOD reading).
@@ -88,6 +89,14 @@ CamParams cam_params(const gi_view *v);
 typedef uint32_t SlotWord;  // tag = fingerprint << 8 | (home mod 256); 0 = empty
 __device__ __forceinline__ uint32_t word_tag(SlotWord w) { return w; }
 
+// Large tables: 32 consecutive slots.
+struct __align__(16) RankWord {
+    uint32_t keep;     // slots with a dense accumulator, one bit each
+    uint32_t base;     // index of the first one's
+    uint32_t touched;  // slots touched since the last resolve (the cache's bitmap)
+    uint32_t recent;   // slots touched since the last aging of `keep`
+};
+
 struct UpdateArgs {
     const float *p[3];
     const float *nrm[3];
@@ -97,10 +106,13 @@ struct UpdateArgs {
     uint32_t *slot_ids;
     unsigned long long n;
     SlotWord *tags;
-    Accum *accum;
-    uint32_t acc_stride;  // Accum units between consecutive slots
+    Accum *accum;         // by slot
+    Accum *dense;         // large tables: accumulators of the cells that `rank` keeps
+    RankWord *rank;       // large tables, else NULL (every cell accumulates by slot)
+    const uint32_t *stamps;  // 1 + frame of the last resolve with samples; slot s at s * stamp_stride
+    uint32_t stamp_stride;
     uint32_t *touch;
-    uint32_t *bitmap;     // touched slots, one bit each (NULL: first touches go to the touch list)
+    uint32_t *bitmap;     // touched slots, one bit each (NULL: in `rank`, or first touches go to the touch list)
     Counters *ctr;
     uint32_t mask;
     uint32_t max_probe;
@@ -118,7 +130,11 @@ struct ResolveArgs {
     uint32_t *bitmap;     // touched slots (walked and cleared by the resolve)
     uint32_t words;       // bitmap words = slots / 32
     Accum *accum;
-    uint32_t acc_stride;
+    Accum *dense;         // large tables (else NULL): see UpdateArgs
+    RankWord *rank;
+    uint32_t age;         // this resolve keeps dense accumulators only for the recently touched slots
+    uint32_t *stamps;     // large float16 tables: stamps by slot
+    uint32_t *cold;       // large tables: cells whose last resolve found no history, one bit each
     void *resolved;
     uint32_t res_stride;  // bytes between consecutive resolved values
     Counters *ctr;
@@ -271,6 +287,7 @@ struct CacheView {
     uint32_t resolved_stride;  // bytes between the resolved values of consecutive slots
     int resolved_f16;
     uint32_t slots;
+    const uint32_t *cold;      // large tables: cold cells, one bit each (else in the resolved values)
 };
 CacheView cache_view(gi_cache_t c);
 
@@ -308,7 +325,7 @@ uint32_t update_blocks_for(unsigned long long n, uint32_t records_per_block);
 gi_status launch_update_batched(const UpdateArgs *args, const uint32_t *prefix, uint32_t nviews, uint32_t blocks,
                                 int key_dir, cudaStream_t st);
 gi_status launch_resolve_batched(const ResolveArgs *args, const uint32_t *prefix, uint32_t nviews, uint32_t blocks,
-                                 cudaStream_t st);
+                                 bool dense, cudaStream_t st);
 gi_status launch_spawn_batched(const SpawnArgs *args, const uint32_t *prefix, uint32_t nviews, uint32_t blocks,
                                cudaStream_t st);
 gi_status launch_integrate_batched(const IntegrateArgs *args, const uint32_t *prefix, uint32_t nviews,
@@ -348,7 +365,7 @@ __device__ __forceinline__ uint32_t view_of_block(const uint32_t *prefix, uint32
 // zero when the pass starts), so that blocks that drew cheap items take more; a view's arguments
 // are reloaded into shared memory only when an item belongs to another view than the last.  The
 // body sees `item` (the view-local block) and `items` (the view's block count).
-#define GI_BATCHED_ITEMS(prefix, nviews, sa, args, body)                                   \
+#define GI_BATCHED_ITEMS(prefix, nviews, sa, args, ...)                                    \
     do {                                                                                 \
         __shared__ uint32_t s_w_;                                                        \
         const uint32_t total_ = __ldg((prefix) + (nviews));                              \
@@ -368,7 +385,7 @@ __device__ __forceinline__ uint32_t view_of_block(const uint32_t *prefix, uint32
             const uint32_t p0_ = __ldg((prefix) + v_), p1_ = __ldg((prefix) + v_ + 1);   \
             const uint32_t item = w_ - p0_, items = p1_ - p0_;                           \
             (void)items;                                                                 \
-            body;                                                                        \
+            __VA_ARGS__;                                                                 \
             __syncthreads();                                                             \
         }                                                                                \
     } while (0)

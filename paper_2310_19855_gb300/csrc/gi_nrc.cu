@@ -231,6 +231,12 @@ __device__ __forceinline__ float4 cache_value(const CacheView &cv, uint32_t s) {
     return __ldg(reinterpret_cast<const float4 *>(r));
 }
 
+// a cell resolved without history (see store_resolved)
+__device__ __forceinline__ bool cache_cold(const CacheView &cv, uint32_t s) {
+    if (cv.cold) return (__ldg(cv.cold + (s >> 5)) >> (s & 31u)) & 1u;
+    return cache_value(cv, s).w != 0.0f;
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
     uint32_t n = a.n;
@@ -798,7 +804,7 @@ __global__ void __launch_bounds__(256) k_nrc_select(SelectArgs a) {
             } else if (slot == GI_SLOT_NONE) {
                 use = true;
             } else if (slot < a.cv.slots) {
-                const bool cold = cache_value(a.cv, slot).w != 0.0f;
+                const bool cold = cache_cold(a.cv, slot);
                 use = cold || key_lod(a.kp, __ldg(a.pos[0] + r), __ldg(a.pos[1] + r), __ldg(a.pos[2] + r)) >=
                                   (int)a.query_lod;
             }

@@ -64,14 +64,15 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) { return a >
 
 // ---------------------------------------------------------------- update
 // Three launches.  (1) k_tile_key: per record the tile descriptor, bucket + fingerprint of the
-// tile and the cell; the leader of each group of same-cell hits in a warp finds or inserts the
-// tile by linear probing and sets the cell's bit in the tile's touched mask (a reduction); the
-// record's slot id is tile slot * 64 + cell.  (2) k_tile_compact: every tile touched since the
-// last resolve that has no accumulator block yet gets the next one (a per-frame index, cidx).
-// (3) k_tile_accumulate: per record the fixed-point radiance, merged per cell within the warp
-// and added into the cell's accumulator of its tile's block with one 32-byte bulk reduction.  The accumulator
+// tile and the cell; it finds or inserts the tile by linear probing and sets the cell's bit in the
+// tile's touched mask (a reduction); the record's slot id is tile slot * 64 + cell.
+// (2) k_tile_compact: every tile touched since the last resolve that has no accumulator block yet
+// gets the next one (a per-frame index, cidx).  (3) k_tile_accumulate: per record the fixed-point
+// radiance, added into the cell's accumulator of its tile's block (warp_add_accum).  The accumulator
 // blocks of one frame are contiguous (touched tiles x 2 KB), so the reductions of a frame span
 // that range only, not the whole table: the cost of scattered reductions grows with the span.
+// Neither pass merges a warp's same-cell hits first: a probe's rays share few cells, and at 1080p
+// with 2x2 upscale the merge (__match_any_sync, pointer-jumping sums) cost 5 us of the frame.
 template <int KEY_DIR>
 __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) {
     const UpdateArgs &a = ta.u;
@@ -110,13 +111,8 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) 
                 tile_key(a.kp, px, py, pz, sx, sy, sz, len, KEY_DIR == GI_KEY_DIR_NORMAL ? 0u : 1u, cell);
             cell_of_key(key, a.mask, home, tag);
         }
-        // same cell = same (home, tag, cell); home < 2^22, so the cell fits above it
-        const unsigned hm = __ballot_sync(kFull, hit);
-        unsigned peers = 0;
-        if (hit) peers = __match_any_sync(hm, ((unsigned long long)(home | (cell << 26)) << 32) | tag);
-        const bool leader = hit && (peers & ((1u << lane) - 1u)) == 0u;
         uint32_t slot = GI_SLOT_NONE;
-        if (leader) {
+        if (hit) {
             uint32_t s = home, k = 0;
             for (; k < a.max_probe; ++k) {
                 const uint32_t t = __ldcg(a.tags + s);
@@ -136,13 +132,11 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) 
             }
             my_maxp = max(my_maxp, k + 1u);
             if (slot != GI_SLOT_NONE) atomicOr(ta.tmask + slot, 1ull << cell);
-            else my_dropped += (unsigned long long)__popc(peers);
+            else ++my_dropped;
         }
-        const int lead = hit ? (__ffs(peers) - 1) : lane;
-        const uint32_t my_slot = __shfl_sync(kFull, slot, lead);
         uint32_t id = miss ? GI_SLOT_MISS : GI_SLOT_NONE;
-        if (hit && my_slot != GI_SLOT_NONE) id = my_slot * kTileCells + cell;
-        if (hit && my_slot == GI_SLOT_NONE) {
+        if (slot != GI_SLOT_NONE) id = slot * kTileCells + cell;
+        if (hit && slot == GI_SLOT_NONE) {
             uint32_t bad = 0;
             quantize(__ldcs(a.rad[0] + i), bad);
             quantize(__ldcs(a.rad[1] + i), bad);
@@ -229,40 +223,18 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_accumulate(const uint32
         // a tile with a slot id always has a block (the compaction ran after the keys); a missing
         // one would be a broken invariant: the record is skipped rather than written out of range
         ok = ok && blk < cells / kTileCells;
-        const unsigned vm = __ballot_sync(kFull, ok);
-        unsigned peers = 0;
-        if (ok) peers = __match_any_sync(vm, id);
-        const unsigned above = peers & (0xFFFFFFFEu << lane);
-        int nxt = above ? (__ffs(above) - 1) : -1;
-        uint32_t cnt = ok ? 1u : 0u;
-        while (__any_sync(kFull, nxt >= 0)) {
-            const int src = nxt >= 0 ? nxt : lane;
-            const unsigned long long o0 = __shfl_sync(kFull, q0, src);
-            const unsigned long long o1 = __shfl_sync(kFull, q1, src);
-            const unsigned long long o2 = __shfl_sync(kFull, q2, src);
-            const uint32_t oc = __shfl_sync(kFull, cnt, src);
-            const int on = __shfl_sync(kFull, nxt, src);
-            if (nxt >= 0) {
-                q0 += o0;
-                q1 += o1;
-                q2 += o2;
-                cnt += oc;
-                nxt = on;
-            }
-        }
-        if (ok && (peers & ((1u << lane) - 1u)) == 0u) {
-            // the group's sums and count in one 32-byte bulk reduction (the stamp half of the
-            // last lane is unused in the blocks)
-            Accum *ac = accum + (size_t)blk * kTileCells + (id % kTileCells);
-            bulk_wait_read();  // the previous reduction has read the slot
+        // {r, g, b, count} of the hit, four lanes per record (the stamp half of the last word is unused
+        // in the blocks)
+        uint32_t loc = GI_SLOT_NONE;
+        if (ok) {
+            loc = blk * kTileCells + (id % kTileCells);
             s_red[threadIdx.x][0] = q0;
             s_red[threadIdx.x][1] = q1;
             s_red[threadIdx.x][2] = q2;
-            s_red[threadIdx.x][3] = cnt;
-            bulk_add_accum(ac, s_red[threadIdx.x]);
+            s_red[threadIdx.x][3] = 1ull;
         }
+        warp_add_accum(accum, nullptr, loc, &s_red[threadIdx.x & ~31u][0], lane);
     }
-    bulk_wait_all();
     // hits with a tile whose radiance was clamped (k_tile_key counts those of dropped hits)
     my_clamped = __reduce_add_sync(kFull, my_clamped);
     if (lane == 0 && my_clamped) atomicAdd(&s_clamped, my_clamped);

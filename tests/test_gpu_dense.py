@@ -1,0 +1,77 @@
+"""Tables of 2^22 slots and more accumulate recently touched cells in side-by-side accumulators; the
+touch-list form accumulates every cell in its own slot.  Both must give the same cells, sums, counts,
+stamps and values: over fresh cells, cells kept, dropped by aging and touched again, several updates
+per resolve, eviction and a compaction of the table, and in the state between update and resolve."""
+import numpy as np
+import pytest
+
+import paper_2310_19855_gb300 as gi
+import workload as wl
+from _gpu_util import close, dev, require_gpu, u32  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+import torch  # noqa: E402
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def _view(frame):
+    return gi.make_view(frame, 640, 360, (0, 0, 0), (0, 0, -1), (1, 0, 0), (0, 1, 0), 1.0)
+
+
+def _same(a, b):
+    ea, eb = gi.gi_cache_export(a), gi.gi_cache_export(b)
+    assert ea.size == eb.size
+    for name in ("identity", "sum", "count", "stamp", "value"):
+        assert np.array_equal(ea[name], eb[name]), name
+    sa, sb = gi.gi_cache_stats(a), gi.gi_cache_stats(b)
+    for name in ("occupied", "live", "touched", "dropped", "clamped", "rebuilds"):
+        assert sa[name] == sb[name], name
+    return ea.size
+
+
+@pytest.mark.parametrize("f16,merge,key_dir", [(0, 0, 0), (1, 0, 1), (0, 1, 0)])
+def test_dense_accumulators_equal_the_list_form(f16, merge, key_dir):
+    kw = dict(resolved_format=f16, merge=merge, key_dir=key_dir, evict_frames=3, rebuild_load=0.25, cell_size=0.05)
+    caches = [gi.gi_cache_create(22, first_touch=ft, **kw) for ft in (gi.GI_FIRST_TOUCH_AUTO, gi.GI_FIRST_TOUCH_LIST)]
+    try:
+        stay = wl.records_random(30011, 1, extent=3.0)  # touched in every frame: kept
+        rare = wl.records_random(5003, 2, extent=1.0)   # touched in frames 0 and 20: dropped, then again
+        frame = 0
+        for k in range(22):
+            # the last frames fill the table beyond the compaction's load
+            n = 777 if k < 18 else 600_001
+            batches = [stay, wl.records_random(n, 100 + k, extent=4.0 if k < 18 else 40.0)]
+            if k in (0, 20):
+                batches.append(rare)
+            for h in caches:
+                for b in batches:
+                    r = dev(b)
+                    s = torch.empty(b.shape[1], dtype=torch.int32, device="cuda")
+                    gi.gi_cache_update(h, gi.hits_from_planes(r, b.shape[1]), _view(frame), s)
+                if k in (0, 1, 9, 20):
+                    torch.cuda.synchronize()
+            if k in (0, 1, 9, 20):
+                _same(*caches)  # between the updates and the resolve
+            for h in caches:
+                gi.gi_cache_resolve(h, frame)
+            torch.cuda.synchronize()
+            if k in (0, 8, 17, 20, 21):
+                _same(*caches)
+            frame += 1
+        assert gi.gi_cache_stats(caches[0])["rebuilds"] >= 1
+        pts = wl.records_random(20000, 7, extent=3.5)
+        out = []
+        for h in caches:
+            o = torch.empty((20000, 4), device="cuda")
+            r = dev(pts)
+            gi.gi_cache_query(h, o, 20000, points=gi.hits_from_planes(r, 20000), view=_view(frame))
+            out.append(o)
+        assert torch.equal(out[0], out[1])
+    finally:
+        for h in caches:
+            gi.gi_cache_destroy(h)
