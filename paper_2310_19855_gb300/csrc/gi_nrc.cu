@@ -13,8 +13,9 @@
 //                  the CTA's tiles, input gradients out to global memory
 //   k_nrc_scatter  one thread per (sample, level): trilinear weights x input gradient added to the
 //                  8 vertices' gradient accumulators (float2 atomics)
-//   k_nrc_adam_*   Adam on the table entries and the weights; refreshes the float16 table copy and
-//                  the bf16 weight images the MLP kernel loads
+//   k_nrc_adam     Adam on the table entries and the weights (with the network kernel's partial weight
+//                  gradients summed); refreshes the float16 table copy and the bf16 weight images
+//                  the MLP kernel loads
 //
 // Shared-memory operand layout: see gi_tc.cuh (K-major core matrices, no swizzle).  Every tile of
 // the MLP kernel is stored sample-major; the weight-gradient products, which contract over the
@@ -40,7 +41,7 @@ constexpr int kIn = 2 * kL;          // 32 encoded features
 constexpr int kHid = GI_NRC_HIDDEN;  // 64 hidden units
 constexpr int kOut = GI_NRC_OUTPUTS; // 3 outputs
 constexpr int kTile = 128;           // samples per tile = M of every forward / backward product
-constexpr int kEncThreads = 256;
+constexpr int kEncThreads = 256, kEncBlocksPerSm = 5;
 constexpr uint32_t kPrimeY = 2654435761u, kPrimeZ = 805459861u, kPrimeD = 2246822519u;
 
 // bf16 weight images (core-matrix tiles), loaded into shared memory by every MLP CTA
@@ -61,7 +62,7 @@ constexpr int kPartStride = kWCount + 4;
 constexpr uint32_t kXTile = kTile * kIn * 2;  // 8192
 constexpr uint32_t kTTile = 4 * kTile * 4;    // target planes r, g, b and the mask: 2048
 
-// MLP kernel shared memory (bytes)
+// training kernel shared memory (bytes)
 constexpr uint32_t kSmImg = 0;
 constexpr uint32_t kSmXH0 = 28672;   // [128][96]: H1 (features 0..63) | X (64..95), SBO 1536
 constexpr uint32_t kSmXH1 = 53248;
@@ -71,7 +72,6 @@ constexpr uint32_t kSmH2 = 81920;    // [128][64], SBO 1024
 constexpr uint32_t kSmDY = 98304;    // [128][16], SBO 256
 constexpr uint32_t kSmZ = 102400;    // [128][128]: dZ2 (0..63) | dZ1 (64..127), SBO 2048
 constexpr uint32_t kSmTrain = 135168;
-constexpr uint32_t kSmInfer = 98304; // image, XH0, XH1, (targets unused), H2
 constexpr uint32_t kXHStride = 1536, kH2Stride = 1024, kDYStride = 256, kZStride = 2048;
 
 // tensor memory columns (256 allocated)
@@ -81,6 +81,11 @@ constexpr uint32_t kTmD3 = 128;  // output (16 columns, 3 used)
 constexpr uint32_t kTmGC = 144;  // dW3^T accumulator (16 columns)
 constexpr uint32_t kTmGA = 160;  // [dW2 | dW1] accumulator (96 columns)
 constexpr uint32_t kTmCols = 256;
+
+// inference kernel: shared memory (W1, W2 and W3 of the image, two input tiles, one tile of hidden
+// units) and tensor memory small enough for four CTAs per SM
+constexpr uint32_t kInfW1 = 0, kInfW2 = 4096, kInfW3 = 12288, kInfX = 14336, kInfH = 30720, kInfBytes = 47104;
+constexpr uint32_t kInfCols = 128, kInfD = 0, kInfD3 = 64;
 
 constexpr uint32_t kErrTimeout = 1u;
 
@@ -132,15 +137,22 @@ struct MlpArgs {
     const uint16_t *X;
     const float *T;
     const uint8_t *wimg;
-    uint32_t n;                // samples, unless count is given
-    const uint32_t *count;     // device sample count (queries), clamped to n
+    uint32_t n;                // samples
     float dy_scale;            // 2 / B
     float loss_eps;
-    float *dX;                 // train: [n_pad][32] float32
-    float *wpart;              // train: per-CTA partial W1 | W2 | W3 gradients and loss sums,
-                               // rows of kPartStride floats (reduced by k_nrc_wgrad_reduce)
-    float4 *out;               // infer: (max(y, 0), 1)
-    const uint32_t *out_idx;   // infer: out[out_idx[s]] when given, else out[s]
+    float *dX;                 // [n_pad][32] float32
+    float *wpart;              // per-CTA partial W1 | W2 | W3 gradients and loss sums, rows of
+                               // kPartStride floats (summed by k_nrc_adam or k_nrc_wgrad_reduce)
+    uint32_t *err;
+};
+
+struct InferArgs {
+    const uint16_t *X;
+    const uint8_t *wimg;
+    uint32_t n;                // samples, unless count is given
+    const uint32_t *count;     // device sample count (queries), clamped to n
+    float4 *out;               // (max(y, 0), 1)
+    const uint32_t *out_idx;   // out[out_idx[s]] when given, else out[s]
     uint32_t *err;
 };
 
@@ -237,10 +249,31 @@ __device__ __forceinline__ bool cache_cold(const CacheView &cv, uint32_t s) {
     return cache_value(cv, s).w != 0.0f;
 }
 
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+
+// The features of the 8 vertices, gathered together, then weighted in corner order.
+__device__ __forceinline__ void interpolate_level(const __half2 *tab, const uint32_t (&idx)[8], const float (&w)[8],
+                                                  float &e0, float &e1) {
+    __half2 f[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) f[c] = __ldg(tab + idx[c]);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float2 v = __half22float2(f[c]);
+        e0 = fmaf(w[c], v.x, e0);
+        e1 = fmaf(w[c], v.y, e1);
+    }
+}
+
+// Points and training samples (drawn at random over the view): one thread per sample and level, a warp
+// takes two samples.  MODE: kEncPoints or kEncSampled.
 template <int MODE>
 __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
-    uint32_t n = a.n;
-    if (MODE == kEncQueries) n = min(__ldg(a.qcount), a.n);
+    const uint32_t n = a.n;
     const uint32_t n_pad = (n + kTile - 1) / kTile * kTile;
     const uint32_t T = 1u << a.geo.log2_table;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_pad * kL; i += gridDim.x * blockDim.x) {
@@ -248,7 +281,6 @@ __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
         const bool valid = s < n;
         uint32_t r = s;
         if (MODE == kEncSampled) r = pcg_hash((a.offset + s) ^ a.seed) % a.n_records;
-        if (MODE == kEncQueries && valid) r = __ldg(a.qidx + s);
         float e0 = 0.0f, e1 = 0.0f;
         if (valid) {
             float x[3];
@@ -257,21 +289,12 @@ __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
             uint32_t idx[8];
             float w[8];
             level_corners(x, a.geo.lv.res[l], a.geo.lv.dense[l] != 0u, d, T - 1u, idx, w);
-            const __half2 *tab = a.tab16 + (size_t)l * T;
-            __half2 f[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) f[c] = __ldg(tab + idx[c]);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float2 v = __half22float2(f[c]);
-                e0 = fmaf(w[c], v.x, e0);
-                e1 = fmaf(w[c], v.y, e1);
-            }
+            interpolate_level(a.tab16 + (size_t)l * T, idx, w, e0, e1);
         }
         const uint32_t tile = s / kTile, row = s % kTile;
         uint8_t *xt = reinterpret_cast<uint8_t *>(a.X) + (size_t)tile * kXTile;
         *reinterpret_cast<__nv_bfloat162 *>(xt + tc::cm_offset(row, 2u * l, kIn)) = __floats2bfloat162_rn(e0, e1);
-        if (MODE != kEncQueries && a.T && l == 0) {
+        if (a.T && l == 0) {
             float t[3] = {0.f, 0.f, 0.f}, m = 0.0f;
             if (valid && MODE == kEncPoints) {
                 for (int c = 0; c < 3; ++c) t[c] = __ldg(a.target[c] + s);
@@ -295,12 +318,75 @@ __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
     }
 }
 
-// ---------------------------------------------------------------- the network on the tensor cores
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&h);
+// The records a view leaves to the network (kEncQueries).  A warp takes 32 consecutive ones through a
+// group of consecutive levels, one level at a time: its lanes' vertices then lie in one level's table,
+// close together where the records are (they come probe by probe), and each record's position and normal
+// are read once per group.  A block takes a contiguous run of such items, so that the records of an
+// SM are neighbours too.  The gathers are bound by the sectors the L2 delivers (45 % of them hit the
+// L1 with a thread per record and level), so what counts is how many the L1 answers.  Groups of 16, 8, 4
+// or 2 levels, the longest that leave every resident warp an item; fewer records take k_nrc_encode's
+// form.  On the far hits of a 1080p frame the frame took 366, 363 and 396 us on three scenes, against
+// 381, 368 and 417 us with k_nrc_encode's form (random samples and points: 3 us slower, so they keep
+// theirs).  48 registers, 5 blocks per SM: at 6 blocks the eight gathers of a level no longer fly
+// together, 32 us slower.
+__global__ void __launch_bounds__(kEncThreads, kEncBlocksPerSm) k_nrc_encode_queries(EncArgs a) {
+    const uint32_t n = min(__ldg(a.qcount), a.n);
+    const uint32_t T = 1u << a.geo.log2_table;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    // log2 of the levels per group
+    const uint32_t want = gridDim.x * (kEncThreads / 32), ng = n / 32u;
+    const uint32_t glog = ng >= want ? 4u : (2u * ng >= want ? 3u : (4u * ng >= want ? 2u : (8u * ng >= want ? 1u : 0u)));
+    const uint32_t lgs = kL >> glog;  // level groups
+    const uint32_t n_pad = (n + kTile - 1) / kTile * kTile;
+    const uint32_t items = glog ? n_pad / 32u * lgs : n_pad / 2u;
+    // contiguous runs of 8 items (one per warp) per block, as even as they divide
+    const uint32_t rounds = (items + kEncThreads / 32 - 1) / (kEncThreads / 32);
+    const uint32_t r0 = (uint32_t)((uint64_t)rounds * blockIdx.x / gridDim.x),
+                   r1 = (uint32_t)((uint64_t)rounds * (blockIdx.x + 1) / gridDim.x);
+    for (uint32_t it = r0 * (kEncThreads / 32) + warp; it < min(items, r1 * (kEncThreads / 32)); it += kEncThreads / 32) {
+        const uint32_t s = glog ? (it / lgs) * 32u + lane : it * 2u + (lane >> 4);
+        const uint32_t l0 = glog ? (it % lgs) << glog : (lane & 15u);
+        const bool valid = s < n;
+        float x[3] = {0.f, 0.f, 0.f};
+        uint32_t d = 0;
+        if (valid) {
+            const uint32_t r = __ldg(a.qidx + s);
+            normalise(a.geo, __ldg(a.pos[0] + r), __ldg(a.pos[1] + r), __ldg(a.pos[2] + r), x);
+            d = dir_code(__ldg(a.nrm[0] + r), __ldg(a.nrm[1] + r), __ldg(a.nrm[2] + r));
+        }
+        const uint32_t tile = s / kTile, row = s % kTile;
+        uint8_t *xt = reinterpret_cast<uint8_t *>(a.X) + (size_t)tile * kXTile;
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+        for (uint32_t l = l0; l < l0 + (1u << glog); ++l) {
+            float e0 = 0.0f, e1 = 0.0f;
+            if (valid) {
+                uint32_t idx[8];
+                float w[8];
+                level_corners(x, a.geo.lv.res[l], a.geo.lv.dense[l] != 0u, d, T - 1u, idx, w);
+                interpolate_level(a.tab16 + (size_t)l * T, idx, w, e0, e1);
+            }
+            const uint32_t pk = pack_bf16x2(e0, e1);
+            if (glog == 0u) {
+                *reinterpret_cast<uint32_t *>(xt + tc::cm_offset(row, 2u * l, kIn)) = pk;
+            } else if (glog == 1u) {
+                if (l & 1u) *reinterpret_cast<uint2 *>(xt + tc::cm_offset(row, 2u * (l - 1u), kIn)) = make_uint2(q.x, pk);
+                else q.x = pk;
+            } else {  // four levels fill 16 bytes of the sample's row
+                const uint32_t j = l & 3u;
+                if (j == 0u) q.x = pk;
+                else if (j == 1u) q.y = pk;
+                else if (j == 2u) q.z = pk;
+                else {
+                    q.w = pk;
+                    *reinterpret_cast<uint4 *>(xt + tc::cm_offset(row, 2u * (l & ~3u), kIn)) = q;
+                }
+            }
+        }
+    }
 }
+
+// ---------------------------------------------------------------- the network on the tensor cores
 
 // Store 8 consecutive features (k0 .. k0 + 7) of sample row t as one 16-byte core-matrix row.
 __device__ __forceinline__ void store_row8(uint8_t *tile, uint32_t row_stride, uint32_t t, uint32_t k0, const float *v) {
@@ -333,16 +419,13 @@ __device__ __forceinline__ uint32_t idesc_mn(uint32_t M, uint32_t N) {
 // Persistent kernel: CTA b takes tiles b, b + gridDim.x, ...; thread t owns sample row t of a tile
 // (tensor-memory lane t: warp w reads lanes 32 w .. 32 w + 31).  Thread 0 issues every MMA and
 // bulk copy; completion comes back through mbarriers, every wait bounded in time.
-template <bool TRAIN>
-__global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
+__global__ void __launch_bounds__(kTile, 1) k_nrc_mlp(MlpArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar_w, bar_ld[2], bar_mma;
     __shared__ uint32_t tmem_s;
     __shared__ int abort_s;
     const uint32_t t = threadIdx.x, warp = t >> 5;
-    uint32_t n = a.n;
-    if (a.count) n = min(__ldg(a.count), a.n);
-    const uint32_t tiles = (n + kTile - 1) / kTile;
+    const uint32_t tiles = (a.n + kTile - 1) / kTile;
     if (blockIdx.x >= tiles) return;
 
     if (t == 0) {
@@ -353,11 +436,9 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
         tc::mbar_init(&bar_mma, 1);
         tc::mbar_init_fence();
     }
-    if (TRAIN) {
-        // dY columns 3..15 stay zero; written once here, never again
-        for (uint32_t i = t; i < kTile * 16 / 8; i += kTile)
-            reinterpret_cast<uint4 *>(smem + kSmDY)[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
+    // dY columns 3..15 stay zero; written once here, never again
+    for (uint32_t i = t; i < kTile * 16 / 8; i += kTile)
+        reinterpret_cast<uint4 *>(smem + kSmDY)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (warp == 0) {
         tc::tmem_alloc(&tmem_s, kTmCols);
         tc::tmem_relinquish();
@@ -378,14 +459,12 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
 
     auto load_tile = [&](uint32_t tile, int buf) {  // thread 0 only
         ++ld_issued[buf];
-        const uint32_t bytes = kXTile + (TRAIN ? kTTile : 0u);
-        tc::mbar_expect_tx(&bar_ld[buf], bytes);
+        tc::mbar_expect_tx(&bar_ld[buf], kXTile + kTTile);
         const uint8_t *src = reinterpret_cast<const uint8_t *>(a.X) + (size_t)tile * kXTile;
         for (uint32_t g = 0; g < kTile / 8; ++g)
             tc::bulk_g2s(smem + xh_off(buf) + g * kXHStride + 1024u, src + g * 512u, 512u, &bar_ld[buf]);
-        if (TRAIN)
-            tc::bulk_g2s(smem + t_off(buf), reinterpret_cast<const uint8_t *>(a.T) + (size_t)tile * kTTile, kTTile,
-                         &bar_ld[buf]);
+        tc::bulk_g2s(smem + t_off(buf), reinterpret_cast<const uint8_t *>(a.T) + (size_t)tile * kTTile, kTTile,
+                     &bar_ld[buf]);
     };
     if (t == 0) {
         tc::mbar_expect_tx(&bar_w, kImgBytes);
@@ -483,16 +562,6 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
         tc::wait_ld();
         const uint32_t s = tile * kTile + t;
 
-        if (!TRAIN) {
-            if (s < n) {
-                const uint32_t o = a.out_idx ? __ldg(a.out_idx + s) : s;
-                a.out[o] = make_float4(fmaxf(y[0], 0.0f), fmaxf(y[1], 0.0f), fmaxf(y[2], 0.0f), 1.0f);
-            }
-            tc::fence_before_sync();
-            __syncthreads();  // the next tile's products overwrite the accumulators just read
-            continue;
-        }
-
         // ---- loss gradient: dy = m (2 / B) (y - t) / (y^2 + eps); relative L2 and the judge's sums
         const float *tt = reinterpret_cast<const float *>(smem + t_off(buf));
         const float msk = tt[3 * kTile + t];
@@ -585,7 +654,7 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
         if (abort_s) break;
     }
 
-    float *part = TRAIN ? a.wpart + (size_t)blockIdx.x * kPartStride : nullptr;
+    float *part = a.wpart + (size_t)blockIdx.x * kPartStride;
     if (abort_s) {
         if (t == 0) {
             atomicOr(a.err, kErrTimeout);
@@ -597,9 +666,8 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
                 if (ld_issued[b] > ld_done[b]) tc::mbar_wait(&bar_ld[b], (ld_issued[b] - 1u) & 1u);
             if (mma_issued > mma_done) tc::mbar_wait(&bar_mma, (mma_issued - 1u) & 1u);
         }
-        if (TRAIN)
-            for (int i = t; i < kPartStride; i += kTile) part[i] = 0.0f;
-    } else if (TRAIN && it > 0) {
+        for (int i = t; i < kPartStride; i += kTile) part[i] = 0.0f;
+    } else if (it > 0) {
         // weight gradients of this CTA's tiles: rows 0..63 of GA are dW2, rows 64..127 columns
         // 64..95 are dW1; rows 0..63 of GC are dW3^T.  Plain stores into the CTA's partial row.
         tc::fence_after_sync();
@@ -644,26 +712,168 @@ __global__ void __launch_bounds__(kTile, TRAIN ? 1 : 2) k_nrc_mlp(MlpArgs a) {
     if (warp == 0) tc::tmem_dealloc(tmem, kTmCols);
 }
 
+// Forward only, four CTAs of 128 threads per SM (two with the training kernel's layout: 43 us for
+// 323 k samples, a chain of three products and three tensor-memory reads per tile with too little
+// else on the SM; 25 us with four).  The hidden layers share one shared-memory tile and one
+// accumulator: each product has completed before its operand or accumulator is written again.
+__global__ void __launch_bounds__(kTile, 4) k_nrc_infer(InferArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t bar_w, bar_ld[2], bar_mma;
+    __shared__ uint32_t tmem_s;
+    __shared__ int abort_s;
+    const uint32_t t = threadIdx.x, warp = t >> 5;
+    uint32_t n = a.n;
+    if (a.count) n = min(__ldg(a.count), a.n);
+    const uint32_t tiles = (n + kTile - 1) / kTile;
+    if (blockIdx.x >= tiles) return;
+    if (t == 0) {
+        abort_s = 0;
+        tc::mbar_init(&bar_w, 1);
+        tc::mbar_init(&bar_ld[0], 1);
+        tc::mbar_init(&bar_ld[1], 1);
+        tc::mbar_init(&bar_mma, 1);
+        tc::mbar_init_fence();
+    }
+    if (warp == 0) {
+        tc::tmem_alloc(&tmem_s, kInfCols);
+        tc::tmem_relinquish();
+    }
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_s, sm = tc::smem_u32(smem);
+    // what thread 0 started and saw complete (see k_nrc_mlp)
+    uint32_t ld_issued[2] = {0u, 0u}, ld_done[2] = {0u, 0u}, mma_issued = 0u, mma_done = 0u;
+    auto load_tile = [&](uint32_t tile, int buf) {  // thread 0 only
+        ++ld_issued[buf];
+        tc::mbar_expect_tx(&bar_ld[buf], kXTile);
+        tc::bulk_g2s(smem + kInfX + buf * kXTile, reinterpret_cast<const uint8_t *>(a.X) + (size_t)tile * kXTile, kXTile,
+                     &bar_ld[buf]);
+    };
+    if (t == 0) {
+        tc::mbar_expect_tx(&bar_w, kInfX);
+        tc::bulk_g2s(smem + kInfW1, a.wimg + kImgW1, kInfW2 - kInfW1, &bar_w);
+        tc::bulk_g2s(smem + kInfW2, a.wimg + kImgW2, kInfW3 - kInfW2, &bar_w);
+        tc::bulk_g2s(smem + kInfW3, a.wimg + kImgW3P, kInfX - kInfW3, &bar_w);
+        load_tile(blockIdx.x, 0);
+    }
+    const bool w_done = tc::mbar_wait(&bar_w, 0);
+    bool ok = w_done;
+    uint32_t ph = 0, it = 0;
+    auto commit_mma = [&]() {  // thread 0 only
+        tc::commit(&bar_mma);
+        ++mma_issued;
+    };
+    auto mma_wait = [&]() {
+        const bool got = tc::mbar_wait(&bar_mma, ph);
+        if (got) ++mma_done;
+        ok = got && ok;
+        ph ^= 1u;
+        tc::fence_after_sync();
+    };
+    // this thread's row of a hidden layer: ReLU, bf16, into the shared tile; then every row is there
+    auto hidden = [&]() {
+        float z[64];
+        tmem_ld64(tmem, warp, kInfD, z);
+#pragma unroll
+        for (int j = 0; j < 64; ++j) z[j] = fmaxf(z[j], 0.0f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) store_row8(smem + kInfH, kH2Stride, t, 8u * j, z + 8 * j);
+        tc::fence_async_smem();
+        tc::fence_before_sync();
+        if (!ok) abort_s = 1;
+        __syncthreads();
+    };
+    for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+        const int buf = it & 1;
+        const bool got = tc::mbar_wait(&bar_ld[buf], (it >> 1) & 1u);
+        if (got) ++ld_done[buf];
+        ok = got && ok;
+        if (!ok) abort_s = 1;
+        tc::fence_before_sync();
+        __syncthreads();  // the previous tile's output has been read out of tensor memory
+        if (abort_s) break;
+        if (t == 0) {
+            if (tile + gridDim.x < tiles) load_tile(tile + gridDim.x, buf ^ 1);
+            tc::fence_after_sync();
+            for (uint32_t ks = 0; ks < kIn / 16; ++ks)
+                tc::mma_bf16(tmem + kInfD, tc::smem_desc(sm + kInfX + buf * kXTile + ks * 256u, 128u, 512u),
+                             tc::smem_desc(sm + kInfW1 + ks * 256u, 128u, 512u), tc::idesc_bf16(128, 64), ks);
+            commit_mma();
+        }
+        mma_wait();
+        hidden();
+        if (abort_s) break;
+        if (t == 0) {
+            tc::fence_after_sync();
+            for (uint32_t ks = 0; ks < kHid / 16; ++ks)
+                tc::mma_bf16(tmem + kInfD, tc::smem_desc(sm + kInfH + ks * 256u, 128u, kH2Stride),
+                             tc::smem_desc(sm + kInfW2 + ks * 256u, 128u, 1024u), tc::idesc_bf16(128, 64), ks);
+            commit_mma();
+        }
+        mma_wait();
+        hidden();
+        if (abort_s) break;
+        if (t == 0) {
+            tc::fence_after_sync();
+            for (uint32_t ks = 0; ks < kHid / 16; ++ks)
+                tc::mma_bf16(tmem + kInfD3, tc::smem_desc(sm + kInfH + ks * 256u, 128u, kH2Stride),
+                             tc::smem_desc(sm + kInfW3 + ks * 256u, 128u, 1024u), tc::idesc_bf16(128, 16), ks);
+            commit_mma();
+        }
+        mma_wait();
+        float y[16];
+        tc::tmem_ld16(tc::tmem_lane_addr(tmem, warp, kInfD3), y);
+        tc::wait_ld();
+        const uint32_t s = tile * kTile + t;
+        if (s < n && ok) {
+            const uint32_t o = a.out_idx ? __ldg(a.out_idx + s) : s;
+            a.out[o] = make_float4(fmaxf(y[0], 0.0f), fmaxf(y[1], 0.0f), fmaxf(y[2], 0.0f), 1.0f);
+        }
+    }
+    if (!ok) abort_s = 1;
+    tc::fence_before_sync();
+    __syncthreads();
+    if (abort_s && t == 0) {
+        atomicOr(a.err, kErrTimeout);
+        if (!w_done) tc::mbar_wait(&bar_w, 0);
+        for (int b = 0; b < 2; ++b)
+            if (ld_issued[b] > ld_done[b]) tc::mbar_wait(&bar_ld[b], (ld_issued[b] - 1u) & 1u);
+        if (mma_issued > mma_done) tc::mbar_wait(&bar_mma, (mma_issued - 1u) & 1u);
+    }
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem, kInfCols);
+}
+
 // ---------------------------------------------------------------- gradient scatter and Adam
 
-// Sum the MLP kernel's per-CTA partials into the weight-gradient accumulators and the loss sums.
-// Block = 32 consecutive values x 8 warps; warp w sums parts w, w + 8, ...; then the 8 warp sums
-// in a fixed order (deterministic).
-__global__ void __launch_bounds__(256) k_nrc_wgrad_reduce(const float *wpart, int parts, float *wg, float *stats) {
-    __shared__ float acc[8][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
+// Sum of the network kernel's per-CTA partials of value i (a weight gradient, then the loss sums): a
+// block takes 32 consecutive values x 8 warps; warp w sums parts w, w + 8, ...; then the 8 warp sums in
+// a fixed order (deterministic).  Warp 0 gets the sum; acc: 8 x 32 floats of shared memory.
+__device__ __forceinline__ float wgrad_sum(const float *wpart, int parts, int i, int lane, int w, float *acc) {
     float s = 0.0f;
     if (i < kWCount + 3) {
 #pragma unroll 4
         for (int p = w; p < parts; p += 8) s += __ldcg(wpart + (size_t)p * kPartStride + i);
     }
-    acc[w][lane] = s;
+    acc[32 * w + lane] = s;
     __syncthreads();
-    if (w == 0 && i < kWCount + 3) {
-        float t = 0.0f;
+    float t = 0.0f;
+    if (w == 0) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t += acc[k][lane];
+        for (int k = 0; k < 8; ++k) t += acc[32 * k + lane];
+    }
+    return t;
+}
+
+// ... added to the weight-gradient accumulators and the loss sums.
+__global__ void __launch_bounds__(256) k_nrc_wgrad_reduce(const float *wpart, int parts, float *wg, float *stats) {
+    __shared__ float acc[8 * 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    const float t = wgrad_sum(wpart, parts, i, lane, w, acc);
+    if (w == 0 && i < kWCount + 3) {
         if (i < kWCount) wg[i] += t;
         else stats[i - kWCount] += t;
     }
@@ -698,42 +908,90 @@ __device__ __forceinline__ float adam_update(float p, float &m, float &v, float 
     return p - a.lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
 }
 
+struct AdamTableArgs {
+    Entry *tab;
+    float2 *grad;
+    __half2 *tab16;
+    uint32_t log2_table;
+    uint32_t chunk0[kL + 1];  // first chunk of kAdamChunk entries of each level, then their number
+};
+constexpr int kAdamWarps = 8, kAdamChunk = 256, kAdamBlocksPerSm = 4;
+
 // Sparse Adam on the table: an entry whose gradient is (0, 0) this step keeps its value and its
 // moments (the samples of the step did not touch it); the others take an Adam step with the
-// global step count's bias correction.  Gradients are cleared as they are consumed.  A thread
-// takes 4 consecutive entries: one 32-byte gradient read, then the touched entries' loads issued
-// together before any is used.  total is a multiple of 4.
-__global__ void __launch_bounds__(256) k_nrc_adam_table(Entry *tab, float2 *grad, __half2 *tab16, uint64_t total,
-                                                        AdamArgs a) {
-    const uint64_t groups = total >> 2;
-    for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < groups;
-         q += (uint64_t)gridDim.x * blockDim.x) {
-        float4 *gq = reinterpret_cast<float4 *>(grad) + 2 * q;
-        const float4 g01 = gq[0], g23 = gq[1];
-        const float2 g[4] = {make_float2(g01.x, g01.y), make_float2(g01.z, g01.w), make_float2(g23.x, g23.y),
-                             make_float2(g23.z, g23.w)};
-        bool t[4];
-        bool any = false;
+// global step count's bias correction.  Gradients are cleared as they are consumed.
+// A step touches an eighth of the entries, at hash-random places.  A warp therefore reads the
+// gradients of 256 consecutive entries (four 16-byte loads a lane in flight), lists the touched ones in
+// shared memory and updates the list lane by lane, so that every lane holds an entry's loads and
+// arithmetic instead of one in eight (4 entries a thread, skipping the untouched: 40 us a step of 16,384
+// samples, 2^19 entries a level; this form with the weights 27.5 us).
+__device__ __forceinline__ void adam_table(const AdamTableArgs &t, const AdamArgs &a, uint32_t warp, uint32_t warps,
+                                           float2 *s_g, uint16_t *s_i) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t c = warp; c < t.chunk0[kL]; c += warps) {
+        uint32_t l = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            t[k] = g[k].x != 0.0f || g[k].y != 0.0f;
-            any |= t[k];
+        for (int k = 1; k < kL; ++k) l += c >= t.chunk0[k] ? 1u : 0u;
+        uint32_t first = t.chunk0[0];
+#pragma unroll
+        for (int k = 1; k < kL; ++k) first = c >= t.chunk0[k] ? t.chunk0[k] : first;
+        const size_t e0 = ((size_t)l << t.log2_table) + (size_t)(c - first) * kAdamChunk;
+        float4 *gq = reinterpret_cast<float4 *>(t.grad + e0);
+        float4 g[kAdamChunk / 64];
+#pragma unroll
+        for (int j = 0; j < kAdamChunk / 64; ++j) g[j] = __ldcg(gq + 32 * j + lane);
+        uint32_t hit = 0;
+#pragma unroll
+        for (int j = 0; j < kAdamChunk / 64; ++j) {
+            if (g[j].x != 0.0f || g[j].y != 0.0f) hit |= 1u << (2 * j);
+            if (g[j].z != 0.0f || g[j].w != 0.0f) hit |= 2u << (2 * j);
+            if ((hit >> (2 * j)) & 3u) gq[32 * j + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if (!any) continue;
-        Entry e[4];
+        const int cnt = __popc(hit);
+        int incl = cnt;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (t[k]) e[k] = tab[4 * q + k];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (!t[k]) continue;
-            e[k].p.x = adam_update(e[k].p.x, e[k].m.x, e[k].v.x, g[k].x, a);
-            e[k].p.y = adam_update(e[k].p.y, e[k].m.y, e[k].v.y, g[k].y, a);
-            tab[4 * q + k] = e[k];
-            tab16[4 * q + k] = __floats2half2_rn(e[k].p.x, e[k].p.y);
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if ((int)lane >= d) incl += v;
         }
-        gq[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-        gq[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        int pos = incl - cnt;
+#pragma unroll
+        for (int j = 0; j < kAdamChunk / 64; ++j) {
+            if ((hit >> (2 * j)) & 1u) {
+                s_i[pos] = (uint16_t)(64 * j + 2 * lane);
+                s_g[pos++] = make_float2(g[j].x, g[j].y);
+            }
+            if ((hit >> (2 * j)) & 2u) {
+                s_i[pos] = (uint16_t)(64 * j + 2 * lane + 1);
+                s_g[pos++] = make_float2(g[j].z, g[j].w);
+            }
+        }
+        __syncwarp();
+        for (int k = (int)lane; k < total; k += 64) {
+            float4 pm[2], vp[2];
+            size_t e[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (k + 32 * u >= total) continue;
+                e[u] = e0 + s_i[k + 32 * u];
+                const float4 *src = reinterpret_cast<const float4 *>(t.tab + e[u]);
+                pm[u] = __ldcg(src);
+                vp[u] = __ldcg(src + 1);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (k + 32 * u >= total) continue;
+                const float2 gr = s_g[k + 32 * u];
+                pm[u].x = adam_update(pm[u].x, pm[u].z, vp[u].x, gr.x, a);
+                pm[u].y = adam_update(pm[u].y, pm[u].w, vp[u].y, gr.y, a);
+                float4 *dst = reinterpret_cast<float4 *>(t.tab + e[u]);
+                dst[0] = pm[u];
+                dst[1] = vp[u];
+                t.tab16[e[u]] = __floats2half2_rn(pm[u].x, pm[u].y);
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -756,68 +1014,124 @@ __device__ __forceinline__ void put_bf16(uint8_t *img, uint32_t off, float v) {
     *reinterpret_cast<__nv_bfloat16 *>(img + off) = __float2bfloat16_rn(v);
 }
 
-// Adam on the weights (update != 0), then the bf16 images W, W^T of every layer.
-__global__ void __launch_bounds__(256) k_nrc_adam_mlp(float *w, float *m, float *v, float *g, uint8_t *img, int update,
-                                                      AdamArgs a) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kWCount; i += gridDim.x * blockDim.x) {
-        float p = w[i];
-        if (update) {
-            float mm = m[i], vv = v[i];
-            p = adam_update(p, mm, vv, g[i], a);
-            m[i] = mm;
-            v[i] = vv;
-            g[i] = 0.0f;
-            w[i] = p;
-        }
-        if (i < kW2) {
-            const uint32_t o = i / kIn, k = i % kIn;
-            put_bf16(img, kImgW1 + tc::cm_offset(o, k, kIn), p);
-            put_bf16(img, kImgW1T + tc::cm_offset(k, o, kHid), p);
-        } else if (i < kW3) {
-            const uint32_t o = (i - kW2) / kHid, k = (i - kW2) % kHid;
-            put_bf16(img, kImgW2 + tc::cm_offset(o, k, kHid), p);
-            put_bf16(img, kImgW2T + tc::cm_offset(k, o, kHid), p);
-        } else {
-            const uint32_t o = (i - kW3) / kHid, k = (i - kW3) % kHid;
-            put_bf16(img, kImgW3P + tc::cm_offset(o, k, kHid), p);
-            put_bf16(img, kImgW3PT + tc::cm_offset(k, o, 16), p);
-        }
+// Weight i's value into the bf16 images W, W^T of its layer.
+__device__ __forceinline__ void weight_images(uint8_t *img, int i, float p) {
+    if (i < kW2) {
+        const uint32_t o = i / kIn, k = i % kIn;
+        put_bf16(img, kImgW1 + tc::cm_offset(o, k, kIn), p);
+        put_bf16(img, kImgW1T + tc::cm_offset(k, o, kHid), p);
+    } else if (i < kW3) {
+        const uint32_t o = (i - kW2) / kHid, k = (i - kW2) % kHid;
+        put_bf16(img, kImgW2 + tc::cm_offset(o, k, kHid), p);
+        put_bf16(img, kImgW2T + tc::cm_offset(k, o, kHid), p);
+    } else {
+        const uint32_t o = (i - kW3) / kHid, k = (i - kW3) % kHid;
+        put_bf16(img, kImgW3P + tc::cm_offset(o, k, kHid), p);
+        put_bf16(img, kImgW3PT + tc::cm_offset(k, o, 16), p);
     }
+}
+
+// The bf16 images from the master weights.
+__global__ void __launch_bounds__(256) k_nrc_images(const float *w, uint8_t *img) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kWCount) weight_images(img, i, w[i]);
+}
+
+// One Adam step: blocks 0 .. kAdamWBlocks - 1 take 32 weights (and the loss sums) each, with the
+// network kernel's per-CTA partials added to their gradients as k_nrc_wgrad_reduce does (parts = 0:
+// none), the others the table.  One launch, so that the weights' two short passes cost no launches of
+// their own (4.9 and 2.9 us a step).
+struct AdamWeightArgs {
+    float *w, *m, *v, *g;
+    uint8_t *img;
+    const float *wpart;
+    int parts;
+    float *stats;
+};
+constexpr int kAdamWBlocks = (kWCount + 3 + 31) / 32;
+__global__ void __launch_bounds__(32 * kAdamWarps, kAdamBlocksPerSm) k_nrc_adam(AdamTableArgs t, AdamWeightArgs q, AdamArgs a) {
+    __shared__ float2 s_g[kAdamWarps][kAdamChunk];
+    __shared__ uint16_t s_i[kAdamWarps][kAdamChunk];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (blockIdx.x >= kAdamWBlocks) {
+        adam_table(t, a, (blockIdx.x - kAdamWBlocks) * kAdamWarps + w, (gridDim.x - kAdamWBlocks) * kAdamWarps, s_g[w],
+                   s_i[w]);
+        return;
+    }
+    const int i = blockIdx.x * 32 + lane;
+    const float sum = wgrad_sum(q.wpart, q.parts, i, lane, w, &s_g[0][0].x);
+    if (w != 0 || i >= kWCount + 3) return;
+    if (i >= kWCount) {
+        if (q.parts) q.stats[i - kWCount] += sum;
+        return;
+    }
+    float mm = q.m[i], vv = q.v[i];
+    const float g = q.parts ? q.g[i] + sum : q.g[i];
+    const float p = adam_update(q.w[i], mm, vv, g, a);
+    q.m[i] = mm;
+    q.v[i] = vv;
+    q.g[i] = 0.0f;
+    q.w[i] = p;
+    weight_images(q.img, i, p);
 }
 
 // ---------------------------------------------------------------- query selection
 
-__global__ void __launch_bounds__(256) k_nrc_select(SelectArgs a) {
-    const uint32_t lane = threadIdx.x & 31u;
+// A block takes 64 words (2048 records) at a time: each warp decides its 8 words, the block's answered
+// records take consecutive places with one addition to the counter (one addition per warp of 32
+// records, 64,800 at 1080p on one address, took 57 us, next to nothing of it the reads; now 29 us).
+constexpr int kSelWarps = 8, kSelWords = 8;
+__global__ void __launch_bounds__(32 * kSelWarps) k_nrc_select(SelectArgs a) {
+    __shared__ uint32_t s_cnt[kSelWarps], s_base;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const bool trusted = a.trained && __ldg(a.stats + 2) > 0.0f && __ldg(a.stats + 1) <= a.trust * __ldg(a.stats + 2);
     const uint32_t words = (a.n + 31u) / 32u;
-    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    for (uint32_t wd = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; wd < words; wd += warps) {
-        const uint32_t r = wd * 32u + lane;
-        bool use = false;
-        if (r < a.n && record_hit(a.pos, a.len, r)) {
-            const uint32_t slot = __ldg(a.slot_ids + r);
-            if (slot == GI_SLOT_FAR) {
-                // left out of the table by the update (gi_cache_route_far): the network is its only answer
-                use = true;
-            } else if (!trusted) {
-            } else if (slot == GI_SLOT_NONE) {
-                use = true;
-            } else if (slot < a.cv.slots) {
-                const bool cold = cache_cold(a.cv, slot);
-                use = cold || key_lod(a.kp, __ldg(a.pos[0] + r), __ldg(a.pos[1] + r), __ldg(a.pos[2] + r)) >=
-                                  (int)a.query_lod;
+    for (uint32_t b0 = blockIdx.x * (kSelWarps * kSelWords); b0 < words; b0 += gridDim.x * (kSelWarps * kSelWords)) {
+        const uint32_t w0 = b0 + warp * kSelWords;
+        uint32_t ball[kSelWords], total = 0;
+#pragma unroll
+        for (int k = 0; k < kSelWords; ++k) {
+            const uint32_t r = (w0 + k) * 32u + lane;
+            bool use = false;
+            if (r < a.n && record_hit(a.pos, a.len, r)) {
+                const uint32_t slot = __ldg(a.slot_ids + r);
+                if (slot == GI_SLOT_FAR) {
+                    // left out of the table by the update (gi_cache_route_far): the network is its only answer
+                    use = true;
+                } else if (!trusted) {
+                } else if (slot == GI_SLOT_NONE) {
+                    use = true;
+                } else if (slot < a.cv.slots) {
+                    use = cache_cold(a.cv, slot) ||
+                          key_lod(a.kp, __ldg(a.pos[0] + r), __ldg(a.pos[1] + r), __ldg(a.pos[2] + r)) >= (int)a.query_lod;
+                }
             }
+            ball[k] = __ballot_sync(0xFFFFFFFFu, use);
+            total += __popc(ball[k]);
         }
-        const uint32_t ball = __ballot_sync(0xFFFFFFFFu, use);
-        uint32_t base = 0;
-        if (lane == 0 && ball) base = atomicAdd(a.qcount, __popc(ball));
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        const uint32_t pos = base + __popc(ball & ((1u << lane) - 1u));
-        use = use && pos < a.max_q;
-        if (use) a.qidx[pos] = r;
-        const uint32_t kept = __ballot_sync(0xFFFFFFFFu, use);
-        if (lane == 0) a.bits[wd] = kept;
+        if (lane == 0) s_cnt[warp] = total;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t sum = 0;
+            for (int w = 0; w < kSelWarps; ++w) {
+                const uint32_t c = s_cnt[w];
+                s_cnt[w] = sum;
+                sum += c;
+            }
+            s_base = sum ? atomicAdd(a.qcount, sum) : 0u;
+        }
+        __syncthreads();
+        uint32_t base = s_base + s_cnt[warp];
+#pragma unroll
+        for (int k = 0; k < kSelWords; ++k) {
+            const uint32_t pos = base + __popc(ball[k] & ((1u << lane) - 1u));
+            const bool use = ((ball[k] >> lane) & 1u) && pos < a.max_q;
+            if (use) a.qidx[pos] = (w0 + k) * 32u + lane;
+            const uint32_t kept = __ballot_sync(0xFFFFFFFFu, use);
+            if (lane == 0 && w0 + k < words) a.bits[w0 + k] = kept;
+            base += __popc(ball[k]);
+        }
+        __syncthreads();  // the next round reuses the block's counters
     }
 }
 
@@ -877,6 +1191,7 @@ struct gi_nrc_s {
     uint64_t last_query_n = 0;
     bool queried = false;
     uint64_t steps = 0;
+    bool grads_set = false;      // table gradients written by the caller since the last Adam step
     uint32_t last_minibatches = 1;
     int sms = 1;
 };
@@ -940,42 +1255,39 @@ EncArgs enc_base(const gi_nrc_s *s) {
     return e;
 }
 
-unsigned enc_blocks(const gi_nrc_s *s, uint64_t work) {
-    const uint64_t b = (work + kEncThreads - 1) / kEncThreads;
-    const uint64_t cap = (uint64_t)s->sms * 8;
-    return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(b, cap));
+// Blocks of the kernels with one thread per sample and level (n samples, padded to whole tiles).
+unsigned sample_blocks(const gi_nrc_s *s, uint32_t n) {
+    const uint64_t b = (uint64_t)((n + kTile - 1) / kTile * kTile) * kL / kEncThreads;
+    return (unsigned)std::min<uint64_t>(b, (uint64_t)s->sms * 8);
 }
 
-gi_status launch_mlp(gi_nrc_s *s, bool train, uint32_t n, const uint32_t *count, float dy_scale, float4 *out,
-                     const uint32_t *out_idx, cudaStream_t st) {
+// The network on n encoded samples, training: *parts rows of partial sums in s->wpart.
+gi_status launch_train(gi_nrc_s *s, uint32_t n, float dy_scale, int *parts, cudaStream_t st) {
     MlpArgs m;
-    memset(&m, 0, sizeof(m));
     m.X = s->X;
     m.T = s->Tt;
     m.wimg = s->wimg;
     m.n = n;
-    m.count = count;
     m.dy_scale = dy_scale;
     m.loss_eps = s->cfg.loss_eps;
     m.dX = s->dX;
     m.wpart = s->wpart;
-    m.out = out;
-    m.out_idx = out_idx;
     m.err = s->err;
     const uint32_t tiles = (n + kTile - 1) / kTile;
+    *parts = (int)std::min<uint32_t>(tiles, (uint32_t)s->sms);
     if (tiles == 0) return GI_OK;
-    if (train) {
-        const unsigned grid = std::min<uint32_t>(tiles, (uint32_t)s->sms);
-        k_nrc_mlp<true><<<grid, kTile, kSmTrain, st>>>(m);
-        gi_status r = cuda_status(cudaGetLastError(), "k_nrc_mlp launch");
-        if (r != GI_OK) return r;
-        k_nrc_wgrad_reduce<<<(kWCount + 3 + 31) / 32, 256, 0, st>>>(s->wpart, (int)grid, s->wg, s->stats);
-        return cuda_status(cudaGetLastError(), "k_nrc_wgrad_reduce launch");
-    } else {
-        const unsigned grid = std::min<uint32_t>(tiles, 2u * (uint32_t)s->sms);
-        k_nrc_mlp<false><<<grid, kTile, kSmInfer, st>>>(m);
-    }
+    k_nrc_mlp<<<*parts, kTile, kSmTrain, st>>>(m);
     return cuda_status(cudaGetLastError(), "k_nrc_mlp launch");
+}
+
+// Forward only; count: device sample count (at most n), or NULL.
+gi_status launch_infer(gi_nrc_s *s, uint32_t n, const uint32_t *count, float4 *out, const uint32_t *out_idx,
+                       cudaStream_t st) {
+    const uint32_t tiles = (n + kTile - 1) / kTile;
+    if (tiles == 0) return GI_OK;
+    const InferArgs m = {s->X, s->wimg, n, count, out, out_idx, s->err};
+    k_nrc_infer<<<std::min<uint32_t>(tiles, 4u * (uint32_t)s->sms), kTile, kInfBytes, st>>>(m);
+    return cuda_status(cudaGetLastError(), "k_nrc_infer launch");
 }
 
 gi_status scatter_and_return(gi_nrc_s *s, const float *const pos[3], const float *const nrm[3], const uint32_t *idx,
@@ -990,7 +1302,7 @@ gi_status scatter_and_return(gi_nrc_s *s, const float *const pos[3], const float
     c.n = n;
     c.dX = s->dX;
     c.grad = s->grad;
-    k_nrc_scatter<<<enc_blocks(s, (uint64_t)n * kL), kEncThreads, 0, st>>>(c);
+    k_nrc_scatter<<<sample_blocks(s, n), kEncThreads, 0, st>>>(c);
     return cuda_status(cudaGetLastError(), "k_nrc_scatter launch");
 }
 
@@ -1043,10 +1355,9 @@ gi_status read_params(gi_nrc_s *s, float *table, float *w1, float *w2, float *w3
 
 // refresh the float16 table copy and the bf16 weight images from the masters (no Adam step)
 gi_status refresh_copies(gi_nrc_s *s) {
-    AdamArgs a{0.f, 0.f, 0.f, 1.f, 1.f, 1.f};
     const uint64_t entries = (uint64_t)kL * s->T;
     k_nrc_table_f16<<<(unsigned)std::min<uint64_t>((entries + 255) / 256, 65535), 256>>>(s->tab, s->tab16, entries);
-    k_nrc_adam_mlp<<<(kWCount + 255) / 256, 256>>>(s->w, s->wm, s->wv, s->wg, s->wimg, 0, a);
+    k_nrc_images<<<(kWCount + 255) / 256, 256>>>(s->w, s->wimg);
     gi_status st = cuda_status(cudaGetLastError(), "gi_nrc copy refresh");
     if (st == GI_OK) st = cuda_status(cudaDeviceSynchronize(), "gi_nrc copy refresh");
     return st;
@@ -1170,9 +1481,7 @@ gi_status gi_nrc_create(const gi_nrc_config *cfg, gi_nrc_t *out) {
     if (e == cudaSuccess) e = cudaMemset(s->err, 0, 4);
     if (e == cudaSuccess) e = cudaMemset(s->qcount, 0, 4);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_nrc_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmTrain);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_nrc_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmInfer);
+        e = cudaFuncSetAttribute(k_nrc_mlp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmTrain);
     st = cuda_status(e, "gi_nrc_create");
     if (st == GI_OK) {
         // initial parameters from a splitmix64 stream: table, then W1, W2, W3
@@ -1242,6 +1551,7 @@ gi_status gi_nrc_set_gradients(gi_nrc_t nrc, const float *table, const float *w1
     }
     gi_status st = cuda_status(cudaDeviceSynchronize(), "gi_nrc_set_gradients");
     if (st == GI_OK) st = copy_params(nrc, table, w1, w2, w3, true);
+    if (table) nrc->grads_set = true;
     return st;
 }
 
@@ -1269,10 +1579,9 @@ gi_status gi_nrc_infer(gi_nrc_t nrc, const gi_points *pts, float *out, gi_stream
     }
     e.n = pts->n;
     e.T = nullptr;
-    const uint32_t n_pad = (pts->n + kTile - 1) / kTile * kTile;
-    k_nrc_encode<kEncPoints><<<enc_blocks(nrc, (uint64_t)n_pad * kL), kEncThreads, 0, s>>>(e);
+    k_nrc_encode<kEncPoints><<<sample_blocks(nrc, pts->n), kEncThreads, 0, s>>>(e);
     st = cuda_status(cudaGetLastError(), "k_nrc_encode launch");
-    if (st == GI_OK) st = launch_mlp(nrc, false, pts->n, nullptr, 0.f, reinterpret_cast<float4 *>(out), nullptr, s);
+    if (st == GI_OK) st = launch_infer(nrc, pts->n, nullptr, reinterpret_cast<float4 *>(out), nullptr, s);
     return st;
 }
 
@@ -1295,12 +1604,16 @@ gi_status gi_nrc_backward(gi_nrc_t nrc, const gi_points *pts, const float *const
     }
     e.mask = mask;
     e.n = pts->n;
-    const uint32_t n_pad = (pts->n + kTile - 1) / kTile * kTile;
-    k_nrc_encode<kEncPoints><<<enc_blocks(nrc, (uint64_t)n_pad * kL), kEncThreads, 0, s>>>(e);
+    k_nrc_encode<kEncPoints><<<sample_blocks(nrc, pts->n), kEncThreads, 0, s>>>(e);
     st = cuda_status(cudaGetLastError(), "k_nrc_encode launch");
     const float B = (float)(batch_norm ? batch_norm : pts->n);
     nrc->last_minibatches = 1;
-    if (st == GI_OK) st = launch_mlp(nrc, true, pts->n, nullptr, 2.0f / B, nullptr, nullptr, s);
+    int parts = 0;
+    if (st == GI_OK) st = launch_train(nrc, pts->n, 2.0f / B, &parts, s);
+    if (st == GI_OK) {
+        k_nrc_wgrad_reduce<<<(kWCount + 3 + 31) / 32, 256, 0, s>>>(nrc->wpart, parts, nrc->wg, nrc->stats);
+        st = cuda_status(cudaGetLastError(), "k_nrc_wgrad_reduce launch");
+    }
     if (st == GI_OK) st = scatter_and_return(nrc, pts->pos, pts->nrm, nullptr, pts->n, s);
     return st;
 }
@@ -1314,12 +1627,8 @@ gi_status gi_nrc_set_learning_rate(gi_nrc_t nrc, float lr) {
     return GI_OK;
 }
 
-gi_status gi_nrc_adam(gi_nrc_t nrc, gi_stream_t stream) {
-    if (!nrc) {
-        set_error("gi_nrc_adam: NULL surrogate");
-        return GI_ERR_INVALID_ARG;
-    }
-    const cudaStream_t s = (cudaStream_t)stream;
+// One Adam step; parts: rows of s->wpart whose sums belong to the step's weight gradients and losses.
+static gi_status adam_step(gi_nrc_s *nrc, int parts, cudaStream_t s) {
     nrc->steps += 1;
     const double t = (double)nrc->steps;
     AdamArgs a;
@@ -1329,13 +1638,31 @@ gi_status gi_nrc_adam(gi_nrc_t nrc, gi_stream_t stream) {
     a.eps = nrc->cfg.adam_eps;
     a.c1 = (float)(1.0 - std::pow((double)nrc->cfg.beta1, t));
     a.c2 = (float)(1.0 - std::pow((double)nrc->cfg.beta2, t));
-    const uint64_t entries = (uint64_t)kL * nrc->T;
-    const unsigned blocks = (unsigned)std::min<uint64_t>((entries / 4 + 255) / 256, (uint64_t)nrc->sms * 8);
-    k_nrc_adam_table<<<blocks, 256, 0, s>>>(nrc->tab, nrc->grad, nrc->tab16, entries, a);
-    gi_status st = cuda_status(cudaGetLastError(), "k_nrc_adam_table launch");
-    if (st != GI_OK) return st;
-    k_nrc_adam_mlp<<<(kWCount + 255) / 256, 256, 0, s>>>(nrc->w, nrc->wm, nrc->wv, nrc->wg, nrc->wimg, 1, a);
-    return cuda_status(cudaGetLastError(), "k_nrc_adam_mlp launch");
+    AdamTableArgs at;
+    at.tab = nrc->tab;
+    at.grad = nrc->grad;
+    at.tab16 = nrc->tab16;
+    at.log2_table = nrc->cfg.log2_table;
+    at.chunk0[0] = 0;
+    for (int l = 0; l < kL; ++l) {
+        // a dense level's samples reach its first 6 (R + 1)^3 entries; gradients the caller wrote, all
+        const uint64_t V = (uint64_t)nrc->geo.lv.res[l] + 1u;
+        const uint64_t used = nrc->geo.lv.dense[l] && !nrc->grads_set ? 6u * V * V * V : nrc->T;
+        at.chunk0[l + 1] = at.chunk0[l] + (uint32_t)((used + kAdamChunk - 1) / kAdamChunk);
+    }
+    nrc->grads_set = false;
+    const AdamWeightArgs aw = {nrc->w, nrc->wm, nrc->wv, nrc->wg, nrc->wimg, nrc->wpart, parts, nrc->stats};
+    const unsigned blocks = std::min<uint32_t>((at.chunk0[kL] + kAdamWarps - 1) / kAdamWarps, (uint32_t)nrc->sms * kAdamBlocksPerSm);
+    k_nrc_adam<<<kAdamWBlocks + blocks, 32 * kAdamWarps, 0, s>>>(at, aw, a);
+    return cuda_status(cudaGetLastError(), "k_nrc_adam launch");
+}
+
+gi_status gi_nrc_adam(gi_nrc_t nrc, gi_stream_t stream) {
+    if (!nrc) {
+        set_error("gi_nrc_adam: NULL surrogate");
+        return GI_ERR_INVALID_ARG;
+    }
+    return adam_step(nrc, 0, (cudaStream_t)stream);
 }
 
 gi_status gi_nrc_train_frame(gi_nrc_t nrc, gi_cache_t cache, const gi_hits *hits, const uint32_t *slot_ids,
@@ -1365,14 +1692,14 @@ gi_status gi_nrc_train_frame(gi_nrc_t nrc, gi_cache_t cache, const gi_hits *hits
     e.seed = pcg_hash(frame + 1u);
     e.slot_ids = slot_ids;
     e.cv = cache_view(cache);
-    const uint32_t n_pad = (B + kTile - 1) / kTile * kTile;
     for (uint32_t j = 0; j < steps && st == GI_OK; ++j) {
         e.offset = j * B;
-        k_nrc_encode<kEncSampled><<<enc_blocks(nrc, (uint64_t)n_pad * kL), kEncThreads, 0, s>>>(e);
+        k_nrc_encode<kEncSampled><<<sample_blocks(nrc, B), kEncThreads, 0, s>>>(e);
         st = cuda_status(cudaGetLastError(), "k_nrc_encode launch");
-        if (st == GI_OK) st = launch_mlp(nrc, true, B, nullptr, 2.0f / (float)B, nullptr, nullptr, s);
+        int parts = 0;
+        if (st == GI_OK) st = launch_train(nrc, B, 2.0f / (float)B, &parts, s);
         if (st == GI_OK) st = scatter_and_return(nrc, hits->pos, hits->nrm, nrc->idx, B, s);
-        if (st == GI_OK) st = gi_nrc_adam(nrc, stream);
+        if (st == GI_OK) st = adam_step(nrc, parts, s);
     }
     nrc->last_minibatches = steps;
     return st;
@@ -1411,8 +1738,9 @@ gi_status gi_nrc_query_frame(gi_nrc_t nrc, gi_cache_t cache, const gi_hits *hits
     a.qcount = nrc->qcount;
     a.bits = nrc->bits;
     const uint32_t words = (a.n + 31u) / 32u;
-    const unsigned blocks = (unsigned)std::max<uint32_t>(1, std::min<uint32_t>((words + 7) / 8, (uint32_t)nrc->sms * 8));
-    k_nrc_select<<<blocks, 256, 0, s>>>(a);
+    const uint32_t per = kSelWarps * kSelWords;
+    const unsigned blocks = std::min<uint32_t>((words + per - 1) / per, (uint32_t)nrc->sms * 8);
+    k_nrc_select<<<blocks, 32 * kSelWarps, 0, s>>>(a);
     st = cuda_status(cudaGetLastError(), "k_nrc_select launch");
     if (st != GI_OK || nrc->cfg.max_queries == 0) return st;
     EncArgs e = enc_base(nrc);
@@ -1425,9 +1753,9 @@ gi_status gi_nrc_query_frame(gi_nrc_t nrc, gi_cache_t cache, const gi_hits *hits
     e.qidx = nrc->qidx;
     e.qcount = nrc->qcount;
     e.T = nullptr;
-    k_nrc_encode<kEncQueries><<<(unsigned)nrc->sms * 8, kEncThreads, 0, s>>>(e);
+    k_nrc_encode_queries<<<(unsigned)(nrc->sms * kEncBlocksPerSm), kEncThreads, 0, s>>>(e);
     st = cuda_status(cudaGetLastError(), "k_nrc_encode launch");
-    if (st == GI_OK) st = launch_mlp(nrc, false, nrc->cfg.max_queries, nrc->qcount, 0.f, nrc->ovr, nrc->qidx, s);
+    if (st == GI_OK) st = launch_infer(nrc, nrc->cfg.max_queries, nrc->qcount, nrc->ovr, nrc->qidx, s);
     return st;
 }
 

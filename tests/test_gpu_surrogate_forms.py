@@ -1,0 +1,78 @@
+"""The surrogate's kernels come in forms picked by the number of samples (levels per group of the far-hit
+encoding, CTAs per tile of the inference); every form computes a sample's answer with the same operations,
+so all must agree bit for bit."""
+import numpy as np
+import pytest
+
+import paper_2310_19855_gb300 as gi
+import workload as wl
+from _gpu_util import dev, require_gpu, u32
+
+pytestmark = pytest.mark.gpu
+
+import torch  # noqa: E402
+
+SI = wl.surrogate_inputs
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def _network(n, aabb=SI.CORNELL_AABB):
+    cfg = gi.make_nrc_config(*aabb, log2_table=14, resolutions=SI.SMALL_RESOLUTIONS, batch=4096, train_steps=1,
+                             lr=1e-30, trust=1e30, query_lod=0, max_records=n, max_queries=n)
+    nrc = gi.gi_nrc_create(cfg)
+    gi.gi_nrc_set_params(nrc, *SI.params(3, 14))
+    return nrc
+
+
+def _infer(nrc, P, N, n):
+    out = torch.empty((n, 4), device="cuda")
+    gi.gi_nrc_infer(nrc, gi.make_points(P, N, n), out)
+    return out
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 5000, 80_001])
+def test_inference_of_any_count_equals_tile_by_tile(n):
+    nrc = _network(128)
+    try:
+        pos, nrm = SI.points(5, n)
+        P, N = dev(pos), dev(nrm)
+        whole = _infer(nrc, P, N, n)
+        for a in sorted({0, (n // 2) // 128 * 128, (n - 1) // 128 * 128}):
+            m = min(128, n - a)
+            part = _infer(nrc, P[:, a:a + m].contiguous(), N[:, a:a + m].contiguous(), m)
+            assert torch.equal(whole[a:a + m], part), a
+    finally:
+        gi.gi_nrc_destroy(nrc)
+
+
+@pytest.mark.parametrize("n", [33, 9_999, 30_011, 70_001, 140_003, 260_001])
+def test_answers_of_a_view_equal_the_inference_of_their_points(n):
+    # from below two samples a warp up to groups of 16 levels
+    rec = wl.records_random(n, 11, extent=0.9, cam=(0.0, 1.0, 0.0))
+    view = gi.make_view(0, 640, 360, (0, 1, 3), (0, 0, -1), (1, 0, 0), (0, 1, 0), 1.0)
+    R = dev(rec)
+    hits = gi.hits_from_planes(R, n)
+    cache = gi.gi_cache_create(18)
+    nrc = _network(n)
+    try:
+        slots = torch.empty(n, dtype=torch.int32, device="cuda")
+        gi.gi_cache_update(cache, hits, view, slots)
+        gi.gi_cache_resolve(cache, 0)
+        gi.gi_nrc_train_frame(nrc, cache, hits, slots, 0)  # a step too small to move a parameter: trusted
+        gi.gi_nrc_query_frame(nrc, cache, hits, slots, view)
+        m = gi.gi_nrc_answers(nrc)
+        assert m == int(np.isfinite(rec[9]).sum())  # every hit is cold or of LOD >= 0
+        records = torch.empty(m, dtype=torch.int32, device="cuda")
+        rad = torch.empty((m, 4), device="cuda")
+        gi.gi_nrc_answers(nrc, records, rad, m)
+        at = torch.from_numpy(u32(records).astype(np.int64)).cuda()
+        assert torch.equal(torch.sort(at)[0], torch.nonzero(torch.isfinite(R[9]))[:, 0])
+        P, N = R[0:3, at].contiguous(), R[3:6, at].contiguous()
+        assert torch.equal(rad, _infer(nrc, P, N, m))
+    finally:
+        gi.gi_nrc_destroy(nrc)
+        gi.gi_cache_destroy(cache)
