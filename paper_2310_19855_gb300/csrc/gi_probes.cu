@@ -247,50 +247,43 @@ __device__ __forceinline__ bool ray_sample(const IntegrateArgs &a, uint32_t s, f
     return s == GI_SLOT_MISS;
 }
 
-// Cell radiance of probe p's rays (one warp; lane l owns cells l and l + 32, ray k samples cell
-// k mod 64): L = per-cell mean of the rays that produced a sample, with the radiance backup (mean
-// over populated cells) where none did; with HITDIST also hd = the mean ray length of the cell's
-// rays that hit a surface (+inf when none did).  With SURR, records whose bit is set in
-// a.ovr_bits take their radiance from a.ovr (the surrogate's answers) instead of the cache.
-template <bool SURR, bool HITDIST>
-__device__ __forceinline__ void gather_cells(const IntegrateArgs &a, uint32_t p, int lane, float (&L)[2][3],
-                                             float (&hd)[2]) {
+// Cell radiance and hit distance of probe p's rays (one warp; lane l owns cells l and l + 32, ray k
+// samples cell k mod 64): L = per-cell mean of the rays that produced a sample, with the radiance backup
+// (mean over populated cells) where none did; hd = the mean ray length of the cell's rays that hit a
+// surface (+inf when none did).  The first 64 rays' slot ids and lengths come in `first` (they do not
+// depend on the probe, so that the caller loads them beside what tells whether it exists: 24.2 -> 21.6 us
+// for the gather of a 1080p frame, 18.6 -> 17.7 us for the temporal one at 2x2 upscale).
+struct RayPair {
+    uint32_t s0, s1;
+    float l0, l1;
+};
+__device__ __forceinline__ RayPair load_rays(const IntegrateArgs &a, size_t rec) {
+    RayPair r;
+    r.s0 = __ldcs(a.slot_ids + rec);
+    r.s1 = __ldcs(a.slot_ids + rec + 32);
+    r.l0 = __ldcs(a.ray_len + rec);
+    r.l1 = __ldcs(a.ray_len + rec + 32);
+    return r;
+}
+__device__ __forceinline__ void gather_cells(const IntegrateArgs &a, uint32_t p, int lane, RayPair first,
+                                             float (&L)[2][3], float (&hd)[2]) {
     float acc[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
     float cnt[2] = {0.f, 0.f};
     float hs[2] = {0.f, 0.f}, hn[2] = {0.f, 0.f};
-    const uint32_t *ids = a.slot_ids + (size_t)p * a.rpp;
+    RayPair ray = first;
     for (uint32_t k = lane; k < a.rpp; k += 64) {
+        if (k != (uint32_t)lane) ray = load_rays(a, (size_t)p * a.rpp + k);
         // rays k and k + 32 sample cells lane and lane + 32; both gathers in flight together
-        const uint32_t s0 = __ldcs(ids + k), s1 = __ldcs(ids + k + 32);
         float3 r0, r1;
-        bool h0 = ray_sample(a, s0, r0), h1 = ray_sample(a, s1, r1);
-        if (SURR) {
-            // rpp is a multiple of 64: rays k and k + 32 are bit `lane` of two consecutive words
-            const size_t rec = (size_t)p * a.rpp + k;
-            const uint32_t w0 = __ldg(a.ovr_bits + (rec >> 5)), w1 = __ldg(a.ovr_bits + (rec >> 5) + 1);
-            if ((w0 >> lane) & 1u) {
-                const float4 o = __ldg(a.ovr + rec);
-                r0 = make_float3(o.x, o.y, o.z);
-                h0 = true;
-            }
-            if ((w1 >> lane) & 1u) {
-                const float4 o = __ldg(a.ovr + rec + 32);
-                r1 = make_float3(o.x, o.y, o.z);
-                h1 = true;
-            }
-        }
+        const bool h0 = ray_sample(a, ray.s0, r0), h1 = ray_sample(a, ray.s1, r1);
         if (h0) {
             acc[0][0] += r0.x; acc[0][1] += r0.y; acc[0][2] += r0.z; cnt[0] += 1.0f;
         }
         if (h1) {
             acc[1][0] += r1.x; acc[1][1] += r1.y; acc[1][2] += r1.z; cnt[1] += 1.0f;
         }
-        if (HITDIST) {
-            const size_t rec = (size_t)p * a.rpp + k;
-            const float l0 = __ldcs(a.ray_len + rec), l1 = __ldcs(a.ray_len + rec + 32);
-            if (h0 && isfinite(l0) && l0 >= 0.0f) { hs[0] += l0; hn[0] += 1.0f; }
-            if (h1 && isfinite(l1) && l1 >= 0.0f) { hs[1] += l1; hn[1] += 1.0f; }
-        }
+        if (h0 && isfinite(ray.l0) && ray.l0 >= 0.0f) { hs[0] += ray.l0; hn[0] += 1.0f; }
+        if (h1 && isfinite(ray.l1) && ray.l1 >= 0.0f) { hs[1] += ray.l1; hn[1] += 1.0f; }
     }
     // cell means, then the radiance backup: cells without sample take the mean of populated cells
     float pop[4] = {0.f, 0.f, 0.f, 0.f};
@@ -302,12 +295,15 @@ __device__ __forceinline__ void gather_cells(const IntegrateArgs &a, uint32_t p,
         }
         pop[3] += cnt[h] > 0.f ? 1.0f : 0.0f;
     }
-    for (int o = 16; o; o >>= 1)
-        for (int c = 0; c < 4; ++c) pop[c] += __shfl_xor_sync(kFullMask, pop[c], o);
-    const float binv = pop[3] > 0.f ? 1.0f / pop[3] : 0.0f;
-    for (int h = 0; h < 2; ++h)
-        if (cnt[h] == 0.f)
-            for (int c = 0; c < 3; ++c) L[h][c] = pop[c] * binv;
+    // (only a probe with an empty cell needs the sums)
+    if (__any_sync(kFullMask, cnt[0] == 0.f || cnt[1] == 0.f)) {
+        for (int o = 16; o; o >>= 1)
+            for (int c = 0; c < 4; ++c) pop[c] += __shfl_xor_sync(kFullMask, pop[c], o);
+        const float binv = pop[3] > 0.f ? 1.0f / pop[3] : 0.0f;
+        for (int h = 0; h < 2; ++h)
+            if (cnt[h] == 0.f)
+                for (int c = 0; c < 3; ++c) L[h][c] = pop[c] * binv;
+    }
     for (int h = 0; h < 2; ++h) hd[h] = hn[h] > 0.f ? hs[h] / hn[h] : INFINITY;
 }
 
@@ -369,12 +365,13 @@ constexpr int kIntThreads = 128;  // 32 probes per block
 constexpr int kMomStride = 12;    // floats per cell in the shared moment table
 constexpr int kIntPass = 8;       // cells per thread whose loads are in flight together
 
-// Entry 4 i + h of the table holds cell 16 h + i, the i-th cell of thread h: the four threads of a
-// quad read four entries 48 bytes apart (distinct banks).
+// Entry 4 i + h of the table holds the i-th cell of thread h of a quad, cell 16 h + i (RUNS) or 4 i + h:
+// the four threads of a quad read four entries 48 bytes apart (distinct banks).
+template <bool RUNS>
 __device__ __forceinline__ void load_moment_table(float *s_mom) {
     for (int k = threadIdx.x; k < 64 * kMomStride; k += blockDim.x) {
         const int e = k / kMomStride, m = k - e * kMomStride;
-        const int c = 16 * (e & 3) + (e >> 2);
+        const int c = RUNS ? 16 * (e & 3) + (e >> 2) : e;
         s_mom[k] = m < 10 ? g_moments[m][c] : 0.0f;
     }
 }
@@ -522,55 +519,58 @@ __device__ __forceinline__ void integrate_body(const IntegrateArgs &a, uint32_t 
 template <bool RPC1>
 __global__ void __launch_bounds__(kIntThreads, 4) k_integrate(IntegrateArgs a) {
     __shared__ __align__(16) float s_mom[64 * kMomStride];
-    load_moment_table(s_mom);
+    load_moment_table<true>(s_mom);
     __syncthreads();
     integrate_body<false, RPC1>(a, blockIdx.x, s_mom);
 }
 
 // Probe atlas: float4 per (probe, cell) = (mean radiance rgb, mean hit distance); zeros for no probe.
-__global__ void __launch_bounds__(256) k_gather(IntegrateArgs a, float4 *atlas) {
+constexpr int kGatherThreads = 256;
+__global__ void __launch_bounds__(kGatherThreads) k_gather(IntegrateArgs a, float4 *atlas) {
     const uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (p >= a.probes) return;
     float4 *dst = atlas + (size_t)p * 64;
-    if (__ldg(a.nrm + p).w == 0.0f) {
+    const RayPair first = load_rays(a, (size_t)p * a.rpp + lane);
+    if (__ldg(&a.nrm[p].w) == 0.0f) {
         dst[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         dst[lane + 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
     float L[2][3], hd[2];
-    gather_cells<false, true>(a, p, lane, L, hd);
+    gather_cells(a, p, lane, first, L, hd);
     dst[lane] = make_float4(L[0][0], L[0][1], L[0][2], hd[0]);
     dst[lane + 32] = make_float4(L[1][0], L[1][1], L[1][2], hd[1]);
 }
 
-// SH coefficients of every probe from its atlas, four threads per probe as in the probe pass:
-// thread h reads the consecutive cells 16 h + i (eight 16-byte loads in flight at a time) and adds
-// each cell's radiance times its direction moments (shared table); two xor-shuffle steps add the
-// quad's moments, then thread h < 3 projects channel h.  (1080p: one warp per probe with a
-// 31-shuffle reduce-scatter took 19.5 us.)
+// SH coefficients of every probe from its atlas, four threads per probe as in the probe pass, but
+// thread h takes the cells 4 i + h: the quad reads 64 consecutive bytes at a time (eight 16-byte loads a
+// thread in flight), and adds each cell's radiance times its direction moments (shared table); two
+// xor-shuffle steps add the quad's moments, then thread h < 3 projects channel h.  (Cells 16 h + i, one
+// sector per lane and load: 15.4 us at 1080p, now 10.8 us.  The rows staged in shared memory by
+// asynchronous copies: 15.5 us, six blocks per SM leave a second wave of a tenth of them.)
 constexpr int kProjThreads = 128;  // 32 probes per block
 __global__ void __launch_bounds__(kProjThreads) k_project(const float4 *atlas, const float4 *nrm, float *sh,
                                                           uint32_t probes) {
     __shared__ __align__(16) float s_mom[64 * kMomStride];
-    load_moment_table(s_mom);
-    __syncthreads();
-    const uint32_t p = blockIdx.x * (kProjThreads / 4) + (threadIdx.x >> 2);
+    load_moment_table<false>(s_mom);
     const int h = threadIdx.x & 3;
+    const uint32_t p = blockIdx.x * (kProjThreads / 4) + (threadIdx.x >> 2);
     const bool valid = p < probes;
     float4 n4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (valid) n4 = __ldg(nrm + p);
     const bool live = valid && n4.w != 0.0f;
+    __syncthreads();
     float S[10][3];
 #pragma unroll
     for (int m = 0; m < 10; ++m) S[m][0] = S[m][1] = S[m][2] = 0.0f;
     if (live) {
-        const float4 *src = atlas + (size_t)p * 64 + 16 * h;
+        const float4 *src = atlas + (size_t)p * 64 + h;
 #pragma unroll
         for (int i0 = 0; i0 < 16; i0 += 8) {
             float4 L[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) L[i] = __ldg(src + i0 + i);
+            for (int i = 0; i < 8; ++i) L[i] = __ldg(src + 4 * (i0 + i));
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float4 *mc = reinterpret_cast<const float4 *>(s_mom + (4 * (i0 + i) + h) * kMomStride);
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(const float4 *atlas, c
 template <bool RPC1>
 __global__ void __launch_bounds__(kIntThreads, 4) k_integrate_surr(IntegrateArgs a) {
     __shared__ __align__(16) float s_mom[64 * kMomStride];
-    load_moment_table(s_mom);
+    load_moment_table<true>(s_mom);
     __syncthreads();
     integrate_body<true, RPC1>(a, blockIdx.x, s_mom);
 }
@@ -624,47 +624,62 @@ __device__ __forceinline__ float dot3_rn(float ax, float ay, float az, float bx,
     return __fadd_rn(__fadd_rn(__fmul_rn(ax, bx), __fmul_rn(ay, by)), __fmul_rn(az, bz));
 }
 
-// Algorithm 1: four 8x8 tiles per block (one thread per pixel, lane = 8 ly + lx).  A pixel whose
+// Algorithm 1: one warp per 8x8 tile, lane l the pixels l and l + 32 (pixel 8 ly + lx).  A pixel whose
 // previous position q falls on a previous probe that lies within cell_size of the pixel's plane
-// and faces within 0.95 of its normal bids (half(distance) << 16 | lane); the smallest bid places
-// the tile's probe on its pixel, carrying that previous probe.
-__global__ void __launch_bounds__(256) k_reproject(ReprojArgs a) {
-    __shared__ uint32_t s_score[4];
-    const uint32_t tl = threadIdx.x >> 6, lane = threadIdx.x & 63;
-    const uint32_t t = blockIdx.x * 4u + tl;
+// and faces within 0.95 of its normal bids (half(distance) << 16 | pixel); the smallest bid places
+// the tile's probe on its pixel, carrying that previous probe.  Three dependent trips (G-buffer and
+// motion, mask, probe) bound it, so each lane keeps two pixels' loads in flight and the warp's smallest
+// bid needs no shared memory.  (One thread per pixel, four trips, atomicMin in shared memory: 27.8 us at
+// 1080p, now 22.7 us; 50 MB, 7.4 us at the copy rate.)
+__global__ void __launch_bounds__(kGatherThreads) k_reproject(ReprojArgs a) {
+    const uint32_t lane = threadIdx.x & 31u, t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t tx = t % a.tiles_x, ty = t / a.tiles_x;
-    if (lane == 0) s_score[tl] = kScoreNone;
-    __syncthreads();
-    const uint32_t x = 8u * tx + (lane & 7u), y = 8u * ty + (lane >> 3);
-    uint32_t my = kScoreNone, tq = 0;
-    float3 w = make_float3(0.f, 0.f, 0.f);
-    float4 nd = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (ty < a.tiles_y && x < a.width && y < a.height) {
-        nd = __ldg(a.gbuf + (size_t)y * a.width + x);
-        if (isfinite(nd.w) && nd.w >= 0.0f) {
-            const float2 mv = __ldg(a.motion + (size_t)y * a.width + x);
-            const float fx = floorf(__fadd_rn(__fadd_rn((float)x, 0.5f), mv.x));
-            const float fy = floorf(__fadd_rn(__fadd_rn((float)y, 0.5f), mv.y));
+    if (ty >= a.tiles_y) return;
+    const uint32_t x = 8u * tx + (lane & 7u);
+    float4 nd[2];
+    float2 mv[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t y = 8u * ty + (lane >> 3) + 4u * h;
+        nd[h] = make_float4(0.f, 0.f, 0.f, -1.0f);
+        mv[h] = make_float2(0.f, 0.f);
+        if (x < a.width && y < a.height) {
+            nd[h] = __ldcs(a.gbuf + (size_t)y * a.width + x);
+            mv[h] = __ldcs(a.motion + (size_t)y * a.width + x);
+        }
+    }
+    uint32_t tq[2], pm[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t y = 8u * ty + (lane >> 3) + 4u * h;
+        tq[h] = 0u;
+        pm[h] = GI_PROBE_NONE;
+        if (isfinite(nd[h].w) && nd[h].w >= 0.0f) {
+            const float fx = floorf(__fadd_rn(__fadd_rn((float)x, 0.5f), mv[h].x));
+            const float fy = floorf(__fadd_rn(__fadd_rn((float)y, 0.5f), mv[h].y));
             if (fx >= 0.0f && fy >= 0.0f && fx < (float)a.width && fy < (float)a.height) {
-                tq = ((uint32_t)fy >> 3) * a.tiles_x + ((uint32_t)fx >> 3);
-                if (__ldg(a.prev_mask + tq) != GI_PROBE_NONE) {
-                    w = pixel_world_exact(a.cam, x, y, nd.w);
-                    const float4 pp = __ldg(a.prev_pos + tq), pn = __ldg(a.prev_nrm + tq);
-                    const float vx = __fsub_rn(pp.x, w.x), vy = __fsub_rn(pp.y, w.y), vz = __fsub_rn(pp.z, w.z);
-                    const float plane = fabsf(dot3_rn(vx, vy, vz, nd.x, nd.y, nd.z));
-                    const float ncheck = dot3_rn(pn.x, pn.y, pn.z, nd.x, nd.y, nd.z);
-                    if (plane < __fmul_rn(a.dscale, nd.w) && ncheck > 0.95f) {
-                        const float dist = __fsqrt_rn(dot3_rn(vx, vy, vz, vx, vy, vz));
-                        my = ((uint32_t)__half_as_ushort(__float2half_rn(dist)) << 16) | lane;
-                        atomicMin(&s_score[tl], my);
-                    }
-                }
+                tq[h] = ((uint32_t)fy >> 3) * a.tiles_x + ((uint32_t)fx >> 3);
+                pm[h] = __ldg(a.prev_mask + tq[h]);
             }
         }
     }
-    __syncthreads();
-    if (ty >= a.tiles_y) return;
-    const uint32_t best = s_score[tl];
+    uint32_t my[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        my[h] = kScoreNone;
+        if (pm[h] != GI_PROBE_NONE) {
+            const float4 pp = __ldg(a.prev_pos + tq[h]), pn = __ldg(a.prev_nrm + tq[h]);
+            const float3 w = pixel_world_exact(a.cam, x, 8u * ty + (lane >> 3) + 4u * h, nd[h].w);
+            const float vx = __fsub_rn(pp.x, w.x), vy = __fsub_rn(pp.y, w.y), vz = __fsub_rn(pp.z, w.z);
+            const float plane = fabsf(dot3_rn(vx, vy, vz, nd[h].x, nd[h].y, nd[h].z));
+            const float ncheck = dot3_rn(pn.x, pn.y, pn.z, nd[h].x, nd[h].y, nd[h].z);
+            if (plane < __fmul_rn(a.dscale, nd[h].w) && ncheck > 0.95f) {
+                const float dist = __fsqrt_rn(dot3_rn(vx, vy, vz, vx, vy, vz));
+                my[h] = min(kScoreNone, ((uint32_t)__half_as_ushort(__float2half_rn(dist)) << 16) | (lane + 32u * h));
+            }
+        }
+    }
+    const uint32_t best = __reduce_min_sync(kFullMask, min(my[0], my[1]));
     if (best == kScoreNone) {
         if (lane == 0) {
             a.mask[t] = GI_PROBE_NONE;
@@ -672,12 +687,18 @@ __global__ void __launch_bounds__(256) k_reproject(ReprojArgs a) {
             a.nrm[t] = make_float4(0.f, 0.f, 0.f, 0.f);
             a.src[t] = GI_PROBE_NONE;
         }
-    } else if (my == best) {
-        a.mask[t] = (y << 16) | x;
-        a.pos[t] = make_float4(w.x, w.y, w.z, nd.w);
-        a.nrm[t] = make_float4(nd.x, nd.y, nd.z, 1.0f);
-        a.src[t] = tq;
+        return;
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (my[h] == best) {
+            const uint32_t y = 8u * ty + (lane >> 3) + 4u * h;
+            const float3 w = pixel_world_exact(a.cam, x, y, nd[h].w);
+            a.mask[t] = (y << 16) | x;
+            a.pos[t] = make_float4(w.x, w.y, w.z, nd[h].w);
+            a.nrm[t] = make_float4(nd[h].x, nd[h].y, nd[h].z, 1.0f);
+            a.src[t] = tq[h];
+        }
 }
 
 // Algorithm 4 on one cell: alpha from the normalised luminance difference, squared after the clamp.
@@ -693,7 +714,7 @@ __device__ __forceinline__ float3 temporal_blend(float3 c, float3 p) {
 // One warp per 8x8 tile: a fresh probe gathers its spawn tile's rays (the cells' radiance and hit
 // distance, as k_gather) and blends each cell with the same cell of the tile's reprojected probe;
 // a reprojected-only probe copies its source's cells; a tile without probe gets zeros.
-__global__ void __launch_bounds__(256) k_gather_temporal(TemporalArgs a) {
+__global__ void __launch_bounds__(kGatherThreads) k_gather_temporal(TemporalArgs a) {
     const uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (t >= a.probes) return;
@@ -701,29 +722,35 @@ __global__ void __launch_bounds__(256) k_gather_temporal(TemporalArgs a) {
     const uint32_t st = 8u * a.upscale, sx = tx / a.upscale, sy = ty / a.upscale;
     const uint32_t px = min(st * sx + (uint32_t)a.jx, a.width - 1u);
     const uint32_t py = min(st * sy + (uint32_t)a.jy, a.height - 1u);
+    // the source, the spawn pixel's distance and the rays of a tile that may be fresh, together
+    const uint32_t src = __ldg(a.src + t), sp = sy * a.spawn_x + sx;
     bool fresh = false;
+    RayPair first = {GI_SLOT_NONE, GI_SLOT_NONE, 0.f, 0.f};
     if ((px >> 3) == tx && (py >> 3) == ty) {
+        first = load_rays(a.g, (size_t)sp * a.g.rpp + lane);
         const float d = __ldg(&a.gbuf[(size_t)py * a.width + px].w);
         fresh = isfinite(d) && d >= 0.0f;
     }
-    const uint32_t src = __ldg(a.src + t);
+    float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
+    if (src != GI_PROBE_NONE) {
+        p0 = __ldg(a.prev_atlas + (size_t)src * 64 + lane);
+        p1 = __ldg(a.prev_atlas + (size_t)src * 64 + lane + 32);
+    }
     float4 *dst = a.atlas + (size_t)t * 64;
     float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
     if (fresh) {
         float L[2][3], hd[2];
-        gather_cells<false, true>(a.g, sy * a.spawn_x + sx, lane, L, hd);
+        gather_cells(a.g, sp, lane, first, L, hd);
         float3 c0 = make_float3(L[0][0], L[0][1], L[0][2]), c1 = make_float3(L[1][0], L[1][1], L[1][2]);
         if (src != GI_PROBE_NONE) {
-            const float4 p0 = __ldg(a.prev_atlas + (size_t)src * 64 + lane);
-            const float4 p1 = __ldg(a.prev_atlas + (size_t)src * 64 + lane + 32);
             c0 = temporal_blend(c0, make_float3(p0.x, p0.y, p0.z));
             c1 = temporal_blend(c1, make_float3(p1.x, p1.y, p1.z));
         }
         o0 = make_float4(c0.x, c0.y, c0.z, hd[0]);
         o1 = make_float4(c1.x, c1.y, c1.z, hd[1]);
     } else if (src != GI_PROBE_NONE) {
-        o0 = __ldg(a.prev_atlas + (size_t)src * 64 + lane);
-        o1 = __ldg(a.prev_atlas + (size_t)src * 64 + lane + 32);
+        o0 = p0;
+        o1 = p1;
     }
     dst[lane] = o0;
     dst[lane + 32] = o1;
@@ -736,10 +763,8 @@ __global__ void __launch_bounds__(256) k_gather_temporal(TemporalArgs a) {
 // leaves the level.
 __device__ __forceinline__ uint32_t find_closest_probe(const uint32_t *mask, const MipInfo &mi, int tx, int ty, int ox,
                                                        int oy, int m0) {
-#pragma unroll
-    for (int m = 1; m < GI_MAX_MIPS; ++m) {
-        if (m < m0) continue;
-        if (m >= mi.count) break;
+#pragma unroll 1
+    for (int m = m0; m < mi.count; ++m) {
         const int x = tx + ox, y = ty + oy;
         if (x < 0 || y < 0 || x >= mi.w[m] || y >= mi.h[m]) break;
         const uint32_t p = __ldg(mask + mi.off[m] + y * mi.w[m] + x);
@@ -748,10 +773,6 @@ __device__ __forceinline__ uint32_t find_closest_probe(const uint32_t *mask, con
         ty >>= 1;
     }
     return GI_PROBE_NONE;
-}
-
-__device__ __forceinline__ uint32_t pick_u4(const uint32_t (&v)[4], int i) {
-    return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
 }
 
 // Per-warp copy of the four neighbours' data in shared memory: SH coefficients (27 + pad, seven
@@ -804,12 +825,12 @@ __device__ __forceinline__ void sh_lobe(float nx, float ny, float nz, float (&Yb
 
 // One pixel of the interpolation: weights of the four neighbours (bilinear x normal x plane
 // distance) and the weighted irradiance, or the relaxed / none / sky flags.  (fx, fy) is the
-// pixel's bilinear position between the neighbours.  UNIFORM: the neighbours' irradiance and
+// pixel's bilinear position between the neighbours, bit o of found says that neighbour o is there.  UNIFORM: the neighbours' irradiance and
 // plane and normal terms were evaluated once for the warp (s.eu, s.n8); otherwise each is
 // evaluated for this pixel's normal from the warp's shared copy.
 template <bool UNIFORM>
 __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb &s, int x, int y, float fx, float fy,
-                                             const float4 nd, size_t pix, bool inb, bool act, const uint32_t (&q)[4]) {
+                                             const float4 nd, uint32_t pix, bool inb, bool act, unsigned found) {
     if (!inb) return;
     if (!act) {
         __stcs(a.out + pix, make_float4(0.f, 0.f, 0.f, (float)GI_INTERP_SKY));
@@ -828,10 +849,9 @@ __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb
     float Yb[9];
     if (!UNIFORM) sh_lobe(nx, ny, nz, Yb);
     float wsum = 0.f, es[3] = {0.f, 0.f, 0.f};
-    int nfound = 0;
-#pragma unroll
+#pragma unroll(UNIFORM ? 4 : 1)
     for (int o = 0; o < 4; ++o) {
-        if (q[o] == GI_PROBE_NONE) continue;
+        if (!((found >> o) & 1u)) continue;
         float qn, n8, E[3];
         if (UNIFORM) {
             const float4 u = s.eu[o];
@@ -851,10 +871,9 @@ __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb
         wsum += w;
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) es[ch] += w * E[ch];
-        ++nfound;
     }
     float4 r;
-    if (nfound == 0) {
+    if (found == 0u) {
         r = make_float4(0.f, 0.f, 0.f, (float)GI_INTERP_NONE);
     } else if (wsum > 0.0f) {
         const float inv = 1.0f / wsum;
@@ -862,9 +881,9 @@ __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb
     } else {
         // relaxed: the plain mean of the neighbours found (rare: every weight vanished)
         float er[3] = {0.f, 0.f, 0.f};
-#pragma unroll
+#pragma unroll 1
         for (int o = 0; o < 4; ++o) {
-            if (q[o] == GI_PROBE_NONE) continue;
+            if (!((found >> o) & 1u)) continue;
             float E[3];
             if (UNIFORM) {
                 const float4 u = s.eu[o];
@@ -877,51 +896,61 @@ __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) er[ch] += E[ch];
         }
-        const float inv = 1.0f / (float)nfound;
+        const float inv = 1.0f / (float)__popc(found);
         r = make_float4(er[0] * inv, er[1] * inv, er[2] * inv, (float)GI_INTERP_RELAXED);
     }
     __stcs(a.out + pix, r);
 }
 
-constexpr int kInterpWarps = 8;  // 32 x 16 pixels per 256-thread block
+constexpr int kInterpWarps = 4 * kInterpRows;
+constexpr int kInterpBlocksPerSm = 40 / kInterpWarps;  // 48 registers
 
-// Block = 32x16 pixels starting at (32 bx - 4, 16 by - 4); warp = the 8x8 pixels that share one
+// Block = 32 x 8 kInterpRows pixels starting at (-4, -4); warp = the 8x8 pixels that share one
 // base tile floor((p - 4) / 8): lane l holds column l & 7 of rows l >> 3 and 4 + (l >> 3).  The
-// four neighbour probes are therefore the same for the whole warp: lanes 0..3 run Algorithm 3
-// for one neighbour each, and the warp copies the neighbours' data to shared memory once (28 lanes
-// one SH float4 each, 4 lanes a position and normal).  A warp whose active pixels share one normal
-// evaluates the neighbours' irradiance and plane terms once for its 64 pixels.
+// four neighbour probes are therefore the same for the whole warp, which loads their data (28 lanes one
+// SH float4 each, 4 lanes mask, distance and normal) in one round trip with the G-buffer and copies them
+// to shared memory once.  A warp whose active pixels share one normal evaluates the neighbours' irradiance
+// and plane terms once for its 64 pixels.  It is bound by issue and by the trips of the warps in flight:
+// 48 registers for 40 warps per SM (32 with the masks read before the rest: 29.7 us at 1080p, 423 us for
+// 16 views; now 25.8 and 301 us; 66 MB and 885 MB of pixels, 9.8 and 130 us at the copy rate).
 __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t bx, uint32_t by) {
     __shared__ InterpNb s_nb[kInterpWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     InterpNb &s = s_nb[warp];
     const int x = (int)bx * 32 - 4 + 8 * (warp & 3) + (lane & 7);
-    const int y0 = (int)by * 16 - 4 + 8 * (warp >> 2) + (lane >> 3);
+    const int y0 = (int)by * (8 * kInterpRows) - 4 + 8 * (warp >> 2) + (lane >> 3);
     const int tx = (x - 4) >> 3, ty = (y0 - 4) >> 3;  // the same for y0 and y0 + 4
     // the G-buffer of the lane's two pixels (independent of the probes)
     bool inb[2], act[2];
     float4 nd[2];
-    size_t pix[2];
+    uint32_t pix[2];  // an image has at most 65535^2 pixels
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int y = y0 + 4 * h;
         inb[h] = x >= 0 && y >= 0 && x < (int)a.width && y < (int)a.height;
-        pix[h] = inb[h] ? (size_t)y * a.width + x : 0;
+        pix[h] = inb[h] ? (uint32_t)y * a.width + (uint32_t)x : 0u;
         nd[h] = inb[h] ? __ldcs(a.gbuf + pix[h]) : make_float4(0.f, 0.f, 0.f, -1.0f);
     }
-    // neighbour `lane` (lanes 0..3): Algorithm 3 from the tile (tx + (lane & 1), ty + (lane >> 1)),
-    // continued above level 0 only where level 0 holds no probe
+    // Neighbour o = tile (tx + (o & 1), ty + (o >> 1)).  Its mask word and, as if it held a probe (whose
+    // index is then the tile's), its SH and position are loaded in one round trip: lanes 7 o + k one float4
+    // of SH each, lanes 28..31 the mask, distance and normal.  Only where level 0 names no probe of the
+    // tile does Algorithm 3 go on above it, and that neighbour's data are loaded again.
+    const int o = lane < 28 ? lane / 7 : lane - 28;
+    const int qx = tx + (o & 1), qy = ty + (o >> 1);
+    const bool tile = qx >= 0 && qy >= 0 && qx < a.mi.w[0] && qy < a.mi.h[0];
+    uint32_t pidx = tile ? (uint32_t)qy * a.tiles_x + (uint32_t)qx : 0u;
     uint32_t qo = GI_PROBE_NONE;
-    if (lane < 4) {
-        const int qx = tx + (lane & 1), qy = ty + (lane >> 1);
-        if (qx >= 0 && qy >= 0 && qx < a.mi.w[0] && qy < a.mi.h[0]) {
-            qo = __ldg(a.mask + qy * a.mi.w[0] + qx);
-            if (qo == GI_PROBE_NONE) qo = find_closest_probe(a.mask, a.mi, tx >> 1, ty >> 1, lane & 1, lane >> 1, 1);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    float tq = 0.f;
+    if (tile) {
+        if (lane < 28) {
+            v = __ldg(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
+        } else {
+            qo = __ldg(a.mask + pidx);
+            tq = __ldg(&a.ppos[pidx].w);
+            v = __ldg(a.pnrm + pidx);
         }
     }
-    uint32_t q[4];
-#pragma unroll
-    for (int o = 0; o < 4; ++o) q[o] = __shfl_sync(kFullMask, qo, o);
 #pragma unroll
     for (int h = 0; h < 2; ++h) act[h] = inb[h] && isfinite(nd[h].w) && nd[h].w >= 0.0f;
     const unsigned am0 = __ballot_sync(kFullMask, act[0]), am1 = __ballot_sync(kFullMask, act[1]);
@@ -931,28 +960,38 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
             if (inb[h]) __stcs(a.out + pix[h], make_float4(0.f, 0.f, 0.f, (float)GI_INTERP_SKY));
         return;
     }
-    // the neighbours' data into the warp's shared copy
-    {
-        const int o = lane < 28 ? lane / 7 : lane - 28;
-        const uint32_t qq = pick_u4(q, o);
-        if (qq != GI_PROBE_NONE) {
-            const uint32_t pidx = (qq >> 19) * a.tiles_x + ((qq & 0xFFFFu) >> 3);
+    const bool other = lane >= 28 && tile && (qo >> 19 != (uint32_t)qy || (qo & 0xFFFFu) >> 3 != (uint32_t)qx);
+    if (__any_sync(kFullMask, other)) {
+        uint32_t up = GI_PROBE_NONE;
+        if (other) {
+            if (qo == GI_PROBE_NONE) qo = find_closest_probe(a.mask, a.mi, tx >> 1, ty >> 1, o & 1, o >> 1, 1);
+            up = qo;
+        }
+        up = __shfl_sync(kFullMask, up, 28 + o);
+        if (up != GI_PROBE_NONE) {
+            pidx = (up >> 19) * a.tiles_x + ((up & 0xFFFFu) >> 3);
             if (lane < 28) {
-                const int k = lane - 7 * o;
-                s.c[o][k] = __ldg(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + k);
+                v = __ldg(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
             } else {
-                const float tq = __ldg(a.ppos + pidx).w;
-                const float qpx = (float)(qq & 0xFFFFu), qpy = (float)(qq >> 16);
-                const float sxq = (2.0f * (qpx + 0.5f) * a.cam.inv_w - 1.0f) * a.cam.sx_scale;
-                const float syq = (1.0f - 2.0f * (qpy + 0.5f) * a.cam.inv_h) * a.cam.sy_scale;
-                const float vx = a.cam.fwd[0] + sxq * a.cam.right[0] + syq * a.cam.up[0];
-                const float vy = a.cam.fwd[1] + sxq * a.cam.right[1] + syq * a.cam.up[1];
-                const float vz = a.cam.fwd[2] + sxq * a.cam.right[2] + syq * a.cam.up[2];
-                const float t = tq * rsqrtf(vx * vx + vy * vy + vz * vz);
-                s.pos[o] = make_float4(t * vx, t * vy, t * vz, 0.f);
-                s.nrm[o] = __ldg(a.pnrm + pidx);
+                tq = __ldg(&a.ppos[pidx].w);
+                v = __ldg(a.pnrm + pidx);
             }
         }
+    }
+    const unsigned found = __ballot_sync(kFullMask, qo != GI_PROBE_NONE) >> 28;  // lanes below 28 hold none
+    // the neighbours' data into the warp's shared copy
+    if (lane < 28) {
+        s.c[o][lane - 7 * o] = v;
+    } else {
+        const float qpx = (float)(qo & 0xFFFFu), qpy = (float)(qo >> 16);
+        const float sxq = (2.0f * (qpx + 0.5f) * a.cam.inv_w - 1.0f) * a.cam.sx_scale;
+        const float syq = (1.0f - 2.0f * (qpy + 0.5f) * a.cam.inv_h) * a.cam.sy_scale;
+        const float vx = a.cam.fwd[0] + sxq * a.cam.right[0] + syq * a.cam.up[0];
+        const float vy = a.cam.fwd[1] + sxq * a.cam.right[1] + syq * a.cam.up[1];
+        const float vz = a.cam.fwd[2] + sxq * a.cam.right[2] + syq * a.cam.up[2];
+        const float t = tq * rsqrtf(vx * vx + vy * vy + vz * vz);
+        s.pos[o] = make_float4(t * vx, t * vy, t * vz, 0.f);
+        s.nrm[o] = v;
     }
     __syncwarp();
     // the first active pixel's normal stands in for inactive pixels (they only help the warp)
@@ -974,7 +1013,7 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
         if (lane < 12) {
             const int o = lane / 3, ch = lane - 3 * (lane / 3);
             float e = 0.f;
-            if (pick_u4(q, o) != GI_PROBE_NONE) {
+            if ((found >> o) & 1u) {
                 float Yb[9];
                 sh_lobe(sx_, sy_, sz_, Yb);
                 const float *c = reinterpret_cast<const float *>(s.c[o]) + ch;
@@ -985,7 +1024,7 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
         } else if (lane < 16) {
             const int o = lane - 12;
             float qn_u = 0.f, n8_u = 0.f;
-            if (pick_u4(q, o) != GI_PROBE_NONE) nb_terms(s, o, sx_, sy_, sz_, qn_u, n8_u);
+            if ((found >> o) & 1u) nb_terms(s, o, sx_, sy_, sz_, qn_u, n8_u);
             reinterpret_cast<float *>(s.eu)[4 * o + 3] = qn_u;
             reinterpret_cast<float *>(&s.n8)[o] = n8_u;
         }
@@ -993,16 +1032,22 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
 #pragma unroll
         for (int h = 0; h < 2; ++h)
             interp_pixel<true>(a, s, x, y0 + 4 * h, fx, ((float)((lane >> 3) + 4 * h) + 0.5f) * 0.125f,
-                               h ? nd[1] : nd[0], h ? pix[1] : pix[0], h ? inb[1] : inb[0], h ? act[1] : act[0], q);
+                               h ? nd[1] : nd[0], h ? pix[1] : pix[0], h ? inb[1] : inb[0], h ? act[1] : act[0], found);
     } else {
+        // (the G-buffer is read again: its two values held through this path would spill)
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h)
-            interp_pixel<false>(a, s, x, y0 + 4 * h, fx, ((float)((lane >> 3) + 4 * h) + 0.5f) * 0.125f,
-                                h ? nd[1] : nd[0], h ? pix[1] : pix[0], h ? inb[1] : inb[0], h ? act[1] : act[0], q);
+        for (int h = 0; h < 2; ++h) {
+            const int y = y0 + 4 * h;
+            if (x < 0 || y < 0 || x >= (int)a.width || y >= (int)a.height) continue;
+            const uint32_t px = (uint32_t)y * a.width + (uint32_t)x;
+            const float4 g = __ldg(a.gbuf + px);
+            interp_pixel<false>(a, s, x, y, fx, ((float)((lane >> 3) + 4 * h) + 0.5f) * 0.125f, g, px, true,
+                                isfinite(g.w) && g.w >= 0.0f, found);
+        }
     }
 }
 
-__global__ void __launch_bounds__(256, 4) k_interpolate(InterpArgs a) { interpolate_body(a, blockIdx.x, blockIdx.y); }
+__global__ void __launch_bounds__(32 * kInterpWarps, kInterpBlocksPerSm) k_interpolate(InterpArgs a) { interpolate_body(a, blockIdx.x, blockIdx.y); }
 
 static bool layout_matches(const gi_probe_layout &l, uint32_t w, uint32_t h) {
     return l.tiles_x == (w + 7) / 8 && l.tiles_y == (h + 7) / 8 && l.num_probes == l.tiles_x * l.tiles_y &&
@@ -1133,103 +1178,115 @@ struct FilterArgs {
     int axis;            // 0: steps along x, 1: along y
 };
 
-// Algorithm 3 from level 0: the probe at (tx + ox, ty + oy), else up the MIP chain.
-__device__ __forceinline__ uint32_t find_probe_from_level0(const uint32_t *mask, const MipInfo &mi, int tx, int ty,
-                                                            int ox, int oy) {
-    const int x = tx + ox, y = ty + oy;
-    if (x < 0 || y < 0 || x >= mi.w[0] || y >= mi.h[0]) return GI_PROBE_NONE;
-    const uint32_t q = __ldg(mask + y * mi.w[0] + x);
-    if (q != GI_PROBE_NONE) return q;
-    return find_closest_probe(mask, mi, tx >> 1, ty >> 1, ox, oy, 1);
-}
-
-// One thread per (probe, cell), 4 probes per block (2 warps per probe): the cell's radiance and hit
+// One warp per probe, lane l on the cells l and l + 32 one after the other: the cell's radiance and hit
 // distance blurred with the same cell of the probes found at steps -1, +1, -2, +2, -3, +3 along the
 // axis, each accepted when it lies within cell_size of the probe's plane, the cell direction is not
 // behind its normal, and the hit point seen from it (at the smaller hit distance) is within pi/50 of
 // the cell direction seen from the probe; depth weight 1 / (1 + |d_p - d_q| / cell_size(d_p)).
 // What is the same for all 64 cells of a probe -- the neighbour search, its offset from the probe,
-// the plane test and the depth weight -- lanes 0..5 of each warp compute once into shared memory;
-// every thread then issues its six neighbour loads together and takes the per-cell decisions in
-// step order (the running hit distance of one step enters the next).  The angle test avoids the
+// the plane test and the depth weight -- lanes 0..5 compute once into shared memory; every thread
+// then issues its six neighbour loads together and takes the per-cell decisions in
+// step order (the running hit distance of one step enters the next).  Almost every search ends at level
+// 0, at the probe of the tile the step leads to: its mask word, position and normal are loaded at once as if
+// it did, and again only where the search found another probe.  The angle test avoids the
 // square root: cos(angle) >= c  <=>  d.h > 0 and (d.h)^2 >= c^2 |h|^2.
-constexpr int kFiltProbes = 4;
-__global__ void __launch_bounds__(64 * kFiltProbes) k_filter(FilterArgs a) {
-    __shared__ uint32_t s_qi[2 * kFiltProbes][6];
-    __shared__ float4 s_rel[2 * kFiltProbes][6];  // q - p (xyz), depth weight
-    __shared__ float4 s_nq[2 * kFiltProbes][6];
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const uint32_t p = blockIdx.x * kFiltProbes + (t >> 6);
-    const uint32_t c = t & 63;
-    if (p >= a.probes) return;  // both warps of a probe leave together
-    const size_t self = (size_t)p * 64 + c;
-    const float4 v = __ldg(a.in + self);
+// What bounds it is issue and the chain search -> neighbours -> cells of too few warps.  Two warps per probe,
+// each searching for its own 32 cells, loads following one another (48 registers, 40 warps per SM): 40 us a
+// pass at 1080p; this form 30 us (64 registers, 8 blocks of 4 warps; 72 registers 3 us more, 48 spill).  One
+// warp searching for the block's four probes before a barrier: 41 us, the barrier waits for it.
+constexpr int kFiltWarps = 4, kFiltBlocksPerSm = 8;
+__global__ void __launch_bounds__(32 * kFiltWarps, kFiltBlocksPerSm) k_filter(FilterArgs a) {
+    __shared__ uint32_t s_qi[kFiltWarps][6];
+    __shared__ float4 s_rel[kFiltWarps][6];  // q - p (xyz), depth weight
+    __shared__ float4 s_nq[kFiltWarps][6];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t p = blockIdx.x * kFiltWarps + warp;
+    if (p >= a.probes) return;
+    const float4 *in = a.in + (size_t)p * 64 + lane;
+    float4 *out = a.out + (size_t)p * 64 + lane;
     const float4 n4 = __ldg(a.pnrm + p);
-    if (n4.w == 0.0f) {
-        a.out[self] = v;
-        return;
-    }
-    const float4 pp = __ldg(a.ppos + p);
-    const float cs = a.dscale * pp.w;
-    const float nx = n4.x, ny = n4.y, nz = n4.z;
+    const float4 va = __ldg(in), vb = __ldg(in + 32);
     if (lane < 6) {
         const int step = (((lane & 1) << 1) - 1) * ((lane >> 1) + 1);
-        const int tx = (int)(p % a.tiles_x), ty = (int)(p / a.tiles_x);
-        const uint32_t q = find_probe_from_level0(a.mask, a.mi, tx, ty, a.axis == 0 ? step : 0, a.axis == 0 ? 0 : step);
+        const int ox = a.axis == 0 ? step : 0, oy = a.axis == 0 ? 0 : step;
+        const int tx = (int)(p % a.tiles_x), ty = (int)(p / a.tiles_x), qx = tx + ox, qy = ty + oy;
         uint32_t qi = GI_PROBE_NONE;
-        if (q != GI_PROBE_NONE) {
-            const uint32_t k = ((q >> 16) >> 3) * a.tiles_x + ((q & 0xFFFFu) >> 3);
-            const float4 pq = __ldg(a.ppos + k);
-            const float rx = pq.x - pp.x, ry = pq.y - pp.y, rz = pq.z - pp.z;
-            if (fabsf(rx * nx + ry * ny + rz * nz) <= cs) {  // the plane test
-                qi = k;
-                s_rel[warp][lane] = make_float4(rx, ry, rz, __fdividef(cs, cs + fabsf(pp.w - pq.w)));
-                s_nq[warp][lane] = __ldg(a.pnrm + k);
+        if (qx >= 0 && qy >= 0 && qx < a.mi.w[0] && qy < a.mi.h[0]) {
+            uint32_t k = (uint32_t)qy * a.tiles_x + (uint32_t)qx;
+            uint32_t q = __ldg(a.mask + k);
+            const float4 pp = __ldg(a.ppos + p);
+            float4 pq = __ldg(a.ppos + k), nq = __ldg(a.pnrm + k);
+            if (q == GI_PROBE_NONE) q = find_closest_probe(a.mask, a.mi, tx >> 1, ty >> 1, ox, oy, 1);
+            if (q != GI_PROBE_NONE) {
+                const uint32_t found = ((q >> 16) >> 3) * a.tiles_x + ((q & 0xFFFFu) >> 3);
+                if (found != k) {
+                    k = found;
+                    pq = __ldg(a.ppos + k);
+                    nq = __ldg(a.pnrm + k);
+                }
+                const float cs = a.dscale * pp.w;
+                const float rx = pq.x - pp.x, ry = pq.y - pp.y, rz = pq.z - pp.z;
+                if (fabsf(rx * n4.x + ry * n4.y + rz * n4.z) <= cs) {  // the plane test
+                    qi = k;
+                    s_rel[warp][lane] = make_float4(rx, ry, rz, __fdividef(cs, cs + fabsf(pp.w - pq.w)));
+                    s_nq[warp][lane] = nq;
+                }
             }
         }
         s_qi[warp][lane] = qi;
     }
+    if (n4.w == 0.0f) {
+        out[0] = va;
+        out[32] = vb;
+        return;
+    }
     __syncwarp();
-    float4 vq[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const uint32_t qi = s_qi[warp][i];
-        vq[i] = qi != GI_PROBE_NONE ? __ldg(a.in + (size_t)qi * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    // world direction of the cell centre in the probe frame (Duff et al. 2017)
-    const float sgn = copysignf(1.0f, nz);
-    const float ia = -1.0f / (sgn + nz);
-    const float bb = nx * ny * ia;
-    const float t0 = 1.0f + sgn * nx * nx * ia, t1 = sgn * bb, t2 = -sgn * nx;
-    const float b0 = bb, b1 = sgn + ny * ny * ia, b2 = -ny;
-    const float lx = __ldg(&g_cell_dir[c][0]), ly = __ldg(&g_cell_dir[c][1]), lz = __ldg(&g_cell_dir[c][2]);
-    const float dx = lx * t0 + ly * b0 + lz * nx, dy = lx * t1 + ly * b1 + lz * ny, dz = lx * t2 + ly * b2 + lz * nz;
+    const float nx = n4.x, ny = n4.y, nz = n4.z;
     const float cos2 = c_filter_cos * c_filter_cos;
-    float r = v.x, gch = v.y, bch = v.z, acc_a = v.w, weight = 1.0f, hd = v.w;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t c = (uint32_t)lane + 32u * h;
+        const float4 v = h ? vb : va;
+        float4 vq[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        if (s_qi[warp][i] == GI_PROBE_NONE) continue;
-        const float4 nq = s_nq[warp][i];
-        if (dx * nq.x + dy * nq.y + dz * nq.z < 0.0f) continue;  // the cell points behind q
-        const float4 rel = s_rel[warp][i];
-        const float hdc = fminf(vq[i].w, hd);
-        if (isfinite(hdc)) {
-            const float hx = rel.x + dx * hdc, hy = rel.y + dy * hdc, hz = rel.z + dz * hdc;
-            const float hh = hx * hx + hy * hy + hz * hz;
-            const float dh = dx * hx + dy * hy + dz * hz;
-            // a zero vector counts as on the cell direction
-            if (hh > 0.0f && (dh <= 0.0f || dh * dh < cos2 * hh)) continue;
+        for (int i = 0; i < 6; ++i) {
+            const uint32_t qi = s_qi[warp][i];
+            vq[i] = qi != GI_PROBE_NONE ? __ldg(a.in + (size_t)qi * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        const float w = rel.w;
-        r += w * vq[i].x;
-        gch += w * vq[i].y;
-        bch += w * vq[i].z;
-        acc_a += w * hdc;
-        weight += w;
-        hd = __fdividef(acc_a, weight);
+        // world direction of the cell centre in the probe frame (Duff et al. 2017)
+        const float sgn = copysignf(1.0f, nz);
+        const float ia = -1.0f / (sgn + nz);
+        const float bb = nx * ny * ia;
+        const float t0 = 1.0f + sgn * nx * nx * ia, t1 = sgn * bb, t2 = -sgn * nx;
+        const float b0 = bb, b1 = sgn + ny * ny * ia, b2 = -ny;
+        const float lx = __ldg(&g_cell_dir[c][0]), ly = __ldg(&g_cell_dir[c][1]), lz = __ldg(&g_cell_dir[c][2]);
+        const float dx = lx * t0 + ly * b0 + lz * nx, dy = lx * t1 + ly * b1 + lz * ny, dz = lx * t2 + ly * b2 + lz * nz;
+        float r = v.x, gch = v.y, bch = v.z, acc_a = v.w, weight = 1.0f, hd = v.w;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            if (s_qi[warp][i] == GI_PROBE_NONE) continue;
+            const float4 nq = s_nq[warp][i];
+            if (dx * nq.x + dy * nq.y + dz * nq.z < 0.0f) continue;  // the cell points behind q
+            const float4 rel = s_rel[warp][i];
+            const float hdc = fminf(vq[i].w, hd);
+            if (isfinite(hdc)) {
+                const float hx = rel.x + dx * hdc, hy = rel.y + dy * hdc, hz = rel.z + dz * hdc;
+                const float hh = hx * hx + hy * hy + hz * hz;
+                const float dh = dx * hx + dy * hy + dz * hz;
+                // a zero vector counts as on the cell direction
+                if (hh > 0.0f && (dh <= 0.0f || dh * dh < cos2 * hh)) continue;
+            }
+            const float w = rel.w;
+            r += w * vq[i].x;
+            gch += w * vq[i].y;
+            bch += w * vq[i].z;
+            acc_a += w * hdc;
+            weight += w;
+            hd = __fdividef(acc_a, weight);
+        }
+        const float inv = __fdividef(1.0f, weight);
+        out[32 * h] = make_float4(r * inv, gch * inv, bch * inv, acc_a * inv);
     }
-    const float inv = __fdividef(1.0f, weight);
-    a.out[self] = make_float4(r * inv, gch * inv, bch * inv, acc_a * inv);
 }
 
 // ---------------------------------------------------------------- batched passes (many views)
@@ -1254,11 +1311,11 @@ __global__ void __launch_bounds__(128, 4) k_integrate_batched(const IntegrateArg
                                                            uint32_t nviews) {
     __shared__ IntegrateArgs sa;
     __shared__ __align__(16) float s_mom[64 * kMomStride];
-    load_moment_table(s_mom);
+    load_moment_table<true>(s_mom);
     GI_BATCHED_ITEMS(prefix, nviews, sa, args, (integrate_body<false, RPC1>(sa, item, s_mom)));
 }
 
-__global__ void __launch_bounds__(256, 4) k_interpolate_batched(const InterpArgs *args, const uint32_t *prefix,
+__global__ void __launch_bounds__(32 * kInterpWarps, kInterpBlocksPerSm) k_interpolate_batched(const InterpArgs *args, const uint32_t *prefix,
                                                                 uint32_t nviews) {
     __shared__ InterpArgs sa;
     GI_BATCHED_ITEMS(prefix, nviews, sa, args, {
@@ -1292,7 +1349,7 @@ gi_status launch_integrate_batched(const IntegrateArgs *args, const uint32_t *pr
 gi_status launch_interpolate_batched(const InterpArgs *args, const uint32_t *prefix, uint32_t nviews,
                                      uint32_t blocks, cudaStream_t st) {
     if (blocks == 0) return GI_OK;
-    k_interpolate_batched<<<resident_grid(k_interpolate_batched, 256, blocks), 256, 0, st>>>(args, prefix, nviews);
+    k_interpolate_batched<<<resident_grid(k_interpolate_batched, 32 * kInterpWarps, blocks), 32 * kInterpWarps, 0, st>>>(args, prefix, nviews);
     return cuda_status(cudaGetLastError(), "k_interpolate_batched launch");
 }
 
@@ -1404,7 +1461,7 @@ gi_status gi_probes_reproject(const gi_gbuffer *gbuf, const gi_view *view, const
     a.nrm = reinterpret_cast<float4 *>(cur->nrm);
     a.src = src;
     const uint32_t P = cur->layout.num_probes;
-    k_reproject<<<(P + 3) / 4, 256, 0, (cudaStream_t)stream>>>(a);
+    k_reproject<<<(P + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0, (cudaStream_t)stream>>>(a);
     return cuda_status(cudaGetLastError(), "k_reproject launch");
 }
 
@@ -1438,9 +1495,9 @@ gi_status gi_probes_gather_temporal(gi_cache_t cache, const gi_gbuffer *gbuf, co
     a.src = src;
     a.prev_atlas = reinterpret_cast<const float4 *>(prev_atlas);
     a.atlas = reinterpret_cast<float4 *>(atlas);
-    const uint32_t blocks = (a.probes + 7) / 8;
+    const uint32_t blocks = (a.probes + kGatherThreads / 32 - 1) / (kGatherThreads / 32);
     if (blocks == 0) return GI_OK;
-    k_gather_temporal<<<blocks, 256, 0, (cudaStream_t)stream>>>(a);
+    k_gather_temporal<<<blocks, kGatherThreads, 0, (cudaStream_t)stream>>>(a);
     return cuda_status(cudaGetLastError(), "k_gather_temporal launch");
 }
 
@@ -1494,7 +1551,7 @@ gi_status gi_probes_gather(gi_cache_t cache, const gi_probes *pr, const uint32_t
     IntegrateArgs a = integrate_args(cache, pr, slot_ids, rays_per_probe, env);
     if (a.probes == 0) return GI_OK;
     a.ray_len = ray_len;
-    k_gather<<<(a.probes + 7) / 8, 256, 0, (cudaStream_t)stream>>>(a, reinterpret_cast<float4 *>(atlas));
+    k_gather<<<(a.probes + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0, (cudaStream_t)stream>>>(a, reinterpret_cast<float4 *>(atlas));
     return cuda_status(cudaGetLastError(), "k_gather launch");
 }
 
@@ -1523,7 +1580,7 @@ gi_status gi_probes_filter(const gi_probes *pr, const gi_view *view, const float
     a.dscale = (float)distance_scale(view->fov_y, view->width, view->height);
     a.axis = (int)axis;
     if (a.probes == 0) return GI_OK;
-    k_filter<<<(a.probes + kFiltProbes - 1) / kFiltProbes, 64 * kFiltProbes, 0, (cudaStream_t)stream>>>(a);
+    k_filter<<<(a.probes + kFiltWarps - 1) / kFiltWarps, 32 * kFiltWarps, 0, (cudaStream_t)stream>>>(a);
     return cuda_status(cudaGetLastError(), "k_filter launch");
 }
 
@@ -1547,7 +1604,7 @@ gi_status gi_probes_interpolate(const gi_gbuffer *gbuf, const gi_view *view, con
     if (s != GI_OK) return s;
     const InterpArgs a = interp_args(gbuf, view, pr, out);
     dim3 grid(interp_grid_x(view->width), interp_grid_y(view->height));
-    k_interpolate<<<grid, 256, 0, (cudaStream_t)stream>>>(a);
+    k_interpolate<<<grid, 32 * kInterpWarps, 0, (cudaStream_t)stream>>>(a);
     return cuda_status(cudaGetLastError(), "k_interpolate launch");
 }
 
