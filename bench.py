@@ -73,11 +73,11 @@ UPDATE_HEADER = ("gi_internal.cuh", "namespace gi {", "struct ResolveArgs {")
 NRC_ADAM_SECTION = ("gi_nrc.cu", "// ---------------------------------------------------------------- gradient scatter and Adam",
                     "// ---------------------------------------------------------------- query selection")
 NCU_TRAFFIC = {
-    # k_update, boxes-1080p (5th launch): 158.84 MB read + 33.20 MB written
-    "2:update": {"bytes_per_launch": 192040192, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
-                 "source_sha": "4125733ab0d02a56"},
-    # k_nrc_adam (table and weights), Cornell 1080p: 105.82 MB read + 14.31 MB written
-    "4:adam_table": {"bytes_per_launch": 120128000, "sources": (NRC_ADAM_SECTION,), "source_sha": "982b3204c28cfbcd"},
+    # k_update, boxes-1080p (5th launch): 158.97 MB read + 33.27 MB written
+    "2:update": {"bytes_per_launch": 192241152, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
+                 "source_sha": "0d84d9e0fa0f439e"},
+    # k_nrc_adam (table and weights), Cornell 1080p: 105.84 MB read + 14.32 MB written
+    "4:adam_table": {"bytes_per_launch": 120159744, "sources": (NRC_ADAM_SECTION,), "source_sha": "04fc4aad2b956f33"},
 }
 
 

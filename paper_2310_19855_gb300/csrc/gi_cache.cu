@@ -118,7 +118,7 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
     // far hits go to the surrogate while it is trusted (the decision of the whole launch)
     uint32_t route_lod = 4u;
     if (a.route_stats) {
-        const float den = __ldg(a.route_stats + 2), err = __ldg(a.route_stats + 1);
+        const float den = ld(a.route_stats + 2), err = ld(a.route_stats + 1);
         if (den > 0.0f && err <= a.route_trust * den) route_lod = a.route_lod;
     }
     for (unsigned long long base = (unsigned long long)blk * kUpdThreads; base < a.n; base += stride) {
@@ -243,27 +243,29 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
 
 template <int KEY_DIR, bool MERGE>
 __global__ void __launch_bounds__(kUpdThreads, MERGE ? 6 : 8) k_update(UpdateArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
-    update_body<KEY_DIR, MERGE, true>(a, blockIdx.x, gridDim.x, s_acc, nullptr);
+    update_body<KEY_DIR, MERGE, true>(a, bid, gridDim.x, s_acc, nullptr);
 }
 
 // touch-list form: 6 blocks per SM (the returning count's path needs more than 32 registers)
 template <int KEY_DIR, bool MERGE>
 __global__ void __launch_bounds__(kUpdThreads, 6) k_update_list(UpdateArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
     __shared__ uint32_t s_touch[kUpdBlockRecords];
-    update_body<KEY_DIR, MERGE, false>(a, blockIdx.x, gridDim.x, s_acc, s_touch);
+    update_body<KEY_DIR, MERGE, false>(a, bid, gridDim.x, s_acc, s_touch);
 }
 
 // the instantiations of k_update and k_update_list on one stream
 template <int KEY_DIR>
 static inline void launch_update_dir(const UpdateArgs &a, bool merge, int blocks, cudaStream_t st) {
     if (a.bitmap || a.rank) {
-        if (merge) k_update<KEY_DIR, true><<<blocks, kUpdThreads, 0, st>>>(a);
-        else k_update<KEY_DIR, false><<<blocks, kUpdThreads, 0, st>>>(a);
+        if (merge) launch(k_update<KEY_DIR, true>, blocks, kUpdThreads, 0, st, a);
+        else launch(k_update<KEY_DIR, false>, blocks, kUpdThreads, 0, st, a);
     } else {
-        if (merge) k_update_list<KEY_DIR, true><<<blocks, kUpdThreads, 0, st>>>(a);
-        else k_update_list<KEY_DIR, false><<<blocks, kUpdThreads, 0, st>>>(a);
+        if (merge) launch(k_update_list<KEY_DIR, true>, blocks, kUpdThreads, 0, st, a);
+        else launch(k_update_list<KEY_DIR, false>, blocks, kUpdThreads, 0, st, a);
     }
 }
 static inline void launch_update(const UpdateArgs &a, uint32_t key_dir, bool merge, int blocks, cudaStream_t st) {
@@ -329,7 +331,7 @@ __device__ __forceinline__ bool resolve_cell(const ResolveArgs &a, uint32_t s, u
 // the loads and its stamp set to frame + 1
 template <int U>
 __device__ __forceinline__ void resolve_list_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
-    const uint32_t n = __ldcg(&a.ctr->touch_count);
+    const uint32_t n = ld(&a.ctr->touch_count);
     const uint32_t stride = nblk * kResThreads;
     uint32_t fresh_new = 0;
     // accumulators leave the L2 first, resolved values last: the probe pass reads them next
@@ -489,20 +491,24 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs &a, uint32_t blk,
 }
 
 __global__ void __launch_bounds__(kResThreads, kResListBlocksPerSm) k_resolve(ResolveArgs a) {
-    resolve_list_body<kResListUnroll>(a, blockIdx.x, gridDim.x);
+    const uint32_t bid = blockIdx.x + pass_begin();
+    resolve_list_body<kResListUnroll>(a, bid, gridDim.x);
 }
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_bitmap(ResolveArgs a) {
-    resolve_bm_body<kResBmUnroll, false>(a, blockIdx.x, gridDim.x);
+    const uint32_t bid = blockIdx.x + pass_begin();
+    resolve_bm_body<kResBmUnroll, false>(a, bid, gridDim.x);
 }
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_dense(ResolveArgs a) {
-    resolve_bm_body<kResBmUnroll, true>(a, blockIdx.x, gridDim.x);
+    const uint32_t bid = blockIdx.x + pass_begin();
+    resolve_bm_body<kResBmUnroll, true>(a, bid, gridDim.x);
 }
 
 // ---------------------------------------------------------------- queries
 
 __global__ void k_query_slots(const uint32_t *slot_ids, unsigned long long n, const void *resolved, uint32_t res_stride, int f16,
                               uint32_t slots, float e0, float e1, float e2, float4 *out) {
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
+    const uint32_t bid = blockIdx.x + pass_begin();
+    for (unsigned long long i = bid * (unsigned long long)blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         const uint32_t s = __ldcs(slot_ids + i);
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -519,7 +525,8 @@ __global__ void k_query_slots(const uint32_t *slot_ids, unsigned long long n, co
 template <int KEY_DIR>
 __global__ void k_query_points(UpdateArgs a, const void *resolved, uint32_t res_stride, int f16, LiveRule rule,
                                float4 *out) {
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < a.n;
+    const uint32_t bid = blockIdx.x + pass_begin();
+    for (unsigned long long i = bid * (unsigned long long)blockDim.x + threadIdx.x; i < a.n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         const float len = a.len[i];
         const float px = a.p[0][i], py = a.p[1][i], pz = a.p[2][i];
@@ -534,10 +541,10 @@ __global__ void k_query_points(UpdateArgs a, const void *resolved, uint32_t res_
             cell_of_key(key, a.mask, home, tag);
             uint32_t s = home;
             for (uint32_t k = 0; k < a.max_probe; ++k) {
-                const uint32_t t = word_tag(__ldg(a.tags + s));
+                const uint32_t t = word_tag(__ldca(a.tags + s));
                 if (t == kEmpty) break;
                 if (t == tag) {
-                    if (answers(__ldg(a.stamps + (size_t)s * a.stamp_stride), rule)) {
+                    if (answers(__ldca(a.stamps + (size_t)s * a.stamp_stride), rule)) {
                         float3 v = load_resolved(resolved, res_stride, f16, s);
                         o = make_float4(v.x, v.y, v.z, 1.0f);
                     }
@@ -665,11 +672,11 @@ gi_status launch_resolve_batched(const ResolveArgs *args, const uint32_t *prefix
                                  bool dense, cudaStream_t st) {
     if (blocks == 0) return GI_OK;
     if (dense)
-        k_resolve_batched<true><<<resident_grid(k_resolve_batched<true>, kResThreads, blocks), kResThreads, 0, st>>>(
-            args, prefix, nviews);
+        k_resolve_batched<true>
+            <<<resident_grid(k_resolve_batched<true>, kResThreads, blocks), kResThreads, 0, st>>>(args, prefix, nviews);
     else
-        k_resolve_batched<false><<<resident_grid(k_resolve_batched<false>, kResThreads, blocks), kResThreads, 0, st>>>(
-            args, prefix, nviews);
+        k_resolve_batched<false>
+            <<<resident_grid(k_resolve_batched<false>, kResThreads, blocks), kResThreads, 0, st>>>(args, prefix, nviews);
     return cuda_status(cudaGetLastError(), "k_resolve_batched launch");
 }
 
@@ -1187,11 +1194,11 @@ gi_status gi_cache_resolve(gi_cache_t c, uint32_t frame, gi_stream_t stream) {
     } else {
         const ResolveArgs a = cache_resolve_args(c, frame);
         if (a.rank)
-            k_resolve_dense<<<c->res_blocks, kResThreads, 0, st>>>(a);
+            launch(k_resolve_dense, c->res_blocks, kResThreads, 0, st, a);
         else if (a.bitmap)
-            k_resolve_bitmap<<<c->res_blocks, kResThreads, 0, st>>>(a);
+            launch(k_resolve_bitmap, c->res_blocks, kResThreads, 0, st, a);
         else
-            k_resolve<<<c->res_blocks, kResThreads, 0, st>>>(a);
+            launch(k_resolve, c->res_blocks, kResThreads, 0, st, a);
         s = cuda_status(cudaGetLastError(), "k_resolve launch");
     }
     if (s != GI_OK) return s;
@@ -1213,8 +1220,8 @@ gi_status gi_cache_query(gi_cache_t c, const gi_query *q, float *out, gi_stream_
     const int f16 = c->cfg.resolved_format == GI_RESOLVED_F16;
     int blocks = (int)std::min<unsigned long long>((unsigned long long)c->sms * 16, (q->n + 255) / 256);
     if (q->slot_ids) {
-        k_query_slots<<<blocks, 256, 0, st>>>(q->slot_ids, q->n, c->resolved[c->cur], c->res_bytes, f16, c->cells, q->env[0],
-                                              q->env[1], q->env[2], reinterpret_cast<float4 *>(out));
+        launch(k_query_slots, blocks, 256, 0, st, q->slot_ids, q->n, c->resolved[c->cur], c->res_bytes, f16,
+               c->cells, q->env[0], q->env[1], q->env[2], reinterpret_cast<float4 *>(out));
     } else {
         if (!q->points || !hits_ok(q->points, c->cfg.key_dir) || q->points->n < q->n || !view_ok(q->view)) {
             set_error("gi_cache_query: by point needs points with n records and a valid view");
@@ -1232,11 +1239,11 @@ gi_status gi_cache_query(gi_cache_t c, const gi_query *q, float *out, gi_stream_
                                             reinterpret_cast<float4 *>(out), blocks, (int)c->cfg.key_dir, st);
         }
         if (c->cfg.key_dir == GI_KEY_DIR_NORMAL)
-            k_query_points<GI_KEY_DIR_NORMAL><<<blocks, 256, 0, st>>>(a, c->resolved[c->cur], c->res_bytes, f16, live_rule(c),
-                                                                      reinterpret_cast<float4 *>(out));
+            launch(k_query_points<GI_KEY_DIR_NORMAL>, blocks, 256, 0, st, a, c->resolved[c->cur], c->res_bytes, f16,
+                   live_rule(c), reinterpret_cast<float4 *>(out));
         else
-            k_query_points<GI_KEY_DIR_RAY><<<blocks, 256, 0, st>>>(a, c->resolved[c->cur], c->res_bytes, f16, live_rule(c),
-                                                                   reinterpret_cast<float4 *>(out));
+            launch(k_query_points<GI_KEY_DIR_RAY>, blocks, 256, 0, st, a, c->resolved[c->cur], c->res_bytes, f16,
+                   live_rule(c), reinterpret_cast<float4 *>(out));
     }
     return cuda_status(cudaGetLastError(), "k_query launch");
 }

@@ -349,6 +349,52 @@ InterpArgs interp_args(const gi_gbuffer *gbuf, const gi_view *view, const gi_pro
 
 } // namespace gi
 
+// ---------------------------------------------------------------- pass launches
+namespace gi {
+
+// The passes of a frame follow one another within microseconds on one stream.  launch() lets a pass's
+// blocks be scheduled while the pass before still runs (programmatic stream serialisation), and
+// pass_begin(), the first thing every such kernel does, lets the next pass be scheduled in turn and waits
+// until every earlier one has completed and its writes are visible.  Nothing that a kernel may have
+// written is read, and nothing is written, before it: plain accesses and atomics stay behind it by its
+// memory clobber, and the cache-operator loads (__ldca, __ldcg, __ldcs), which the compiler may move across
+// that, by their addresses, which depend on the zero it returns (block indexes and the few fixed
+// addresses have it added).  Non-coherent loads are for data that no kernel writes.  A kernel launched
+// plainly passes through it, and so does the first pass of a capture.
+// What bounds short passes is the gap between them (about 2 us each: drain, launch, ramp): without it
+// the 64 x 64 frame takes 30.9 us for 39.0, the 1080p frame 139.7 for 150.2, the temporal chain 122.8 for
+// 138.4, training 305 for 332.  Two kinds stay with plain launches: the batched passes, resident grids of
+// 150-560 us each whose waiting blocks only hold room (16 views: 1296 us with, 1291 without), and the
+// encoding that follows an inference kernel (beside its launch).
+__device__ __forceinline__ uint32_t pass_begin() {
+    uint32_t zero;
+    asm volatile(
+        "griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+    return zero;
+}
+// a plain (coherent) load, ordered behind pass_begin()
+template <typename T>
+__device__ __forceinline__ T ld(const T *p) {
+    return *p;
+}
+
+template <typename... P, typename... A>
+inline void launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // the callers read the error with cudaGetLastError
+}
+
+} // namespace gi
+
 // ---------------------------------------------------------------- device helpers
 namespace gi {
 

@@ -164,7 +164,7 @@ __device__ __forceinline__ void spawn_body(const SpawnArgs &a, uint32_t bx, uint
         bool fresh = false;
         float4 nd = make_float4(0.f, 0.f, 0.f, 0.f);
         if ((px >> 3) == tx && (py >> 3) == ty) {
-            nd = __ldg(a.gbuf + (size_t)py * a.width + px);
+            nd = __ldca(a.gbuf + (size_t)py * a.width + px);
             fresh = isfinite(nd.w) && nd.w >= 0.0f;
         }
         if (fresh) {
@@ -204,7 +204,10 @@ __device__ __forceinline__ void spawn_body(const SpawnArgs &a, uint32_t bx, uint
     }
 }
 
-__global__ void __launch_bounds__(256) k_spawn(SpawnArgs a) { spawn_body(a, blockIdx.x, blockIdx.y); }
+__global__ void __launch_bounds__(256) k_spawn(SpawnArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
+    spawn_body(a, bid, blockIdx.y);
+}
 
 // Levels 5 and up, from level 4, in one block.
 __device__ __forceinline__ void mip_tail_body(uint32_t *mask, const MipInfo &mi) {
@@ -223,18 +226,20 @@ __device__ __forceinline__ void mip_tail_body(uint32_t *mask, const MipInfo &mi)
     }
 }
 
-__global__ void __launch_bounds__(1024) k_mip_tail(uint32_t *mask, MipInfo mi) { mip_tail_body(mask, mi); }
+__global__ void __launch_bounds__(1024) k_mip_tail(uint32_t *mask, MipInfo mi) {
+    mip_tail_body(mask + pass_begin(), mi);
+}
 
 // ---------------------------------------------------------------- probe irradiance
 
 __device__ __forceinline__ float3 fetch_resolved(const void *r, uint32_t stride, int f16, uint32_t s) {
     r = static_cast<const char *>(r) + (size_t)s * stride;
     if (f16) {
-        const ushort4 h = __ldg(reinterpret_cast<const ushort4 *>(r));
+        const ushort4 h = __ldca(reinterpret_cast<const ushort4 *>(r));
         return make_float3(__half2float(__ushort_as_half(h.x)), __half2float(__ushort_as_half(h.y)),
                            __half2float(__ushort_as_half(h.z)));
     }
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(r));
+    const float4 v = __ldca(reinterpret_cast<const float4 *>(r));
     return make_float3(v.x, v.y, v.z);
 }
 
@@ -380,7 +385,7 @@ template <bool SURR, bool RPC1>
 __device__ __forceinline__ void integrate_quad(const IntegrateArgs &a, uint32_t p, bool valid, const float *s_mom) {
     const int h = threadIdx.x & 3;
     float4 n4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (valid) n4 = __ldg(a.nrm + p);
+    if (valid) n4 = __ldca(a.nrm + p);
     const bool live = valid && n4.w != 0.0f;
     float S[10][3], U[10];
 #pragma unroll
@@ -430,11 +435,11 @@ __device__ __forceinline__ void integrate_quad(const IntegrateArgs &a, uint32_t 
                     // records rec0 + i, rec0 = (p rpp + 64 j + 16 h + i0): bits 16 (h & 1) + i0 + i of
                     // the answer word of the 32 records starting at the probe's 64 j + 32 (h >> 1)
                     const size_t rec0 = rec_base + j * 64u + 16u * h + i0;
-                    const uint32_t wbits = __ldg(a.ovr_bits + (rec0 >> 5)) >> ((rec0 & 31u));
+                    const uint32_t wbits = __ldca(a.ovr_bits + (rec0 >> 5)) >> ((rec0 & 31u));
 #pragma unroll
                     for (int i = 0; i < kIntPass; ++i)
                         if ((wbits >> i) & 1u) {
-                            const float4 o = __ldg(a.ovr + rec0 + i);
+                            const float4 o = __ldca(a.ovr + rec0 + i);
                             r[i] = make_float3(o.x, o.y, o.z);
                             hs[i] = true;
                         }
@@ -518,21 +523,23 @@ __device__ __forceinline__ void integrate_body(const IntegrateArgs &a, uint32_t 
 
 template <bool RPC1>
 __global__ void __launch_bounds__(kIntThreads, 4) k_integrate(IntegrateArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) float s_mom[64 * kMomStride];
     load_moment_table<true>(s_mom);
     __syncthreads();
-    integrate_body<false, RPC1>(a, blockIdx.x, s_mom);
+    integrate_body<false, RPC1>(a, bid, s_mom);
 }
 
 // Probe atlas: float4 per (probe, cell) = (mean radiance rgb, mean hit distance); zeros for no probe.
 constexpr int kGatherThreads = 256;
 __global__ void __launch_bounds__(kGatherThreads) k_gather(IntegrateArgs a, float4 *atlas) {
-    const uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t bid = blockIdx.x + pass_begin();
+    const uint32_t p = (bid * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (p >= a.probes) return;
     float4 *dst = atlas + (size_t)p * 64;
     const RayPair first = load_rays(a, (size_t)p * a.rpp + lane);
-    if (__ldg(&a.nrm[p].w) == 0.0f) {
+    if (__ldca(&a.nrm[p].w) == 0.0f) {
         dst[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         dst[lane + 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
@@ -552,13 +559,14 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(IntegrateArgs a, floa
 constexpr int kProjThreads = 128;  // 32 probes per block
 __global__ void __launch_bounds__(kProjThreads) k_project(const float4 *atlas, const float4 *nrm, float *sh,
                                                           uint32_t probes) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) float s_mom[64 * kMomStride];
     load_moment_table<false>(s_mom);
     const int h = threadIdx.x & 3;
-    const uint32_t p = blockIdx.x * (kProjThreads / 4) + (threadIdx.x >> 2);
+    const uint32_t p = bid * (kProjThreads / 4) + (threadIdx.x >> 2);
     const bool valid = p < probes;
     float4 n4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (valid) n4 = __ldg(nrm + p);
+    if (valid) n4 = __ldca(nrm + p);
     const bool live = valid && n4.w != 0.0f;
     __syncthreads();
     float S[10][3];
@@ -570,7 +578,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(const float4 *atlas, c
         for (int i0 = 0; i0 < 16; i0 += 8) {
             float4 L[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) L[i] = __ldg(src + 4 * (i0 + i));
+            for (int i = 0; i < 8; ++i) L[i] = __ldca(src + 4 * (i0 + i));
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float4 *mc = reinterpret_cast<const float4 *>(s_mom + (4 * (i0 + i) + h) * kMomStride);
@@ -611,10 +619,11 @@ __global__ void __launch_bounds__(kProjThreads) k_project(const float4 *atlas, c
 }
 template <bool RPC1>
 __global__ void __launch_bounds__(kIntThreads, 4) k_integrate_surr(IntegrateArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) float s_mom[64 * kMomStride];
     load_moment_table<true>(s_mom);
     __syncthreads();
-    integrate_body<true, RPC1>(a, blockIdx.x, s_mom);
+    integrate_body<true, RPC1>(a, bid, s_mom);
 }
 
 // ---------------------------------------------------------------- temporal path
@@ -632,7 +641,8 @@ __device__ __forceinline__ float dot3_rn(float ax, float ay, float az, float bx,
 // bid needs no shared memory.  (One thread per pixel, four trips, atomicMin in shared memory: 27.8 us at
 // 1080p, now 22.7 us; 50 MB, 7.4 us at the copy rate.)
 __global__ void __launch_bounds__(kGatherThreads) k_reproject(ReprojArgs a) {
-    const uint32_t lane = threadIdx.x & 31u, t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t bid = blockIdx.x + pass_begin();
+    const uint32_t lane = threadIdx.x & 31u, t = (bid * blockDim.x + threadIdx.x) >> 5;
     const uint32_t tx = t % a.tiles_x, ty = t / a.tiles_x;
     if (ty >= a.tiles_y) return;
     const uint32_t x = 8u * tx + (lane & 7u);
@@ -659,7 +669,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_reproject(ReprojArgs a) {
             const float fy = floorf(__fadd_rn(__fadd_rn((float)y, 0.5f), mv[h].y));
             if (fx >= 0.0f && fy >= 0.0f && fx < (float)a.width && fy < (float)a.height) {
                 tq[h] = ((uint32_t)fy >> 3) * a.tiles_x + ((uint32_t)fx >> 3);
-                pm[h] = __ldg(a.prev_mask + tq[h]);
+                pm[h] = __ldca(a.prev_mask + tq[h]);
             }
         }
     }
@@ -668,7 +678,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_reproject(ReprojArgs a) {
     for (int h = 0; h < 2; ++h) {
         my[h] = kScoreNone;
         if (pm[h] != GI_PROBE_NONE) {
-            const float4 pp = __ldg(a.prev_pos + tq[h]), pn = __ldg(a.prev_nrm + tq[h]);
+            const float4 pp = __ldca(a.prev_pos + tq[h]), pn = __ldca(a.prev_nrm + tq[h]);
             const float3 w = pixel_world_exact(a.cam, x, 8u * ty + (lane >> 3) + 4u * h, nd[h].w);
             const float vx = __fsub_rn(pp.x, w.x), vy = __fsub_rn(pp.y, w.y), vz = __fsub_rn(pp.z, w.z);
             const float plane = fabsf(dot3_rn(vx, vy, vz, nd[h].x, nd[h].y, nd[h].z));
@@ -715,7 +725,8 @@ __device__ __forceinline__ float3 temporal_blend(float3 c, float3 p) {
 // distance, as k_gather) and blends each cell with the same cell of the tile's reprojected probe;
 // a reprojected-only probe copies its source's cells; a tile without probe gets zeros.
 __global__ void __launch_bounds__(kGatherThreads) k_gather_temporal(TemporalArgs a) {
-    const uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t bid = blockIdx.x + pass_begin();
+    const uint32_t t = (bid * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (t >= a.probes) return;
     const uint32_t tx = t % a.tiles_x, ty = t / a.tiles_x;
@@ -723,18 +734,18 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_temporal(TemporalArgs
     const uint32_t px = min(st * sx + (uint32_t)a.jx, a.width - 1u);
     const uint32_t py = min(st * sy + (uint32_t)a.jy, a.height - 1u);
     // the source, the spawn pixel's distance and the rays of a tile that may be fresh, together
-    const uint32_t src = __ldg(a.src + t), sp = sy * a.spawn_x + sx;
+    const uint32_t src = __ldca(a.src + t), sp = sy * a.spawn_x + sx;
     bool fresh = false;
     RayPair first = {GI_SLOT_NONE, GI_SLOT_NONE, 0.f, 0.f};
     if ((px >> 3) == tx && (py >> 3) == ty) {
         first = load_rays(a.g, (size_t)sp * a.g.rpp + lane);
-        const float d = __ldg(&a.gbuf[(size_t)py * a.width + px].w);
+        const float d = __ldca(&a.gbuf[(size_t)py * a.width + px].w);
         fresh = isfinite(d) && d >= 0.0f;
     }
     float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
     if (src != GI_PROBE_NONE) {
-        p0 = __ldg(a.prev_atlas + (size_t)src * 64 + lane);
-        p1 = __ldg(a.prev_atlas + (size_t)src * 64 + lane + 32);
+        p0 = __ldca(a.prev_atlas + (size_t)src * 64 + lane);
+        p1 = __ldca(a.prev_atlas + (size_t)src * 64 + lane + 32);
     }
     float4 *dst = a.atlas + (size_t)t * 64;
     float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
@@ -767,7 +778,7 @@ __device__ __forceinline__ uint32_t find_closest_probe(const uint32_t *mask, con
     for (int m = m0; m < mi.count; ++m) {
         const int x = tx + ox, y = ty + oy;
         if (x < 0 || y < 0 || x >= mi.w[m] || y >= mi.h[m]) break;
-        const uint32_t p = __ldg(mask + mi.off[m] + y * mi.w[m] + x);
+        const uint32_t p = __ldca(mask + mi.off[m] + y * mi.w[m] + x);
         if (p != GI_PROBE_NONE) return p;
         tx >>= 1;
         ty >>= 1;
@@ -944,11 +955,11 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
     float tq = 0.f;
     if (tile) {
         if (lane < 28) {
-            v = __ldg(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
+            v = __ldca(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
         } else {
-            qo = __ldg(a.mask + pidx);
-            tq = __ldg(&a.ppos[pidx].w);
-            v = __ldg(a.pnrm + pidx);
+            qo = __ldca(a.mask + pidx);
+            tq = __ldca(&a.ppos[pidx].w);
+            v = __ldca(a.pnrm + pidx);
         }
     }
 #pragma unroll
@@ -971,10 +982,10 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
         if (up != GI_PROBE_NONE) {
             pidx = (up >> 19) * a.tiles_x + ((up & 0xFFFFu) >> 3);
             if (lane < 28) {
-                v = __ldg(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
+                v = __ldca(reinterpret_cast<const float4 *>(a.sh + (size_t)pidx * GI_SH_STRIDE) + (lane - 7 * o));
             } else {
-                tq = __ldg(&a.ppos[pidx].w);
-                v = __ldg(a.pnrm + pidx);
+                tq = __ldca(&a.ppos[pidx].w);
+                v = __ldca(a.pnrm + pidx);
             }
         }
     }
@@ -1040,14 +1051,18 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
             const int y = y0 + 4 * h;
             if (x < 0 || y < 0 || x >= (int)a.width || y >= (int)a.height) continue;
             const uint32_t px = (uint32_t)y * a.width + (uint32_t)x;
-            const float4 g = __ldg(a.gbuf + px);
+            const float4 g = __ldca(a.gbuf + px);
             interp_pixel<false>(a, s, x, y, fx, ((float)((lane >> 3) + 4 * h) + 0.5f) * 0.125f, g, px, true,
                                 isfinite(g.w) && g.w >= 0.0f, found);
         }
     }
 }
 
-__global__ void __launch_bounds__(32 * kInterpWarps, kInterpBlocksPerSm) k_interpolate(InterpArgs a) { interpolate_body(a, blockIdx.x, blockIdx.y); }
+__global__ void __launch_bounds__(32 * kInterpWarps, kInterpBlocksPerSm) k_interpolate(
+    InterpArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
+    interpolate_body(a, bid, blockIdx.y);
+}
 
 static bool layout_matches(const gi_probe_layout &l, uint32_t w, uint32_t h) {
     return l.tiles_x == (w + 7) / 8 && l.tiles_y == (h + 7) / 8 && l.num_probes == l.tiles_x * l.tiles_y &&
@@ -1196,16 +1211,17 @@ struct FilterArgs {
 // warp searching for the block's four probes before a barrier: 41 us, the barrier waits for it.
 constexpr int kFiltWarps = 4, kFiltBlocksPerSm = 8;
 __global__ void __launch_bounds__(32 * kFiltWarps, kFiltBlocksPerSm) k_filter(FilterArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ uint32_t s_qi[kFiltWarps][6];
     __shared__ float4 s_rel[kFiltWarps][6];  // q - p (xyz), depth weight
     __shared__ float4 s_nq[kFiltWarps][6];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t p = blockIdx.x * kFiltWarps + warp;
+    const uint32_t p = bid * kFiltWarps + warp;
     if (p >= a.probes) return;
     const float4 *in = a.in + (size_t)p * 64 + lane;
     float4 *out = a.out + (size_t)p * 64 + lane;
-    const float4 n4 = __ldg(a.pnrm + p);
-    const float4 va = __ldg(in), vb = __ldg(in + 32);
+    const float4 n4 = __ldca(a.pnrm + p);
+    const float4 va = __ldca(in), vb = __ldca(in + 32);
     if (lane < 6) {
         const int step = (((lane & 1) << 1) - 1) * ((lane >> 1) + 1);
         const int ox = a.axis == 0 ? step : 0, oy = a.axis == 0 ? 0 : step;
@@ -1213,16 +1229,16 @@ __global__ void __launch_bounds__(32 * kFiltWarps, kFiltBlocksPerSm) k_filter(Fi
         uint32_t qi = GI_PROBE_NONE;
         if (qx >= 0 && qy >= 0 && qx < a.mi.w[0] && qy < a.mi.h[0]) {
             uint32_t k = (uint32_t)qy * a.tiles_x + (uint32_t)qx;
-            uint32_t q = __ldg(a.mask + k);
-            const float4 pp = __ldg(a.ppos + p);
-            float4 pq = __ldg(a.ppos + k), nq = __ldg(a.pnrm + k);
+            uint32_t q = __ldca(a.mask + k);
+            const float4 pp = __ldca(a.ppos + p);
+            float4 pq = __ldca(a.ppos + k), nq = __ldca(a.pnrm + k);
             if (q == GI_PROBE_NONE) q = find_closest_probe(a.mask, a.mi, tx >> 1, ty >> 1, ox, oy, 1);
             if (q != GI_PROBE_NONE) {
                 const uint32_t found = ((q >> 16) >> 3) * a.tiles_x + ((q & 0xFFFFu) >> 3);
                 if (found != k) {
                     k = found;
-                    pq = __ldg(a.ppos + k);
-                    nq = __ldg(a.pnrm + k);
+                    pq = __ldca(a.ppos + k);
+                    nq = __ldca(a.pnrm + k);
                 }
                 const float cs = a.dscale * pp.w;
                 const float rx = pq.x - pp.x, ry = pq.y - pp.y, rz = pq.z - pp.z;
@@ -1251,7 +1267,7 @@ __global__ void __launch_bounds__(32 * kFiltWarps, kFiltBlocksPerSm) k_filter(Fi
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             const uint32_t qi = s_qi[warp][i];
-            vq[i] = qi != GI_PROBE_NONE ? __ldg(a.in + (size_t)qi * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            vq[i] = qi != GI_PROBE_NONE ? __ldca(a.in + (size_t)qi * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         // world direction of the cell centre in the probe frame (Duff et al. 2017)
         const float sgn = copysignf(1.0f, nz);
@@ -1300,8 +1316,9 @@ __global__ void __launch_bounds__(256) k_spawn_batched(const SpawnArgs *args, co
 
 // MIP levels 5 and up of every view: one block per view.
 __global__ void __launch_bounds__(1024) k_mip_tail_batched(const SpawnArgs *args) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ SpawnArgs sa;
-    load_view_args(sa, args + blockIdx.x);
+    load_view_args(sa, args + bid);
     __syncthreads();
     if (sa.mi.count > 5) mip_tail_body(sa.mask, sa.mi);
 }
@@ -1349,7 +1366,8 @@ gi_status launch_integrate_batched(const IntegrateArgs *args, const uint32_t *pr
 gi_status launch_interpolate_batched(const InterpArgs *args, const uint32_t *prefix, uint32_t nviews,
                                      uint32_t blocks, cudaStream_t st) {
     if (blocks == 0) return GI_OK;
-    k_interpolate_batched<<<resident_grid(k_interpolate_batched, 32 * kInterpWarps, blocks), 32 * kInterpWarps, 0, st>>>(args, prefix, nviews);
+    k_interpolate_batched<<<resident_grid(k_interpolate_batched, 32 * kInterpWarps, blocks), 32 * kInterpWarps, 0, st>>>(
+        args, prefix, nviews);
     return cuda_status(cudaGetLastError(), "k_interpolate_batched launch");
 }
 
@@ -1399,10 +1417,10 @@ gi_status gi_probes_spawn(const gi_gbuffer *gbuf, const gi_view *view, const gi_
     cudaStream_t st = (cudaStream_t)stream;
     const SpawnArgs a = spawn_args(gbuf, view, pr);
     dim3 grid((a.tiles_x + 15) / 16, (a.tiles_y + 15) / 16);
-    k_spawn<<<grid, 256, 0, st>>>(a);
+    launch(k_spawn, grid, 256, 0, st, a);
     s = cuda_status(cudaGetLastError(), "k_spawn launch");
     if (s == GI_OK && a.mi.count > 5) {
-        k_mip_tail<<<1, 1024, 0, st>>>(pr->mask, a.mi);
+        launch(k_mip_tail, 1, 1024, 0, st, pr->mask, a.mi);
         s = cuda_status(cudaGetLastError(), "k_mip_tail launch");
     }
     return s;
@@ -1423,10 +1441,10 @@ gi_status gi_probes_spawn_upscaled(const gi_gbuffer *gbuf, const gi_view *view, 
     a.jx = halton_scaled(view->frame + 1u, 2, 8u * upscale);
     a.jy = halton_scaled(view->frame + 1u, 3, 8u * upscale);
     dim3 grid((a.tiles_x + 15) / 16, (a.tiles_y + 15) / 16);
-    k_spawn<<<grid, 256, 0, st>>>(a);
+    launch(k_spawn, grid, 256, 0, st, a);
     s = cuda_status(cudaGetLastError(), "k_spawn launch");
     if (s == GI_OK && a.mi.count > 5) {
-        k_mip_tail<<<1, 1024, 0, st>>>(pr->mask, a.mi);
+        launch(k_mip_tail, 1, 1024, 0, st, pr->mask, a.mi);
         s = cuda_status(cudaGetLastError(), "k_mip_tail launch");
     }
     return s;
@@ -1461,7 +1479,8 @@ gi_status gi_probes_reproject(const gi_gbuffer *gbuf, const gi_view *view, const
     a.nrm = reinterpret_cast<float4 *>(cur->nrm);
     a.src = src;
     const uint32_t P = cur->layout.num_probes;
-    k_reproject<<<(P + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0, (cudaStream_t)stream>>>(a);
+    launch(k_reproject, (P + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0,
+           (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_reproject launch");
 }
 
@@ -1497,7 +1516,7 @@ gi_status gi_probes_gather_temporal(gi_cache_t cache, const gi_gbuffer *gbuf, co
     a.atlas = reinterpret_cast<float4 *>(atlas);
     const uint32_t blocks = (a.probes + kGatherThreads / 32 - 1) / (kGatherThreads / 32);
     if (blocks == 0) return GI_OK;
-    k_gather_temporal<<<blocks, kGatherThreads, 0, (cudaStream_t)stream>>>(a);
+    launch(k_gather_temporal, blocks, kGatherThreads, 0, (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_gather_temporal launch");
 }
 
@@ -1510,8 +1529,8 @@ gi_status gi_probes_integrate(gi_cache_t cache, const gi_probes *pr, const uint3
     const IntegrateArgs a = integrate_args(cache, pr, slot_ids, rays_per_probe, env);
     if (a.probes == 0) return GI_OK;
     const unsigned blocks = (a.probes + kIntThreads / 4 - 1) / (kIntThreads / 4);
-    if (rays_per_probe == 64) k_integrate<true><<<blocks, kIntThreads, 0, (cudaStream_t)stream>>>(a);
-    else k_integrate<false><<<blocks, kIntThreads, 0, (cudaStream_t)stream>>>(a);
+    if (rays_per_probe == 64) launch(k_integrate<true>, blocks, kIntThreads, 0, (cudaStream_t)stream, a);
+    else launch(k_integrate<false>, blocks, kIntThreads, 0, (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_integrate launch");
 }
 
@@ -1531,8 +1550,8 @@ gi_status gi_probes_integrate_nrc(gi_cache_t cache, gi_nrc_t nrc, const gi_probe
     s = nrc_override(nrc, n, &a.ovr_bits, &a.ovr);
     if (s != GI_OK) return s;
     const unsigned blocks = (a.probes + kIntThreads / 4 - 1) / (kIntThreads / 4);
-    if (rays_per_probe == 64) k_integrate_surr<true><<<blocks, kIntThreads, 0, (cudaStream_t)stream>>>(a);
-    else k_integrate_surr<false><<<blocks, kIntThreads, 0, (cudaStream_t)stream>>>(a);
+    if (rays_per_probe == 64) launch(k_integrate_surr<true>, blocks, kIntThreads, 0, (cudaStream_t)stream, a);
+    else launch(k_integrate_surr<false>, blocks, kIntThreads, 0, (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_integrate_surr launch");
 }
 
@@ -1551,7 +1570,8 @@ gi_status gi_probes_gather(gi_cache_t cache, const gi_probes *pr, const uint32_t
     IntegrateArgs a = integrate_args(cache, pr, slot_ids, rays_per_probe, env);
     if (a.probes == 0) return GI_OK;
     a.ray_len = ray_len;
-    k_gather<<<(a.probes + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0, (cudaStream_t)stream>>>(a, reinterpret_cast<float4 *>(atlas));
+    launch(k_gather, (a.probes + kGatherThreads / 32 - 1) / (kGatherThreads / 32), kGatherThreads, 0,
+           (cudaStream_t)stream, a, reinterpret_cast<float4 *>(atlas));
     return cuda_status(cudaGetLastError(), "k_gather launch");
 }
 
@@ -1580,7 +1600,7 @@ gi_status gi_probes_filter(const gi_probes *pr, const gi_view *view, const float
     a.dscale = (float)distance_scale(view->fov_y, view->width, view->height);
     a.axis = (int)axis;
     if (a.probes == 0) return GI_OK;
-    k_filter<<<(a.probes + kFiltWarps - 1) / kFiltWarps, 32 * kFiltWarps, 0, (cudaStream_t)stream>>>(a);
+    launch(k_filter, (a.probes + kFiltWarps - 1) / kFiltWarps, 32 * kFiltWarps, 0, (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_filter launch");
 }
 
@@ -1593,8 +1613,8 @@ gi_status gi_probes_project(const gi_probes *pr, const float *atlas, gi_stream_t
     if (s != GI_OK) return s;
     const uint32_t P = pr->layout.num_probes;
     if (P == 0) return GI_OK;
-    k_project<<<(P + kProjThreads / 4 - 1) / (kProjThreads / 4), kProjThreads, 0, (cudaStream_t)stream>>>(reinterpret_cast<const float4 *>(atlas),
-                                                              reinterpret_cast<const float4 *>(pr->nrm), pr->sh, P);
+    launch(k_project, (P + kProjThreads / 4 - 1) / (kProjThreads / 4), kProjThreads, 0, (cudaStream_t)stream,
+           reinterpret_cast<const float4 *>(atlas), reinterpret_cast<const float4 *>(pr->nrm), pr->sh, P);
     return cuda_status(cudaGetLastError(), "k_project launch");
 }
 
@@ -1604,7 +1624,7 @@ gi_status gi_probes_interpolate(const gi_gbuffer *gbuf, const gi_view *view, con
     if (s != GI_OK) return s;
     const InterpArgs a = interp_args(gbuf, view, pr, out);
     dim3 grid(interp_grid_x(view->width), interp_grid_y(view->height));
-    k_interpolate<<<grid, 32 * kInterpWarps, 0, (cudaStream_t)stream>>>(a);
+    launch(k_interpolate, grid, 32 * kInterpWarps, 0, (cudaStream_t)stream, a);
     return cuda_status(cudaGetLastError(), "k_interpolate launch");
 }
 

@@ -75,6 +75,7 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) { return a >
 // with 2x2 upscale the merge (__match_any_sync, pointer-jumping sums) cost 5 us of the frame.
 template <int KEY_DIR>
 __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     const UpdateArgs &a = ta.u;
     __shared__ uint32_t s_clamped, s_maxp, s_new;
     if (threadIdx.x == 0) {
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) 
     const unsigned long long stride = (unsigned long long)gridDim.x * kUpdThreads;
     uint32_t my_clamped = 0, my_maxp = 0, my_new = 0;
     unsigned long long my_dropped = 0;
-    for (unsigned long long base = (unsigned long long)blockIdx.x * kUpdThreads; base < a.n; base += stride) {
+    for (unsigned long long base = (unsigned long long)bid * kUpdThreads; base < a.n; base += stride) {
         const unsigned long long i = base + threadIdx.x;
         const bool inr = i < a.n;
         // the key's planes of an in-range record in one round trip; the radiance is read by
@@ -169,10 +170,11 @@ constexpr int kCompactThreads = 256;
 // out since the last resolve.
 __global__ void __launch_bounds__(kCompactThreads) k_tile_compact(const unsigned long long *tmask, uint32_t *cidx,
                                                                   uint32_t *tlist, uint32_t tiles, Counters *ctr) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ uint32_t s_cnt[kCompactThreads / 32];
     __shared__ uint32_t s_base;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t t = blockIdx.x * kCompactThreads + threadIdx.x;
+    const uint32_t t = bid * kCompactThreads + threadIdx.x;
     bool need = false;
     if (t < tiles) need = __ldcg(tmask + t) != 0ull && __ldcg(cidx + t) == GI_SLOT_NONE;
     const unsigned b = __ballot_sync(kFull, need);
@@ -199,6 +201,7 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_accumulate(const uint32
                                                                     const float *r1, const float *r2,
                                                                     unsigned long long n, const uint32_t *cidx,
                                                                     uint32_t cells, Accum *accum, Counters *ctr) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(32) unsigned long long s_red[kUpdThreads][4];
     __shared__ uint32_t s_clamped;
     if (threadIdx.x == 0) s_clamped = 0;
@@ -206,7 +209,7 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_accumulate(const uint32
     const int lane = threadIdx.x & 31;
     uint32_t my_clamped = 0;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x; base < n; base += stride) {
+    for (unsigned long long base = (unsigned long long)bid * blockDim.x; base < n; base += stride) {
         const unsigned long long i = base + threadIdx.x;
         const uint32_t id = i < n ? __ldcs(slot_ids + i) : GI_SLOT_NONE;
         bool ok = id < cells;
@@ -297,12 +300,13 @@ __device__ __forceinline__ float4 box4(const float4 &a, const float4 &b, const f
 // from its four children; then each live cell takes the finest level with enough samples.
 // Completion is counted per warp, so warps never wait for one another.
 __global__ void __launch_bounds__(kTileResThreads) k_tile_resolve(TileResolveArgs a) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ float4 s_lv[kTileResWarps][kTileCells + kTileMips];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float4 *lv = s_lv[w];
-    const uint32_t warp = (blockIdx.x * kTileResThreads + threadIdx.x) >> 5;
+    const uint32_t warp = (bid * kTileResThreads + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * kTileResThreads) >> 5;
-    const uint32_t n = __ldcg(&a.ctr->touch_count);
+    const uint32_t n = ld(&a.ctr->touch_count);
     uint32_t i = warp;
     uint32_t t = 0;
     unsigned long long m = 0, o = 0;
@@ -449,8 +453,9 @@ __global__ void __launch_bounds__(kTileResThreads) k_tile_resolve(TileResolveArg
 template <int KEY_DIR>
 __global__ void k_tile_query_points(TileUpdateArgs ta, TileArrays t, uint32_t res_stride, int f16, LiveRule rule,
                                     float4 *out) {
+    const uint32_t bid = blockIdx.x + pass_begin();
     const UpdateArgs &a = ta.u;
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < a.n;
+    for (unsigned long long i = bid * (unsigned long long)blockDim.x + threadIdx.x; i < a.n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         const float len = a.len[i];
         const float px = a.p[0][i], py = a.p[1][i], pz = a.p[2][i];
@@ -466,11 +471,11 @@ __global__ void k_tile_query_points(TileUpdateArgs ta, TileArrays t, uint32_t re
             cell_of_key(key, a.mask, home, tag);
             uint32_t s = home;
             for (uint32_t k = 0; k < a.max_probe; ++k) {
-                const uint32_t w = __ldg(t.tags + s);
+                const uint32_t w = __ldca(t.tags + s);
                 if (w == kEmpty) break;
                 if (w == tag) {
                     const uint32_t e = s * kTileCells + cell;
-                    if (answers(__ldg(t.stamp + e), rule)) {
+                    if (answers(__ldca(t.stamp + e), rule)) {
                         const float3 v = load_resolved(t.resolved, res_stride, f16, e);
                         o = make_float4(v.x, v.y, v.z, 1.0f);
                     }
@@ -587,18 +592,18 @@ gi_status tile_update_launch(const TileUpdateArgs &a, int key_dir, int resident_
         std::max<unsigned long long>((unsigned long long)resident_blocks, chunks), (a.u.n + kUpdThreads - 1) / kUpdThreads);
     if (blocks == 0) return GI_OK;
     if (key_dir == GI_KEY_DIR_NORMAL)
-        k_tile_key<GI_KEY_DIR_NORMAL><<<blocks, kUpdThreads, 0, st>>>(a);
+        launch(k_tile_key<GI_KEY_DIR_NORMAL>, blocks, kUpdThreads, 0, st, a);
     else
-        k_tile_key<GI_KEY_DIR_RAY><<<blocks, kUpdThreads, 0, st>>>(a);
+        launch(k_tile_key<GI_KEY_DIR_RAY>, blocks, kUpdThreads, 0, st, a);
     gi_status s = cuda_status(cudaGetLastError(), "k_tile_key launch");
     if (s != GI_OK) return s;
     const uint32_t tiles = a.u.mask + 1u;
-    k_tile_compact<<<(tiles + kCompactThreads - 1) / kCompactThreads, kCompactThreads, 0, st>>>(a.tmask, a.cidx,
-                                                                                                a.tlist, tiles, a.u.ctr);
+    launch(k_tile_compact, (tiles + kCompactThreads - 1) / kCompactThreads, kCompactThreads, 0, st, a.tmask, a.cidx,
+           a.tlist, tiles, a.u.ctr);
     s = cuda_status(cudaGetLastError(), "k_tile_compact launch");
     if (s != GI_OK) return s;
-    k_tile_accumulate<<<blocks, kUpdThreads, 0, st>>>(a.u.slot_ids, a.u.rad[0], a.u.rad[1], a.u.rad[2], a.u.n, a.cidx,
-                                                      tiles * (uint32_t)kTileCells, a.u.accum, a.u.ctr);
+    launch(k_tile_accumulate, blocks, kUpdThreads, 0, st, a.u.slot_ids, a.u.rad[0], a.u.rad[1], a.u.rad[2], a.u.n,
+           a.cidx, tiles * (uint32_t)kTileCells, a.u.accum, a.u.ctr);
     return cuda_status(cudaGetLastError(), "k_tile_accumulate launch");
 }
 
@@ -612,16 +617,16 @@ int tile_resolve_blocks_per_sm() {
 gi_status tile_resolve_launch(const TileResolveArgs &a, int blocks, cudaStream_t st) {
     // no more warps than tiles
     blocks = std::min<int>(blocks, (int)((a.tiles + kTileResWarps - 1) / kTileResWarps));
-    k_tile_resolve<<<blocks, kTileResThreads, 0, st>>>(a);
+    launch(k_tile_resolve, blocks, kTileResThreads, 0, st, a);
     return cuda_status(cudaGetLastError(), "k_tile_resolve launch");
 }
 
 gi_status tile_query_points_launch(const TileUpdateArgs &a, const TileArrays &t, uint32_t res_stride, int f16,
                                    LiveRule rule, float4 *out, int blocks, int key_dir, cudaStream_t st) {
     if (key_dir == GI_KEY_DIR_NORMAL)
-        k_tile_query_points<GI_KEY_DIR_NORMAL><<<blocks, 256, 0, st>>>(a, t, res_stride, f16, rule, out);
+        launch(k_tile_query_points<GI_KEY_DIR_NORMAL>, blocks, 256, 0, st, a, t, res_stride, f16, rule, out);
     else
-        k_tile_query_points<GI_KEY_DIR_RAY><<<blocks, 256, 0, st>>>(a, t, res_stride, f16, rule, out);
+        launch(k_tile_query_points<GI_KEY_DIR_RAY>, blocks, 256, 0, st, a, t, res_stride, f16, rule, out);
     return cuda_status(cudaGetLastError(), "k_tile_query_points launch");
 }
 
