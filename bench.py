@@ -73,9 +73,9 @@ UPDATE_HEADER = ("gi_internal.cuh", "namespace gi {", "struct ResolveArgs {")
 NRC_ADAM_SECTION = ("gi_nrc.cu", "// ---------------------------------------------------------------- gradient scatter and Adam",
                     "// ---------------------------------------------------------------- query selection")
 NCU_TRAFFIC = {
-    # k_update, boxes-1080p (5th launch): 158.97 MB read + 33.27 MB written
-    "2:update": {"bytes_per_launch": 192241152, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
-                 "source_sha": "0d84d9e0fa0f439e"},
+    # k_update, boxes-1080p (5th launch): 158.88 MB read + 33.17 MB written
+    "2:update": {"bytes_per_launch": 192052224, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
+                 "source_sha": "530c436e01a8c6ee"},
     # k_nrc_adam (table and weights), Cornell 1080p: 105.84 MB read + 14.32 MB written
     "4:adam_table": {"bytes_per_launch": 120159744, "sources": (NRC_ADAM_SECTION,), "source_sha": "04fc4aad2b956f33"},
 }
@@ -610,7 +610,7 @@ def run_native(args, rank, world, local_rank):
             "roofline": {"bound": "hbm", "kernel": "k_filter", "algorithmic_bytes_per_launch": filt_bytes,
                          "achieved": filt_bytes / (filt_ms * 1e-3) / 1e9, "peak": peak,
                          "frac": filt_bytes / (filt_ms * 1e-3) / 1e9 / peak, "unit": "GB/s"}}
-    launches_per_step = 6  # k_spawn, k_mip_tail, k_update, k_resolve_bitmap, k_integrate, k_interpolate
+    launches_per_step = 6  # k_spawn, k_mip_tail, k_update, k_resolve_dense, k_integrate, k_interpolate
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": float(tot[1] / args.steps), "higher_is_better": True,
@@ -1539,10 +1539,10 @@ def run_surrogate(args, rank, world, local_rank):
                      "algorithmic_bytes_per_launch": adam_bytes, "touched_entries": n_touched,
                      "launch_ms": adam_ms, "peak_source": peak_src},
         "cpu_baseline": cpu,
-        # per surrogate-form frame: spawn 2, update, resolve, 5 per training minibatch (encode, network,
-        # scatter, two Adam kernels), query 3 (select, encode, network), integrate, interpolate;
+        # per surrogate-form frame: spawn 2, update, resolve, 4 per training minibatch (encode, network,
+        # scatter, Adam), query 3 (select, encode, network), integrate, interpolate;
         # per plain frame 6
-        "gpu_launches": int(args.steps * ((9 + 5 * cfg["nrc_train_steps"]) + 6)),
+        "gpu_launches": int(args.steps * ((9 + 4 * cfg["nrc_train_steps"]) + 6)),
         "clocks": clk,
     }
     return line
@@ -1697,7 +1697,7 @@ def run_far_routing(args, rank, world, local_rank):
         "routed_hits_last_frame": int(far.sum()), "answered_last_frame": int(cnt),
         "network_rel_l1_error_on_routed_hits_vs_plain_cache": net_err,
         "judged_error": float(st["judged_error"]),
-        "gpu_launches": int(steps * (4 + 7 + 5 * cfg4["nrc_train_steps"])),
+        "gpu_launches": int(steps * (4 + 7 + 4 * cfg4["nrc_train_steps"])),
         "clocks": clk,
     }
 

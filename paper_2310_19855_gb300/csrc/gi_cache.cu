@@ -190,10 +190,12 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
                     nxt = on;
                 }
             }
-            s_red[0] = q0;
-            s_red[1] = q1;
-            s_red[2] = q2;
-            s_red[3] = cnt;
+            if (BITMAP) {
+                s_red[0] = q0;
+                s_red[1] = q1;
+                s_red[2] = q2;
+                s_red[3] = cnt;
+            }
         }
         const bool leader = hit && (peers & ((1u << lane) - 1u)) == 0u;
         uint32_t slot = GI_SLOT_NONE, loc = GI_SLOT_NONE;
@@ -220,7 +222,19 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
         uint32_t my_slot = slot;
         if (MERGE) my_slot = __shfl_sync(kFull, slot, hit ? (__ffs(peers) - 1) : lane);
         if (inr) __stcs(a.slot_ids + i, hit ? my_slot : code);
-        warp_add_accum<!BITMAP>(a.accum, a.dense, loc, s_warp, lane, s_touch, &s_n);
+        if (MERGE && !BITMAP) {
+            // few leaders are left, and each waits for its own count: four lanes a record would add the
+            // trips of the other leaders (the calls on 1,000,000 records: 138.5 us so, 127.5 us like this)
+            if (loc != GI_SLOT_NONE) {
+                Accum *ac = a.accum + loc;
+                atomicAdd(&ac->sum[0], q0);
+                atomicAdd(&ac->sum[1], q1);
+                atomicAdd(&ac->sum[2], q2);
+                if (atomicAdd(&ac->count, cnt) == 0u) s_touch[atomicAdd(&s_n, 1u)] = loc;
+            }
+        } else {
+            warp_add_accum<!BITMAP>(a.accum, a.dense, loc, s_warp, lane, s_touch, &s_n);
+        }
     }
     // block totals of the statistics, one global atomic each
     my_clamped = __reduce_add_sync(kFull, my_clamped);
@@ -249,8 +263,9 @@ __global__ void __launch_bounds__(kUpdThreads, MERGE ? 6 : 8) k_update(UpdateArg
 }
 
 // touch-list form: 6 blocks per SM (the returning count's path needs more than 32 registers)
+constexpr int kUpdListBlocksPerSm = 6;
 template <int KEY_DIR, bool MERGE>
-__global__ void __launch_bounds__(kUpdThreads, 6) k_update_list(UpdateArgs a) {
+__global__ void __launch_bounds__(kUpdThreads, kUpdListBlocksPerSm) k_update_list(UpdateArgs a) {
     const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ __align__(16) unsigned long long s_acc[4 * kUpdThreads];
     __shared__ uint32_t s_touch[kUpdBlockRecords];
@@ -276,6 +291,13 @@ static inline void launch_update(const UpdateArgs &a, uint32_t key_dir, bool mer
 // Grid of k_update: enough blocks that none takes more than kUpdBlockRecords records.
 static inline int update_blocks(unsigned long long n) {
     return (int)((n + kUpdBlockRecords - 1) / kUpdBlockRecords);
+}
+// Grid of k_update_list: the resident blocks (as many as the records fill) or, where those would take more
+// than kUpdBlockRecords records each, more.  With only the blocks that the staging needs, 493,000 records
+// (576 x 428 pixels, 2 rays a cell) ran on 241 blocks and took 42 us; on 912 they take 21.
+static inline int list_update_blocks(unsigned long long n, uint32_t resident) {
+    const unsigned long long full = (n + kUpdThreads - 1) / kUpdThreads;
+    return std::max(update_blocks(n), (int)std::min<unsigned long long>(full, resident));
 }
 
 // ---------------------------------------------------------------- resolve
@@ -1086,7 +1108,7 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
         int per_sm = 0;
         s = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<0, false>, kUpdThreads, 0),
                         "occupancy");
-        c->upd_blocks = c->sms * std::max(per_sm, 1);
+        c->upd_blocks = c->sms * (c->touch ? kUpdListBlocksPerSm : std::max(per_sm, 1));
         c->res_blocks = c->sms * (c->touch ? kResListBlocksPerSm : kResBmBlocksPerSm);
         c->tres_blocks = c->sms * tile_resolve_blocks_per_sm();
     }
@@ -1143,7 +1165,7 @@ gi_status gi_cache_update(gi_cache_t c, const gi_hits *hits, const gi_view *view
     // the bitmap form stages nothing per block: a resident grid strides over the records
     const int blocks = !c->touch ? (int)std::min<unsigned long long>((unsigned long long)c->upd_blocks,
                                                                       (hits->n + kUpdThreads - 1) / kUpdThreads)
-                                 : update_blocks(hits->n);
+                                 : list_update_blocks(hits->n, (uint32_t)c->upd_blocks);
     launch_update(a, c->cfg.key_dir, c->cfg.merge == GI_MERGE_WARP, blocks, st);
     s = cuda_status(cudaGetLastError(), "k_update launch");
     if (s == GI_OK) c->touched_since_resolve = true;
@@ -1604,7 +1626,9 @@ extern "C" gi_status gi_cell_means_noalloc(const gi_hits *hits, const gi_view *v
     a.route_trust = 0.0f;
     a.route_lod = 4u;
     const int ub = update_blocks(hits->n);
-    launch_update(a, key_dir, false, ub, st);
+    const uint32_t full = (uint32_t)((hits->n + kUpdThreads - 1) / kUpdThreads);
+    launch_update(a, key_dir, false,
+                  list_update_blocks(hits->n, resident_grid(k_update_list<0, false>, kUpdThreads, full)), st);
     s = cuda_status(cudaGetLastError(), "k_update launch");
     if (s != GI_OK) return s;
     const float e0 = env ? env[0] : 0.0f, e1 = env ? env[1] : 0.0f, e2 = env ? env[2] : 0.0f;
