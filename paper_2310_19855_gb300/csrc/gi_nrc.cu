@@ -1084,10 +1084,12 @@ __global__ void __launch_bounds__(32 * kAdamWarps, kAdamBlocksPerSm) k_nrc_adam(
 
 // ---------------------------------------------------------------- query selection
 
-// A block takes 64 words (2048 records) at a time: each warp decides its 8 words, the block's answered
+// A block takes 32 words (1024 records) at a time: each warp decides its 2 words, the block's answered
 // records take consecutive places with one addition to the counter (one addition per warp of 32
-// records, 64,800 at 1080p on one address, took 57 us, next to nothing of it the reads; now 29 us).
-constexpr int kSelWarps = 8, kSelWords = 8;
+// records, 64,800 at 1080p on one address, took 57 us).  What bounds a round is its chain of
+// dependent loads, so a warp reads the planes and slots of its words in one trip and the cells' cold
+// marks in a second: 17 us at 1080p and 5.1 us for 230,400 records, against 30 and 24 us word after word.
+constexpr int kSelWarps = 16, kSelWords = 2;
 __global__ void __launch_bounds__(32 * kSelWarps) k_nrc_select(SelectArgs a) {
     const uint32_t bid = blockIdx.x + pass_begin();
     __shared__ uint32_t s_cnt[kSelWarps], s_base;
@@ -1096,25 +1098,34 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_nrc_select(SelectArgs a) {
     const uint32_t words = (a.n + 31u) / 32u;
     for (uint32_t b0 = bid * (kSelWarps * kSelWords); b0 < words; b0 += gridDim.x * (kSelWarps * kSelWords)) {
         const uint32_t w0 = b0 + warp * kSelWords;
-        uint32_t ball[kSelWords], total = 0;
+        float len[kSelWords], px[kSelWords], py[kSelWords], pz[kSelWords];
+        uint32_t slot[kSelWords], ball[kSelWords], total = 0;
 #pragma unroll
         for (int k = 0; k < kSelWords; ++k) {
             const uint32_t r = (w0 + k) * 32u + lane;
-            bool use = false;
-            if (r < a.n && record_hit(a.pos, a.len, r)) {
-                const uint32_t slot = __ldca(a.slot_ids + r);
-                if (slot == GI_SLOT_FAR) {
-                    // left out of the table by the update (gi_cache_route_far): the network is its only answer
-                    use = true;
-                } else if (!trusted) {
-                } else if (slot == GI_SLOT_NONE) {
-                    use = true;
-                } else if (slot < a.cv.slots) {
-                    use = cache_cold(a.cv, slot) ||
-                          key_lod(a.kp, __ldca(a.pos[0] + r), __ldca(a.pos[1] + r), __ldca(a.pos[2] + r)) >= (int)a.query_lod;
-                }
+            len[k] = -1.0f;
+            px[k] = py[k] = pz[k] = 0.0f;
+            slot[k] = GI_SLOT_MISS;
+            if (r < a.n) {
+                len[k] = __ldca(a.len + r);
+                px[k] = __ldca(a.pos[0] + r);
+                py[k] = __ldca(a.pos[1] + r);
+                pz[k] = __ldca(a.pos[2] + r);
+                slot[k] = __ldca(a.slot_ids + r);
             }
-            ball[k] = __ballot_sync(0xFFFFFFFFu, use);
+        }
+        bool use[kSelWords];
+#pragma unroll
+        for (int k = 0; k < kSelWords; ++k) {
+            const bool hit = isfinite(len[k]) && len[k] >= 0.0f && isfinite(px[k]) && isfinite(py[k]) && isfinite(pz[k]);
+            // GI_SLOT_FAR: left out of the table by the update (gi_cache_route_far), the network is its only answer
+            use[k] = hit && (slot[k] == GI_SLOT_FAR || (trusted && slot[k] == GI_SLOT_NONE));
+            if (hit && trusted && slot[k] < a.cv.slots)
+                use[k] = cache_cold(a.cv, slot[k]) || key_lod(a.kp, px[k], py[k], pz[k]) >= (int)a.query_lod;
+        }
+#pragma unroll
+        for (int k = 0; k < kSelWords; ++k) {
+            ball[k] = __ballot_sync(0xFFFFFFFFu, use[k]);
             total += __popc(ball[k]);
         }
         if (lane == 0) s_cnt[warp] = total;
@@ -1133,9 +1144,9 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_nrc_select(SelectArgs a) {
 #pragma unroll
         for (int k = 0; k < kSelWords; ++k) {
             const uint32_t pos = base + __popc(ball[k] & ((1u << lane) - 1u));
-            const bool use = ((ball[k] >> lane) & 1u) && pos < a.max_q;
-            if (use) a.qidx[pos] = (w0 + k) * 32u + lane;
-            const uint32_t kept = __ballot_sync(0xFFFFFFFFu, use);
+            const bool take = ((ball[k] >> lane) & 1u) && pos < a.max_q;
+            if (take) a.qidx[pos] = (w0 + k) * 32u + lane;
+            const uint32_t kept = __ballot_sync(0xFFFFFFFFu, take);
             if (lane == 0 && w0 + k < words) a.bits[w0 + k] = kept;
             base += __popc(ball[k]);
         }
