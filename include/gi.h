@@ -92,7 +92,7 @@ typedef void *gi_stream_t; /* cudaStream_t */
  *                   a slot appends it to a list, staged per block), GI_FIRST_TOUCH_BITMAP (the
  *                   same without a returning addition, and a non-returning set of the slot's bit
  *                   in a bitmap of one bit per slot that the resolve walks in slot order; tables
- *                   of 2^22 slots and more keep the accumulators of recently touched cells side
+ *                   of 2^21 slots and more keep the accumulators of recently touched cells side
  *                   by side), or GI_FIRST_TOUCH_AUTO (the bitmap).  Results are identical.
  *   tiles           0: a slot holds one cell.  1: two-level cache of Section 2.2.3 ("Prefiltering
  *                   Radiance"): a slot holds a tile of 8 x 8 cells on the plane that drops the
@@ -252,7 +252,7 @@ uint32_t gi_version(void);
 /*
  * Create a cache (Section 2.2.1): allocates the slot table (fingerprints,
  * 32-byte fixed-point accumulators, resolved radiance), a spare table for
- * compaction (from 2^22 slots on the second set of accumulators serves recently touched cells
+ * compaction (from 2^21 slots on the second set of accumulators serves recently touched cells
  * instead, with 4 bytes of stamp per slot and table), the record of touched slots (a bitmap of one
  * bit per slot, or a touch list of 4 bytes per slot in the list form) and counters, on the
  * current CUDA device.  The library owns this memory until gi_cache_destroy.

@@ -308,11 +308,12 @@ static inline int list_update_blocks(unsigned long long n, uint32_t resident) {
 // entries per lane and iteration, 4 blocks per SM.  (1080p: the bitmap form 34 us, against 44 us
 // when a thread walked its own word's bits 4 at a time with 3 blocks per SM: a word holds 0 to 32
 // touched slots, so those threads' chains were as uneven as their words.)
-// Large tables start at 2^22 slots (128 MB of accumulators, the size of the L2): there the frame's
-// update fell from 62 to 55 us and its resolve stayed at 34 us; at 2^24 the update fell from 370 to
-// 281 us and the resolve from 135 to 97 us (both 1 ray a cell, 1080p and 4K).  At 2^20 and 2^21 slots
-// (16 views) the rank loads cost what the shorter span gave.
-constexpr uint32_t kDenseLog2Slots = 22, kDenseAge = 8;
+// Large tables start at 2^21 slots (64 MB of accumulators, half of the L2).  At 2^22 the frame's update
+// fell from 62 to 55 us and its resolve stayed at 34 us; at 2^24 the update fell from 370 to 281 us and
+// the resolve from 135 to 97 us (both 1 ray a cell, 1080p and 4K); at 2^21 the cache's calls on 777777
+// records fell from 71.2 to 66.0 us and 16 views of 2^20 and 2^21 slots from 1291 to 1248 us.  At 2^20 the rank
+// loads cost what the shorter span gives (the same calls at 1249 us).
+constexpr uint32_t kDenseLog2Slots = 21, kDenseAge = 8;
 constexpr int kResListUnroll = 2, kResListBlocksPerSm = 4;
 constexpr int kResBmUnroll = 2, kResBmBlocksPerSm = 4, kResBmWords = 16;
 // a table has at least 2^10 slots: its bitmap words are a whole number of chunks
