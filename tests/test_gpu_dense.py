@@ -77,3 +77,26 @@ def test_dense_accumulators_equal_the_list_form(log2, f16, merge, key_dir):
     finally:
         for h in caches:
             gi.gi_cache_destroy(h)
+
+
+@pytest.mark.parametrize("merge", [0, 1])
+@pytest.mark.parametrize("n", [1, 257, 233_472, 233_473, 1_867_776, 1_867_777])
+def test_list_form_of_any_count_equals_the_bitmap_form(n, merge):
+    # around one record a thread and 2048 records a block of a grid of 6 blocks on each of 152 SMs
+    rec = wl.records_random(n, 21, extent=30.0)
+    r = dev(rec)
+    caches = [gi.gi_cache_create(22, first_touch=ft, merge=merge, cell_size=0.05)
+              for ft in (gi.GI_FIRST_TOUCH_BITMAP, gi.GI_FIRST_TOUCH_LIST)]
+    try:
+        for h in caches:
+            s = torch.empty(n, dtype=torch.int32, device="cuda")
+            gi.gi_cache_update(h, gi.hits_from_planes(r, n), _view(0), s)
+        torch.cuda.synchronize()
+        _same(*caches)
+        for h in caches:
+            gi.gi_cache_resolve(h, 0)
+        torch.cuda.synchronize()
+        _same(*caches)
+    finally:
+        for h in caches:
+            gi.gi_cache_destroy(h)
