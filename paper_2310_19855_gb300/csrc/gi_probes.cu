@@ -971,7 +971,8 @@ __device__ __forceinline__ void interpolate_body(const InterpArgs &a, uint32_t b
             if (inb[h]) __stcs(a.out + pix[h], make_float4(0.f, 0.f, 0.f, (float)GI_INTERP_SKY));
         return;
     }
-    const bool other = lane >= 28 && tile && (qo >> 19 != (uint32_t)qy || (qo & 0xFFFFu) >> 3 != (uint32_t)qx);
+    const bool other = lane >= 28 && tile &&
+                       (qo == GI_PROBE_NONE || qo >> 19 != (uint32_t)qy || (qo & 0xFFFFu) >> 3 != (uint32_t)qx);
     if (__any_sync(kFullMask, other)) {
         uint32_t up = GI_PROBE_NONE;
         if (other) {
