@@ -66,3 +66,24 @@ def test_filter_of_a_view_without_probes_only_copies():
         if dist > 2.0:
             assert torch.equal(a, b)
     assert took[0] < 0.6 * took[1], took
+
+
+def test_more_rays_per_probe_cost_in_proportion():
+    # 641 x 359 pixels: 6.1 us with 64 rays per probe, 10.9 us with 128; 18.3 us where the gathers did not fly together
+    w, h = 641, 359
+    view = gi.make_view(0, w, h, (0, 0, 0), (0, 0, -1), (1, 0, 0), (0, 1, 0), 1.0)
+    gbuf = torch.tensor((0.0, 0.0, 1.0, 2.0), device="cuda").repeat(h, w, 1)
+    pb = ProbeBuffers(w, h)
+    gi.gi_probes_spawn(gi.make_gbuffer(gbuf, w, h), view, pb.struct)
+    n = pb.layout.num_probes * 128
+    rec = torch.rand((13, n), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda") * 6.0 - 3.0
+    rec[9] = 1.0
+    slots = torch.empty(n, dtype=torch.int32, device="cuda")
+    c = gi.gi_cache_create(20)
+    try:
+        gi.gi_cache_update(c, gi.hits_from_planes(rec, n), view, slots)
+        gi.gi_cache_resolve(c, 0)
+        t = [us(lambda: gi.gi_probes_integrate(c, pb.struct, slots, rpp), k=20) for rpp in (64, 128)]
+        assert t[1] < 2.3 * t[0], t
+    finally:
+        gi.gi_cache_destroy(c)
