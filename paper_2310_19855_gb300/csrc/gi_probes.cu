@@ -839,9 +839,11 @@ __device__ __forceinline__ void sh_lobe(float nx, float ny, float nz, float (&Yb
 
 // One pixel of the interpolation: weights of the four neighbours (bilinear x normal x plane
 // distance) and the weighted irradiance, or the relaxed / none / sky flags.  (fx, fy) is the
-// pixel's bilinear position between the neighbours, bit o of found says that neighbour o is there.  UNIFORM: the neighbours' irradiance and
-// plane and normal terms were evaluated once for the warp (s.eu, s.n8); otherwise each is
-// evaluated for this pixel's normal from the warp's shared copy.
+// pixel's bilinear position between the neighbours, bit o of found says that neighbour o is there.
+// UNIFORM: the neighbours' irradiance and plane and normal terms were evaluated once for the warp (s.eu,
+// s.n8); otherwise each is evaluated for this pixel's normal from the warp's shared copy, two neighbours'
+// at a time: a normal per pixel at 1080p 41.6 us one at a time, 40.0 two, and the batched kernel no longer
+// spills (16 views 1,256 us a frame, now 1,241); four spill.
 template <bool UNIFORM>
 __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb &s, int x, int y, float fx, float fy,
                                              const float4 nd, uint32_t pix, bool inb, bool act, unsigned found) {
@@ -863,7 +865,7 @@ __device__ __forceinline__ void interp_pixel(const InterpArgs &a, const InterpNb
     float Yb[9];
     if (!UNIFORM) sh_lobe(nx, ny, nz, Yb);
     float wsum = 0.f, es[3] = {0.f, 0.f, 0.f};
-#pragma unroll(UNIFORM ? 4 : 1)
+#pragma unroll(UNIFORM ? 4 : 2)
     for (int o = 0; o < 4; ++o) {
         if (!((found >> o) & 1u)) continue;
         float qn, n8, E[3];
