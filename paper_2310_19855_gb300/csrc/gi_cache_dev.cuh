@@ -50,6 +50,14 @@ __device__ __forceinline__ void warp_add_accum(Accum *accum, Accum *dense, uint3
     __syncwarp();
 }
 
+// Whether the warp's hits lie in at most half as many cells: every hit's cell (mix: any 32 bits that
+// name it) falls into one of 32 buckets, and the buckets taken are counted.  32 different cells take 20
+// of them (16 or fewer in 1 of 100 warps), k cells at most k.
+__device__ __forceinline__ bool warp_shares_cells(bool hit, uint32_t mix, unsigned hits) {
+    const uint32_t taken = __reduce_or_sync(kFull, hit ? 1u << ((mix * 2654435761u) >> 27) : 0u);
+    return 2 * __popc(taken) <= __popc(hits);
+}
+
 // Accumulator of a slot: the dense one where its rank word keeps it, else the slot's own.
 __device__ __forceinline__ uint32_t accum_loc(uint32_t keep, uint32_t base, uint32_t slot) {
     const uint32_t bit = 1u << (slot & 31u);

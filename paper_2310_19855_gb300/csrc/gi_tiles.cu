@@ -71,8 +71,12 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) { return a >
 // radiance, added into the cell's accumulator of its tile's block (warp_add_accum).  The accumulator
 // blocks of one frame are contiguous (touched tiles x 2 KB), so the reductions of a frame span
 // that range only, not the whole table: the cost of scattered reductions grows with the span.
-// Neither pass merges a warp's same-cell hits first: a probe's rays share few cells, and at 1080p
-// with 2x2 upscale the merge (__match_any_sync, pointer-jumping sums) cost 5 us of the frame.
+// Both merge a warp's same-cell hits first where the warp holds at most half as many cells as hits
+// (warp_shares_cells).  A probe's rays share few cells: at 1080p with 2x2 upscale merging every warp
+// (__match_any_sync, pointer-jumping sums) cost 5 us of the frame.  But unmerged additions to one address
+// follow one another: 1,000,000 records in one cell 1190 us, in eight 197 us, now 54 and 63 (merging every
+// warp 62 and 67; scattered records 83 so, 94 with every warp merged).  With a quarter instead of a half
+// 16 cells took 164 us for 82.
 template <int KEY_DIR>
 __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) {
     const uint32_t bid = blockIdx.x + pass_begin();
@@ -112,8 +116,13 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) 
                 tile_key(a.kp, px, py, pz, sx, sy, sz, len, KEY_DIR == GI_KEY_DIR_NORMAL ? 0u : 1u, cell);
             cell_of_key(key, a.mask, home, tag);
         }
+        // same cell = same (home, tag, cell); home < 2^22, so the cell fits above it
+        const unsigned hm = __ballot_sync(kFull, hit);
+        unsigned peers = 1u << lane;
+        const bool merge = warp_shares_cells(hit, tag ^ (cell << 8), hm);
+        if (merge && hit) peers = __match_any_sync(hm, ((unsigned long long)(home | (cell << 26)) << 32) | tag);
         uint32_t slot = GI_SLOT_NONE;
-        if (hit) {
+        if (hit && (peers & ((1u << lane) - 1u)) == 0u) {
             uint32_t s = home, k = 0;
             for (; k < a.max_probe; ++k) {
                 const uint32_t t = __ldcg(a.tags + s);
@@ -133,8 +142,9 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_key(TileUpdateArgs ta) 
             }
             my_maxp = max(my_maxp, k + 1u);
             if (slot != GI_SLOT_NONE) atomicOr(ta.tmask + slot, 1ull << cell);
-            else ++my_dropped;
+            else my_dropped += (unsigned long long)__popc(peers);
         }
+        if (merge) slot = __shfl_sync(kFull, slot, hit ? (__ffs(peers) - 1) : lane);
         uint32_t id = miss ? GI_SLOT_MISS : GI_SLOT_NONE;
         if (slot != GI_SLOT_NONE) id = slot * kTileCells + cell;
         if (hit && slot == GI_SLOT_NONE) {
@@ -228,13 +238,38 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_tile_accumulate(const uint32
         ok = ok && blk < cells / kTileCells;
         // {r, g, b, count} of the hit, four lanes per record (the stamp half of the last word is unused
         // in the blocks)
+        const unsigned vm = __ballot_sync(kFull, ok);
+        uint32_t cnt = 1u;
+        if (warp_shares_cells(ok, id, vm)) {
+            // pointer jumping from each hit to the next one of its cell: the first gets the cell's sums
+            unsigned peers = 0;
+            if (ok) peers = __match_any_sync(vm, id);
+            const unsigned above = peers & (0xFFFFFFFEu << lane);
+            int nxt = above ? (__ffs(above) - 1) : -1;
+            while (__any_sync(kFull, nxt >= 0)) {
+                const int src = nxt >= 0 ? nxt : lane;
+                const unsigned long long o0 = __shfl_sync(kFull, q0, src);
+                const unsigned long long o1 = __shfl_sync(kFull, q1, src);
+                const unsigned long long o2 = __shfl_sync(kFull, q2, src);
+                const uint32_t oc = __shfl_sync(kFull, cnt, src);
+                const int on = __shfl_sync(kFull, nxt, src);
+                if (nxt >= 0) {
+                    q0 += o0;
+                    q1 += o1;
+                    q2 += o2;
+                    cnt += oc;
+                    nxt = on;
+                }
+            }
+            ok = ok && (peers & ((1u << lane) - 1u)) == 0u;
+        }
         uint32_t loc = GI_SLOT_NONE;
         if (ok) {
             loc = blk * kTileCells + (id % kTileCells);
             s_red[threadIdx.x][0] = q0;
             s_red[threadIdx.x][1] = q1;
             s_red[threadIdx.x][2] = q2;
-            s_red[threadIdx.x][3] = 1ull;
+            s_red[threadIdx.x][3] = cnt;
         }
         warp_add_accum(accum, nullptr, loc, &s_red[threadIdx.x & ~31u][0], lane);
     }
