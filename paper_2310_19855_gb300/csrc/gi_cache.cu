@@ -98,7 +98,8 @@ __device__ __forceinline__ uint32_t probe_cell(const UpdateArgs &a, uint32_t hom
 // different directions, so few of them share a cell: at 1080p the merge cost 9 us of the update
 // for ~5 % fewer reductions (update 72 us with it, 63 us without), and on the Cornell box at
 // 1080p 41 us against 38 us.  It stays available (GI_MERGE_WARP) for workloads whose warps do hit
-// the same cells.
+// the same cells, and then merges the warps that hold at most half as many cells as hits (1,000,000
+// scattered records over 2^20 slots: 74 us with every warp, 59 us so; all in one cell 33 and 35 us).
 // s_acc: one 32-byte slot per thread; s_touch: the block's first touches (list form only, else NULL).
 template <int KEY_DIR, bool MERGE, bool BITMAP>
 __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, uint32_t nblk,
@@ -150,13 +151,11 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
             q1 = quantize(r1, bad);
             q2 = quantize(r2, bad);
             my_clamped += bad;
-            if (!MERGE) {
-                // the contribution waits in shared memory while the probe runs
-                s_red[0] = q0;
-                s_red[1] = q1;
-                s_red[2] = q2;
-                s_red[3] = 1ull;
-            }
+            // the contribution waits in shared memory while the probe runs
+            s_red[0] = q0;
+            s_red[1] = q1;
+            s_red[2] = q2;
+            s_red[3] = 1ull;
             unsigned long long key =
                 cell_key(a.kp, px, py, pz, sx, sy, sz, len, KEY_DIR == GI_KEY_DIR_NORMAL ? 0u : 1u);
             cell_of_key(key, a.mask, home, tag);
@@ -168,9 +167,10 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
         }
         uint32_t cnt = hit ? 1u : 0u;
         unsigned peers = 1u << lane;
-        if (MERGE) {
+        const unsigned hm = MERGE ? __ballot_sync(kFull, hit) : 0u;
+        const bool merge = MERGE && warp_shares_cells(hit, home ^ tag, hm);
+        if (merge) {
             // one leader per cell adds the group's integer sums (order-independent, so still bit-exact)
-            const unsigned hm = __ballot_sync(kFull, hit);
             if (hit) peers = __match_any_sync(hm, ((unsigned long long)home << 32) | tag);
             const unsigned above = peers & (0xFFFFFFFEu << lane);
             int nxt = above ? (__ffs(above) - 1) : -1;
@@ -190,12 +190,10 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
                     nxt = on;
                 }
             }
-            if (BITMAP) {
-                s_red[0] = q0;
-                s_red[1] = q1;
-                s_red[2] = q2;
-                s_red[3] = cnt;
-            }
+            s_red[0] = q0;
+            s_red[1] = q1;
+            s_red[2] = q2;
+            s_red[3] = cnt;
         }
         const bool leader = hit && (peers & ((1u << lane) - 1u)) == 0u;
         uint32_t slot = GI_SLOT_NONE, loc = GI_SLOT_NONE;
@@ -220,9 +218,9 @@ __device__ __forceinline__ void update_body(const UpdateArgs &a, uint32_t blk, u
             }
         }
         uint32_t my_slot = slot;
-        if (MERGE) my_slot = __shfl_sync(kFull, slot, hit ? (__ffs(peers) - 1) : lane);
+        if (merge) my_slot = __shfl_sync(kFull, slot, hit ? (__ffs(peers) - 1) : lane);
         if (inr) __stcs(a.slot_ids + i, hit ? my_slot : code);
-        if (MERGE && !BITMAP) {
+        if (merge && !BITMAP) {
             // few leaders are left, and each waits for its own count: four lanes a record would add the
             // trips of the other leaders (the calls on 1,000,000 records: 138.5 us so, 127.5 us like this)
             if (loc != GI_SLOT_NONE) {
@@ -1107,7 +1105,8 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
     }
     if (s == GI_OK) {
         int per_sm = 0;
-        s = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<0, false>, kUpdThreads, 0),
+        s = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                            &per_sm, cfg->merge == GI_MERGE_WARP ? k_update<0, true> : k_update<0, false>, kUpdThreads, 0),
                         "occupancy");
         c->upd_blocks = c->sms * (c->touch ? kUpdListBlocksPerSm : std::max(per_sm, 1));
         c->res_blocks = c->sms * (c->touch ? kResListBlocksPerSm : kResBmBlocksPerSm);
