@@ -316,6 +316,13 @@ constexpr int kResListUnroll = 2, kResListBlocksPerSm = 4;
 constexpr int kResBmUnroll = 2, kResBmBlocksPerSm = 4, kResBmWords = 16;
 // a table has at least 2^10 slots: its bitmap words are a whole number of chunks
 static_assert(((1u << 10) / 32u) % kResBmWords == 0, "bitmap chunk must divide the smallest table");
+// Large tables (resolve_dense_body): rank words of a block's share at most and at least, slots listed at a
+// time, and the accumulators that a share's hand-out is rounded up to.
+constexpr uint32_t kDenseWords = 512, kDenseMinWords = 64, kDenseList = 2048, kDenseAlign = 32;
+static_assert(kDenseWords % kResThreads == 0 && kDenseWords * 32 <= 1u << 15, "a share's counts take 16 bits each");
+
+// The slots of a rank word that keep a dense accumulator through this resolve.
+__device__ __forceinline__ uint32_t kept(bool age, const uint4 &rk) { return age ? (rk.w | rk.z) : (rk.x | rk.z); }
 
 // Resolve one touched slot whose accumulator (lo, hi) and resolved history (old) are loaded:
 // mean = sum / (count 2^24); a cell without history (never resolved, or evicted by an earlier
@@ -391,55 +398,35 @@ __device__ __forceinline__ void resolve_list_body(const ResolveArgs &a, uint32_t
 // slots of their set bits in slot order to its shared list (a prefix sum of the words' bit counts
 // over the lanes gives each lane its place) and resolves the list U entries per lane at a time:
 // every lane gets the same share of the warp's touched slots whatever the words hold.
-// DENSE: the accumulators of the cells in the chunk's rank words lie side by side (warp after warp in
-// the order the previous resolve handed them out), the stamps in an array of their own; the cells
-// touched lately (not since one to two aging periods) get the next dense accumulators.
-template <int U, bool DENSE>
+template <int U>
 __device__ __forceinline__ void resolve_bm_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
     __shared__ uint16_t s_list[kResThreads / 32][kResBmWords * 32];
-    __shared__ uint32_t s_loc[DENSE ? kResThreads / 32 : 1][DENSE ? kResBmWords * 32 : 1];
-    __shared__ uint32_t s_cold[DENSE ? kResThreads / 32 : 1][kResBmWords];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nw = nblk * (kResThreads / 32);
     const uint32_t chunks = a.words / kResBmWords;
     uint32_t fresh_new = 0;
-    // accumulators by slot leave the L2 first, resolved values last: the probe pass reads them next
+    // accumulators leave the L2 first, resolved values last: the probe pass reads them next
     const unsigned long long pfirst = l2_policy_evict_first(), plast = l2_policy_evict_last();
     for (uint32_t c = blk * (kResThreads / 32) + warp; c < chunks; c += nw) {
         const uint32_t wi = c * kResBmWords + lane, slot0 = c * (kResBmWords * 32);
-        const bool mine = lane < kResBmWords;
-        uint4 rk = make_uint4(0u, 0u, 0u, 0u);
-        uint32_t cold = 0;
-        if (DENSE && mine) {
-            rk = __ldcg(reinterpret_cast<const uint4 *>(a.rank + wi));
-            cold = __ldcg(a.cold + wi) & ~rk.z;  // of the untouched cells
-            s_cold[warp][lane] = 0u;
-        }
-        uint32_t bits = DENSE ? rk.z : (mine ? __ldcg(a.bitmap + wi) : 0u);
-        if (!DENSE && bits) a.bitmap[wi] = 0u;
-        const uint32_t recent = rk.w | bits, keep = a.age ? recent : (rk.x | bits);
-        const int cnt = __popc(bits), kcnt = DENSE ? __popc(keep) : 0;
-        int incl = cnt | (kcnt << 16);  // both prefix sums at once (at most 512 each)
+        uint32_t bits = lane < kResBmWords ? __ldcg(a.bitmap + wi) : 0u;
+        if (bits) a.bitmap[wi] = 0u;
+        const int cnt = __popc(bits);
+        int incl = cnt;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const int t = __shfl_up_sync(kFull, incl, d);
             if (lane >= d) incl += t;
         }
-        const int totals = __shfl_sync(kFull, incl, 31);
-        const int total = totals & 0xFFFF;
-        uint32_t base = 0;
-        if (DENSE && lane == 0 && (totals >> 16)) base = atomicAdd(&a.ctr->dense_next, (uint32_t)(totals >> 16));
-        int pos = (incl & 0xFFFF) - cnt;
+        const int total = __shfl_sync(kFull, incl, 31);
+        int pos = incl - cnt;
         while (bits) {
-            const uint32_t b = (uint32_t)(__ffs(bits) - 1);
-            s_list[warp][pos] = (uint16_t)(32u * lane + b);
-            if (DENSE) s_loc[warp][pos] = accum_loc(rk.x, rk.y, wi * 32u + b);
-            ++pos;
+            s_list[warp][pos++] = (uint16_t)(32u * lane + (uint32_t)(__ffs(bits) - 1));
             bits &= bits - 1u;
         }
         __syncwarp();
         for (int k = lane; k < total; k += 32 * U) {
-            uint32_t s[U], loc[U], stamp[U];
+            uint32_t s[U];
             uint4 lo[U], hi[U];
             float3 old[U];
 #pragma unroll
@@ -448,53 +435,21 @@ __device__ __forceinline__ void resolve_bm_body(const ResolveArgs &a, uint32_t b
                 s[u] = 0xFFFFFFFFu;
                 if (idx < total) {
                     s[u] = slot0 + s_list[warp][idx];
-                    if (DENSE) {
-                        loc[u] = s_loc[warp][idx];
-                        const uint4 *src = reinterpret_cast<const uint4 *>(accum_at(a.accum, a.dense, loc[u]));
-                        lo[u] = __ldcg(src);
-                        hi[u] = __ldcg(src + 1);
-                    } else {
-                        const uint4 *src = reinterpret_cast<const uint4 *>(a.accum + s[u]);
-                        lo[u] = ld_cg_hint(src, pfirst);
-                        hi[u] = ld_cg_hint(src + 1, pfirst);
-                        stamp[u] = hi[u].w;
-                    }
+                    const uint4 *src = reinterpret_cast<const uint4 *>(a.accum + s[u]);
+                    lo[u] = ld_cg_hint(src, pfirst);
+                    hi[u] = ld_cg_hint(src + 1, pfirst);
                     // the history is read speculatively: a cell without one ignores it
-                    if (DENSE && !a.f16) {
-                        const float4 v = __ldcg(static_cast<const float4 *>(a.resolved) + s[u]);
-                        old[u] = make_float3(v.x, v.y, v.z);
-                        stamp[u] = __float_as_uint(v.w);
-                    } else {
-                        if (DENSE) stamp[u] = __ldcg(a.stamps + s[u]);
-                        old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
-                    }
+                    old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
                 }
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (s[u] == 0xFFFFFFFFu) continue;
-                const bool fresh = resolve_cell<DENSE>(a, s[u], stamp[u], lo[u], hi[u], old[u], plast, fresh_new);
-                if (DENSE) {
-                    if (fresh) atomicOr(&s_cold[warp][(s[u] >> 5) % kResBmWords], 1u << (s[u] & 31u));
-                    uint4 *dst = reinterpret_cast<uint4 *>(accum_at(a.accum, a.dense, loc[u]));
-                    dst[0] = make_uint4(0u, 0u, 0u, 0u);
-                    dst[1] = make_uint4(0u, 0u, 0u, 0u);
-                    if (a.f16) a.stamps[s[u]] = a.stamp_now;
-                } else {
-                    // the cleared accumulator is next read by the next frame's update
-                    uint4 *dst = reinterpret_cast<uint4 *>(a.accum + s[u]);
-                    st_hint(dst, make_uint4(0u, 0u, 0u, 0u), pfirst);
-                    st_hint(dst + 1, make_uint4(0u, 0u, 0u, a.stamp_now), pfirst);
-                }
-            }
-        }
-        if (DENSE) {
-            __syncwarp();
-            base = __shfl_sync(kFull, base, 0);
-            if (mine) {
-                *reinterpret_cast<uint4 *>(a.rank + wi) =
-                    make_uint4(keep, base + (uint32_t)((incl >> 16) - kcnt), 0u, a.age ? 0u : recent);
-                if (rk.z) a.cold[wi] = cold | s_cold[warp][lane];
+                resolve_cell<false>(a, s[u], hi[u].w, lo[u], hi[u], old[u], plast, fresh_new);
+                // the cleared accumulator is next read by the next frame's update
+                uint4 *dst = reinterpret_cast<uint4 *>(a.accum + s[u]);
+                st_hint(dst, make_uint4(0u, 0u, 0u, 0u), pfirst);
+                st_hint(dst + 1, make_uint4(0u, 0u, 0u, a.stamp_now), pfirst);
             }
         }
         __syncwarp();
@@ -502,12 +457,167 @@ __device__ __forceinline__ void resolve_bm_body(const ResolveArgs &a, uint32_t b
     resolve_finish(a.ctr, a.occ_out, a.stamp_now, nw, fresh_new);
 }
 
+// Large tables: a block takes its share of the rank words (all of it at once where it fits).  Its threads load
+// the words together, list the touched slots in shared memory and resolve the list U entries per thread at a
+// time.  The accumulators of the kept cells lie side by side in the order in which the previous resolve
+// handed them out; the cells touched lately (not since one to two aging periods) get the next dense
+// accumulators, with one addition to the counter per share, and the table's ticket is one per block: additions
+// to one address follow one another at 0.88 ns.  (An addition per 512 slots: the calls on 65,536 records
+// took 21 us over 2^22 slots, 37 over 2^24 and 62 over 2^26, now 16, 22 and 31; the resolve of 429,000 cells
+// of 2^22 slots 23 us, now 18.)  What bounds it is the chain of a share: words, list, cells, words back.
+// A hand-out starts on a multiple of kDenseAlign accumulators (1 KB), so that the few cells of a concentrated
+// frame do not meet in the same lines: a million records on 8 cells of 2^22 slots took 526 us without, 92 with.
+// Shares are short because the next pass is scheduled beside this one and has the L1 that this one's shared
+// memory leaves: with room for 1024 words and 8192 listed slots (38 KB a block) the 1080p frame took 144 us,
+// with 15 KB 134.  Shares of 256 words are the faster ones where most words hold a cell (4K frame 594 us
+// against 599 with 512), of 512 where a block has many shares and few cells in each (65,536 records over 2^26
+// slots: 44 us with 256, 30 with 512): tables of 2^25 slots and more take those.
+template <int U>
+__device__ __forceinline__ void resolve_dense_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
+    constexpr int W = kResThreads / 32, J = kDenseWords / kResThreads;
+    __shared__ uint4 s_rk[kDenseWords];
+    __shared__ uint32_t s_cold[kDenseWords];
+    __shared__ uint16_t s_list[kDenseList];  // slots from the share's first on
+    __shared__ uint32_t s_sum[W], s_before[kResThreads], s_base;
+    const uint32_t t = threadIdx.x;
+    const int warp = t >> 5, lane = t & 31;
+    uint32_t fresh_new = 0;
+    // resolved values leave the L2 last: the probe pass reads them next
+    const unsigned long long plast = l2_policy_evict_last();
+    const bool age = a.age != 0u;
+    const uint32_t cap = a.words >= 1u << 20 ? kDenseWords : kDenseWords / 2;
+    const uint32_t per = (a.words + nblk - 1u) / nblk, parts = (per + cap - 1u) / cap;
+    const uint32_t share = max(kDenseMinWords, (per + parts - 1u) / parts);
+    for (uint32_t first = blk * share; first < a.words; first += nblk * share) {
+        const uint32_t n = min(share, a.words - first);
+        uint32_t sums = 0, cold[J];  // touched slots | kept slots << 16, at most 2^15 of each in a share
+        {
+            uint4 rk[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                rk[j] = make_uint4(0u, 0u, 0u, 0u);
+                cold[j] = 0u;
+                if (t + j * kResThreads < n) {
+                    rk[j] = __ldcg(reinterpret_cast<const uint4 *>(a.rank) + first + t + j * kResThreads);
+                    cold[j] = __ldcg(a.cold + first + t + j * kResThreads);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                cold[j] &= ~rk[j].z;  // of the untouched cells
+                s_rk[t + j * kResThreads] = rk[j];
+                sums += (uint32_t)__popc(rk[j].z) + ((uint32_t)__popc(kept(age, rk[j])) << 16);
+            }
+        }
+        uint32_t incl = sums;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t v = __shfl_up_sync(kFull, incl, d);
+            if (lane >= d) incl += v;
+        }
+        if (lane == 31) s_sum[warp] = incl;
+        __syncthreads();
+        uint32_t before = incl - sums, total = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const uint32_t v = s_sum[w];
+            before += w < warp ? v : 0u;
+            total += v;
+        }
+        s_before[t] = before >> 16;
+        uint32_t base = 0;
+        if (t == 0 && (total >> 16))
+            base = atomicAdd(&a.ctr->dense_next, ((total >> 16) + kDenseAlign - 1u) & ~(kDenseAlign - 1u));
+        const uint32_t touched = total & 0xFFFFu;
+        for (uint32_t win = 0; win < touched; win += kDenseList) {
+            if (win) __syncthreads();  // the list's last window has been resolved
+            uint32_t pos = (before & 0xFFFFu) - win;
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const uint32_t w = t + j * kResThreads;
+                uint32_t bits = w < n ? s_rk[w].z : 0u;
+                if (win == 0) s_cold[w] = cold[j];
+                while (bits) {
+                    if (pos < kDenseList) s_list[pos] = (uint16_t)(32u * w + (uint32_t)(__ffs(bits) - 1));
+                    ++pos;
+                    bits &= bits - 1u;
+                }
+            }
+            __syncthreads();
+            const uint32_t listed = min(touched - win, (uint32_t)kDenseList);
+            for (uint32_t k = t; k < listed; k += U * kResThreads) {
+                uint32_t s[U], loc[U], stamp[U];
+                uint4 lo[U], hi[U];
+                float3 old[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    s[u] = 0xFFFFFFFFu;
+                    if (k + u * kResThreads < listed) {
+                        const uint32_t o = s_list[k + u * kResThreads];
+                        const uint2 rk = *reinterpret_cast<const uint2 *>(&s_rk[o >> 5]);
+                        s[u] = 32u * first + o;
+                        loc[u] = accum_loc(rk.x, rk.y, s[u]);
+                        const uint4 *src = reinterpret_cast<const uint4 *>(accum_at(a.accum, a.dense, loc[u]));
+                        lo[u] = __ldcg(src);
+                        hi[u] = __ldcg(src + 1);
+                        // the history is read speculatively: a cell without one ignores it
+                        if (!a.f16) {
+                            const float4 v = __ldcg(static_cast<const float4 *>(a.resolved) + s[u]);
+                            old[u] = make_float3(v.x, v.y, v.z);
+                            stamp[u] = __float_as_uint(v.w);
+                        } else {
+                            stamp[u] = __ldcg(a.stamps + s[u]);
+                            old[u] = load_resolved(a.resolved, a.res_stride, a.f16, s[u]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (s[u] == 0xFFFFFFFFu) continue;
+                    const bool fresh = resolve_cell<true>(a, s[u], stamp[u], lo[u], hi[u], old[u], plast, fresh_new);
+                    if (fresh) atomicOr(&s_cold[(s[u] >> 5) - first], 1u << (s[u] & 31u));
+                    uint4 *dst = reinterpret_cast<uint4 *>(accum_at(a.accum, a.dense, loc[u]));
+                    dst[0] = make_uint4(0u, 0u, 0u, 0u);
+                    dst[1] = make_uint4(0u, 0u, 0u, 0u);
+                    if (a.f16) a.stamps[s[u]] = a.stamp_now;
+                }
+            }
+        }
+        if (t == 0) s_base = base;
+        __syncthreads();
+        base = s_base + s_before[t];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t w = t + j * kResThreads;
+            if (w < n) {
+                const uint4 rk = s_rk[w];
+                if (rk.x | rk.z) {
+                    const uint32_t keep = kept(age, rk);
+                    *(reinterpret_cast<uint4 *>(a.rank) + first + w) = make_uint4(keep, base, 0u, age ? 0u : rk.w | rk.z);
+                    base += (uint32_t)__popc(keep);
+                    if (rk.z) a.cold[first + w] = s_cold[w];
+                }
+            }
+        }
+    }
+    // a part per block: the warps end together here, and a ticket each would follow one another
+    fresh_new = __reduce_add_sync(kFull, fresh_new);
+    if (lane == 0) s_sum[warp] = fresh_new;
+    __syncthreads();
+    if (t == 0) {
+        fresh_new = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) fresh_new += s_sum[w];
+        resolve_part_done(a.ctr, a.occ_out, a.stamp_now, nblk, fresh_new);
+    }
+}
+
 // DENSE: some view of the batch has a large table (a batch without one keeps clear of that form's
 // registers, which spill beside the others').
 template <bool DENSE>
 __device__ __forceinline__ void resolve_body(const ResolveArgs &a, uint32_t blk, uint32_t nblk) {
-    if (DENSE && a.rank) resolve_bm_body<1, true>(a, blk, nblk);
-    else if (a.bitmap) resolve_bm_body<kResBmUnroll, false>(a, blk, nblk);
+    if (DENSE && a.rank) resolve_dense_body<1>(a, blk, nblk);
+    else if (a.bitmap) resolve_bm_body<kResBmUnroll>(a, blk, nblk);
     else resolve_list_body<kResListUnroll>(a, blk, nblk);
 }
 
@@ -517,11 +627,11 @@ __global__ void __launch_bounds__(kResThreads, kResListBlocksPerSm) k_resolve(Re
 }
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_bitmap(ResolveArgs a) {
     const uint32_t bid = blockIdx.x + pass_begin();
-    resolve_bm_body<kResBmUnroll, false>(a, bid, gridDim.x);
+    resolve_bm_body<kResBmUnroll>(a, bid, gridDim.x);
 }
 __global__ void __launch_bounds__(kResThreads, kResBmBlocksPerSm) k_resolve_dense(ResolveArgs a) {
     const uint32_t bid = blockIdx.x + pass_begin();
-    resolve_bm_body<kResBmUnroll, true>(a, bid, gridDim.x);
+    resolve_dense_body<kResBmUnroll>(a, bid, gridDim.x);
 }
 
 // ---------------------------------------------------------------- queries
@@ -776,6 +886,8 @@ static uint32_t stamp_stride(const gi_cache_s *c) {
     if (!c->rank) return (uint32_t)(sizeof(Accum) / sizeof(uint32_t));
     return c->stamp[0] ? 1u : 4u;
 }
+// Dense accumulators: one per slot, and what the shares' hand-outs (at least kDenseMinWords words each) round up.
+static size_t dense_entries(size_t slots) { return slots + (slots / 32 / kDenseMinWords + 1) * kDenseAlign; }
 // The accumulators by slot: one array for both tables where the stamps lie elsewhere.
 static Accum *accum_of(const gi_cache_s *c) { return c->accum[c->accum[1] ? c->cur : 0]; }
 
@@ -1082,8 +1194,8 @@ gi_status gi_cache_create(const gi_cache_config *cfg, gi_cache_t *out) {
     if (s == GI_OK && use_dense) {
         s = cuda_status(cudaMalloc(&c->rank, N / 32 * sizeof(RankWord)), "cudaMalloc rank");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->rank, 0, N / 32 * sizeof(RankWord)), "memset");
-        if (s == GI_OK) s = cuda_status(cudaMalloc(&c->dense, N * sizeof(Accum)), "cudaMalloc dense accumulators");
-        if (s == GI_OK) s = cuda_status(cudaMemset(c->dense, 0, N * sizeof(Accum)), "memset");
+        if (s == GI_OK) s = cuda_status(cudaMalloc(&c->dense, dense_entries(N) * sizeof(Accum)), "cudaMalloc dense accumulators");
+        if (s == GI_OK) s = cuda_status(cudaMemset(c->dense, 0, dense_entries(N) * sizeof(Accum)), "memset");
     } else if (s == GI_OK && use_bitmap) {
         s = cuda_status(cudaMalloc(&c->bitmap, N / 8), "cudaMalloc bitmap");
         if (s == GI_OK) s = cuda_status(cudaMemset(c->bitmap, 0, N / 8), "memset");
@@ -1361,11 +1473,12 @@ gi_status gi_cache_export(gi_cache_t c, gi_cell *out, uint64_t capacity, uint64_
     if (s == GI_OK && c->rank) {
         // large tables: a cell with a dense accumulator takes its sums from there, every cell its stamp
         std::vector<RankWord> rank(N / 32);
-        std::vector<Accum> dense(N);
+        const size_t D = dense_entries(N);
+        std::vector<Accum> dense(D);
         const uint32_t ss = stamp_stride(c);
         std::vector<uint32_t> stamp(ss == 1u ? N : 0);
         s = cuda_status(cudaMemcpy(rank.data(), c->rank, N / 32 * sizeof(RankWord), cudaMemcpyDeviceToHost), "export");
-        if (s == GI_OK) s = cuda_status(cudaMemcpy(dense.data(), c->dense, N * sizeof(Accum), cudaMemcpyDeviceToHost), "export");
+        if (s == GI_OK) s = cuda_status(cudaMemcpy(dense.data(), c->dense, D * sizeof(Accum), cudaMemcpyDeviceToHost), "export");
         if (s == GI_OK && ss == 1u)
             s = cuda_status(cudaMemcpy(stamp.data(), c->stamp[c->cur], N * sizeof(uint32_t), cudaMemcpyDeviceToHost), "export");
         for (size_t i = 0; i < N && s == GI_OK; ++i) {

@@ -186,28 +186,31 @@ __device__ __forceinline__ bool answers(uint32_t stamp, const LiveRule &r) {
     return stamp != 0u && (!r.has_lr || (r.lr - (stamp - 1u)) < r.evict);
 }
 
-// Newly occupied slots added per warp, then the last warp to finish (a ticket over all nwarps
-// warps of the launch) resets the touch count and publishes the occupancy, followed by the frame it
-// belongs to, to host-mapped memory.  No block barrier: a warp never waits for the others.
+// One of `parts` parts of a resolve is done (its thread calls): newly occupied slots added, then the last
+// part (a ticket) resets the touch count and publishes the occupancy, followed by the frame it belongs to,
+// to host-mapped memory.
+__device__ __forceinline__ void resolve_part_done(Counters *ctr, uint32_t *occ_out, uint32_t stamp_now, uint32_t parts,
+                                                  uint32_t fresh_new) {
+    if (fresh_new) atomicAdd(&ctr->occupied, fresh_new);
+    __threadfence();
+    if (atomicAdd(&ctr->ticket, 1u) == parts - 1u) {
+        // every part has read the touch count: reset it for the next frame
+        ctr->touch_count = 0u;
+        ctr->ticket = 0u;
+        ctr->dense_next = 0u;
+        // occupancy for the host's compaction decision, then the frame it belongs to
+        if (occ_out) {
+            reinterpret_cast<volatile uint32_t *>(occ_out)[0] = atomicAdd(&ctr->occupied, 0u);
+            __threadfence_system();
+            reinterpret_cast<volatile uint32_t *>(occ_out)[1] = stamp_now;
+        }
+    }
+}
+// A part per warp: no block barrier, a warp never waits for the others.
 __device__ __forceinline__ void resolve_finish(Counters *ctr, uint32_t *occ_out, uint32_t stamp_now, uint32_t nwarps,
                                                uint32_t fresh_new) {
     fresh_new = __reduce_add_sync(kFull, fresh_new);
-    if ((threadIdx.x & 31) == 0) {
-        if (fresh_new) atomicAdd(&ctr->occupied, fresh_new);
-        __threadfence();
-        if (atomicAdd(&ctr->ticket, 1u) == nwarps - 1u) {
-            // every warp has read the touch count: reset it for the next frame
-            ctr->touch_count = 0u;
-            ctr->ticket = 0u;
-            ctr->dense_next = 0u;
-            // occupancy for the host's compaction decision, then the frame it belongs to
-            if (occ_out) {
-                reinterpret_cast<volatile uint32_t *>(occ_out)[0] = atomicAdd(&ctr->occupied, 0u);
-                __threadfence_system();
-                reinterpret_cast<volatile uint32_t *>(occ_out)[1] = stamp_now;
-            }
-        }
-    }
+    if ((threadIdx.x & 31) == 0) resolve_part_done(ctr, occ_out, stamp_now, nwarps, fresh_new);
 }
 
 } // namespace gi
