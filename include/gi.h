@@ -791,6 +791,12 @@ gi_status gi_cell_means_noalloc(const gi_hits *hits, const gi_view *view, float 
 gi_status gi_diag_update_atomics(const uint32_t *slot_ids, uint64_t n, uint32_t log2_slots, uint32_t first_touch,
                                  void *scratch, uint32_t *first_touches, gi_stream_t stream);
 
+/*
+ * Number of cells of a bitmap-form table of 2^21 slots and more that hold a side-by-side accumulator (the
+ * cells touched in the last 8 to 16 resolves); 0 for other tables.  Synchronous.
+ * Errors: GI_ERR_INVALID_ARG (NULL argument), GI_ERR_CUDA. */
+gi_status gi_diag_dense_cells(gi_cache_t cache, uint64_t *cells, gi_stream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -209,6 +209,7 @@ def lib() -> ctypes.CDLL:
                                                        ctypes.POINTER(c_f32), c_vp]),
             "gi_nrc_stats": (ctypes.c_int, [c_vp, ctypes.POINTER(gi_nrc_stats_t), c_vp]),
             "gi_diag_update_atomics": (ctypes.c_int, [c_vp, c_u64, c_u32, c_u32, c_vp, c_vp, c_vp]),
+            "gi_diag_dense_cells": (ctypes.c_int, [c_vp, ctypes.POINTER(c_u64), c_vp]),
         }
         for name, (res, args) in sig.items():
             f = getattr(L, name)
@@ -450,6 +451,13 @@ def gi_diag_update_atomics(slot_ids, n: int, log2_slots: int, scratch, first_tou
     bitmap form 2^log2_slots / 8 bytes of bitmap); first_touches: device uint32 counter (list form)."""
     check(lib().gi_diag_update_atomics(_ptr(slot_ids), int(n), int(log2_slots), int(first_touch), _ptr(scratch),
                                        _ptr(first_touches), _stream(stream)), "gi_diag_update_atomics")
+
+
+def gi_diag_dense_cells(cache: int, stream=None) -> int:
+    """Diagnostics (see gi.h): the cells of a large bitmap-form table with a side-by-side accumulator."""
+    n = c_u64()
+    check(lib().gi_diag_dense_cells(cache, ctypes.byref(n), _stream(stream)), "gi_diag_dense_cells")
+    return n.value
 
 
 def gi_batch_create(n_views: int, rays_per_probe: int, tuning: gi_batch_tuning | None = None) -> int:

@@ -484,7 +484,8 @@ __device__ __forceinline__ void resolve_dense_body(const ResolveArgs &a, uint32_
     uint32_t fresh_new = 0;
     // resolved values leave the L2 last: the probe pass reads them next
     const unsigned long long plast = l2_policy_evict_last();
-    const bool age = a.age != 0u;
+    // every kDenseAge-th resolve, counted on the device, so that a captured one ages too
+    const bool age = ld(&a.ctr->resolves) % kDenseAge == kDenseAge - 1u;
     const uint32_t cap = a.words >= 1u << 20 ? kDenseWords : kDenseWords / 2;
     const uint32_t per = (a.words + nblk - 1u) / nblk, parts = (per + cap - 1u) / cap;
     const uint32_t share = max(kDenseMinWords, (per + parts - 1u) / parts);
@@ -1008,9 +1009,8 @@ ResolveArgs cache_resolve_args(gi_cache_s *c, uint32_t frame) {
     a.accum = accum_of(c);
     a.dense = c->dense;
     a.rank = c->rank;
-    a.age = c->resolves % kDenseAge == kDenseAge - 1 ? 1u : 0u;
-    a.stamps = c->stamp[c->cur];
     a.cold = c->cold[c->cur];
+    a.stamps = c->stamp[c->cur];
     a.resolved = c->resolved[c->cur];
     a.res_stride = c->res_bytes;
     a.ctr = c->ctr;
@@ -1515,6 +1515,22 @@ gi_status gi_cache_export(gi_cache_t c, gi_cell *out, uint64_t capacity, uint64_
         cells.push_back(cell);
     }
     return export_sorted(cells, out, capacity, count, "gi_cache_export");
+}
+
+gi_status gi_diag_dense_cells(gi_cache_t c, uint64_t *cells, gi_stream_t stream) {
+    if (!c || !cells) {
+        set_error("gi_diag_dense_cells: NULL argument");
+        return GI_ERR_INVALID_ARG;
+    }
+    std::vector<RankWord> rank(c->rank ? c->N / 32 : 0);
+    gi_status s = cuda_status(cudaStreamSynchronize((cudaStream_t)stream), "gi_diag_dense_cells");
+    if (s == GI_OK && c->rank)
+        s = cuda_status(cudaMemcpy(rank.data(), c->rank, rank.size() * sizeof(RankWord), cudaMemcpyDeviceToHost),
+                        "gi_diag_dense_cells");
+    if (s != GI_OK) return s;
+    *cells = 0;
+    for (const RankWord &r : rank) *cells += (uint64_t)__builtin_popcount(r.keep);
+    return GI_OK;
 }
 
 gi_status gi_cache_export_tiles(gi_cache_t c, gi_tile *out, uint64_t capacity, uint64_t *count, gi_stream_t stream) {

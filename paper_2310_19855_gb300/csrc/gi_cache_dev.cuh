@@ -198,6 +198,7 @@ __device__ __forceinline__ void resolve_part_done(Counters *ctr, uint32_t *occ_o
         ctr->touch_count = 0u;
         ctr->ticket = 0u;
         ctr->dense_next = 0u;
+        ctr->resolves += 1u;
         // occupancy for the host's compaction decision, then the frame it belongs to
         if (occ_out) {
             reinterpret_cast<volatile uint32_t *>(occ_out)[0] = atomicAdd(&ctr->occupied, 0u);

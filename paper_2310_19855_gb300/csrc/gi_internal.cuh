@@ -33,7 +33,8 @@ struct __align__(128) Counters {
     unsigned long long clamped;
     uint32_t error_word;
     uint32_t dense_next;    // dense accumulators handed out by the resolve under way
-    uint32_t pad[22];
+    uint32_t resolves;      // resolves so far (the aging of the dense accumulators)
+    uint32_t pad[21];
 };
 
 // Per-view constants of the cell descriptor (Algorithm 6 + LOD reading).
@@ -132,7 +133,6 @@ struct ResolveArgs {
     Accum *accum;
     Accum *dense;         // large tables (else NULL): see UpdateArgs
     RankWord *rank;
-    uint32_t age;         // this resolve keeps dense accumulators only for the recently touched slots
     uint32_t *stamps;     // large float16 tables: stamps by slot
     uint32_t *cold;       // large tables: cells whose last resolve found no history, one bit each
     void *resolved;

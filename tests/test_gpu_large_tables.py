@@ -92,3 +92,36 @@ def test_few_cells_of_a_large_table_do_not_share_a_line():
     # eight cells, a million records: with their accumulators in one 256-byte run 526 us, now 92 (over 2^20 slots 110)
     rec = gather(1_000_000, 8, 3)
     assert update_us(dict(log2_slots=22), rec) < 2.5 * update_us(dict(log2_slots=20), rec)
+
+
+def test_a_captured_resolve_ages():
+    # cells of set B, touched before the replays only, must lose their side-by-side accumulators
+    a, b = dev(wl.records_random(20_011, 1, extent=3.0)), dev(wl.records_random(50_021, 2, extent=9.0))
+    h = gi.gi_cache_create(21, cell_size=0.05, evict_frames=1 << 20)
+    try:
+        st = torch.cuda.Stream()
+        s = torch.empty(20_011, dtype=torch.int32, device="cuda")
+        n = a.shape[1]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            _update(h, a, 0)
+            gi.gi_cache_resolve(h, 0)
+            torch.cuda.synchronize()
+            only_a = gi.gi_diag_dense_cells(h)
+            assert 0 < only_a <= n
+            _update(h, b, 0)
+            gi.gi_cache_resolve(h, 0)
+        torch.cuda.synchronize()
+        assert gi.gi_diag_dense_cells(h) > 2 * only_a
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st, capture_error_mode="relaxed"):
+            gi.gi_cache_update(h, gi.hits_from_planes(a, n), _view(0), s, stream=st)
+            gi.gi_cache_resolve(h, 0, stream=st)
+        for _ in range(16):
+            graph.replay()
+        torch.cuda.synchronize()
+        assert gi.gi_diag_dense_cells(h) == only_a
+        got = gi.gi_cache_export(h)
+        assert np.all(got["count"] == 0)
+    finally:
+        gi.gi_cache_destroy(h)
