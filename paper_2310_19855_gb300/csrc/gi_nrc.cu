@@ -325,8 +325,9 @@ __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
 // are read once per group.  A block takes a contiguous run of such items, so that the records of an
 // SM are neighbours too.  The gathers are bound by the sectors the L2 delivers (45 % of them hit the
 // L1 with a thread per record and level), so what counts is how many the L1 answers.  Groups of 16, 8, 4
-// or 2 levels, the longest that leave every resident warp an item; fewer records take k_nrc_encode's
-// form.  On the far hits of a 1080p frame the frame took 366, 363 and 396 us on three scenes, against
+// or 2 levels, the longest whose busiest warp takes at most 8/7 of the fewest levels that any length gives it
+// (230,400 records are 1.2 items of 16 levels a warp: the query frame 102 us so, 78 us with 4.7 items of 4);
+// fewer records take k_nrc_encode's form.  On the far hits of a 1080p frame the frame took 366, 363 and 396 us on three scenes, against
 // 381, 368 and 417 us with k_nrc_encode's form (random samples and points: 3 us slower, so they keep
 // theirs).  48 registers, 5 blocks per SM: at 6 blocks the eight gathers of a level no longer fly
 // together, 32 us slower.
@@ -336,10 +337,20 @@ __global__ void __launch_bounds__(kEncThreads, kEncBlocksPerSm) k_nrc_encode_que
     const uint32_t T = 1u << a.geo.log2_table;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     // log2 of the levels per group
-    const uint32_t want = gridDim.x * (kEncThreads / 32), ng = n / 32u;
-    const uint32_t glog = ng >= want ? 4u : (2u * ng >= want ? 3u : (4u * ng >= want ? 2u : (8u * ng >= want ? 1u : 0u)));
-    const uint32_t lgs = kL >> glog;  // level groups
     const uint32_t n_pad = (n + kTile - 1) / kTile * kTile;
+    uint32_t glog = 0;
+    if (n / 32u * 8u >= gridDim.x * (kEncThreads / 32)) {
+        uint32_t best = 0xFFFFFFFFu;
+#pragma unroll
+        for (uint32_t g = 1; g <= 4; ++g) {
+            // levels that the busiest warp takes
+            const uint32_t runs = (n_pad / 32u * (kL >> g) + kEncThreads / 32 - 1) / (kEncThreads / 32);
+            const uint32_t levels = ((runs + gridDim.x - 1) / gridDim.x) << g;
+            if (g == 1 || 7u * levels <= 8u * best) glog = g;
+            best = min(best, levels);
+        }
+    }
+    const uint32_t lgs = kL >> glog;  // level groups
     const uint32_t items = glog ? n_pad / 32u * lgs : n_pad / 2u;
     // contiguous runs of 8 items (one per warp) per block, as even as they divide
     const uint32_t rounds = (items + kEncThreads / 32 - 1) / (kEncThreads / 32);

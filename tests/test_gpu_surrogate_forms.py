@@ -76,3 +76,8 @@ def test_answers_of_a_view_equal_the_inference_of_their_points(n):
     finally:
         gi.gi_nrc_destroy(nrc)
         gi.gi_cache_destroy(cache)
+
+
+def test_answers_in_groups_of_16_levels_equal_the_inference_of_their_points():
+    # 741,000 answers: their groups of 16 levels are four items a warp, no longer run than shorter groups'
+    test_answers_of_a_view_equal_the_inference_of_their_points(780_003)
