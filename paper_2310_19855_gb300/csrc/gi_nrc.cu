@@ -930,9 +930,9 @@ struct AdamTableArgs {
     float2 *grad;
     __half2 *tab16;
     uint32_t log2_table;
-    uint32_t chunk0[kL + 1];  // first chunk of kAdamChunk entries of each level, then their number
+    uint32_t chunk0[kL + 1];  // first chunk of entries of each level, then their number
 };
-constexpr int kAdamWarps = 8, kAdamChunk = 256, kAdamBlocksPerSm = 4;
+constexpr int kAdamWarps = 8, kAdamBlocksPerSm = 4;
 
 // Sparse Adam on the table: an entry whose gradient is (0, 0) this step keeps its value and its
 // moments (the samples of the step did not touch it); the others take an Adam step with the
@@ -941,7 +941,10 @@ constexpr int kAdamWarps = 8, kAdamChunk = 256, kAdamBlocksPerSm = 4;
 // gradients of 256 consecutive entries (four 16-byte loads a lane in flight), lists the touched ones in
 // shared memory and updates the list lane by lane, so that every lane holds an entry's loads and
 // arithmetic instead of one in eight (4 entries a thread, skipping the untouched: 40 us a step of 16,384
-// samples, 2^19 entries a level; this form with the weights 27.5 us).
+// samples, 2^19 entries a level; this form with the weights 27.5 us).  Where that leaves resident warps
+// without a chunk, a warp takes 64 entries: small tables are touched all over, and a warp's 256 follow one
+// another in four trips (10,000 samples, 2^14 entries a level, backward and step: 47 us with 256, 34.5 with 64).
+template <int CHUNK>
 __device__ __forceinline__ void adam_table(const AdamTableArgs &t, const AdamArgs &a, uint32_t warp, uint32_t warps,
                                            float2 *s_g, uint16_t *s_i) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -952,14 +955,14 @@ __device__ __forceinline__ void adam_table(const AdamTableArgs &t, const AdamArg
         uint32_t first = t.chunk0[0];
 #pragma unroll
         for (int k = 1; k < kL; ++k) first = c >= t.chunk0[k] ? t.chunk0[k] : first;
-        const size_t e0 = ((size_t)l << t.log2_table) + (size_t)(c - first) * kAdamChunk;
+        const size_t e0 = ((size_t)l << t.log2_table) + (size_t)(c - first) * CHUNK;
         float4 *gq = reinterpret_cast<float4 *>(t.grad + e0);
-        float4 g[kAdamChunk / 64];
+        float4 g[CHUNK / 64];
 #pragma unroll
-        for (int j = 0; j < kAdamChunk / 64; ++j) g[j] = __ldcg(gq + 32 * j + lane);
+        for (int j = 0; j < CHUNK / 64; ++j) g[j] = __ldcg(gq + 32 * j + lane);
         uint32_t hit = 0;
 #pragma unroll
-        for (int j = 0; j < kAdamChunk / 64; ++j) {
+        for (int j = 0; j < CHUNK / 64; ++j) {
             if (g[j].x != 0.0f || g[j].y != 0.0f) hit |= 1u << (2 * j);
             if (g[j].z != 0.0f || g[j].w != 0.0f) hit |= 2u << (2 * j);
             if ((hit >> (2 * j)) & 3u) gq[32 * j + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -974,7 +977,7 @@ __device__ __forceinline__ void adam_table(const AdamTableArgs &t, const AdamArg
         const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
         int pos = incl - cnt;
 #pragma unroll
-        for (int j = 0; j < kAdamChunk / 64; ++j) {
+        for (int j = 0; j < CHUNK / 64; ++j) {
             if ((hit >> (2 * j)) & 1u) {
                 s_i[pos] = (uint16_t)(64 * j + 2 * lane);
                 s_g[pos++] = make_float2(g[j].x, g[j].y);
@@ -1066,13 +1069,14 @@ struct AdamWeightArgs {
     float *stats;
 };
 constexpr int kAdamWBlocks = (kWCount + 3 + 31) / 32;
+template <int CHUNK>
 __global__ void __launch_bounds__(32 * kAdamWarps, kAdamBlocksPerSm) k_nrc_adam(AdamTableArgs t, AdamWeightArgs q, AdamArgs a) {
     const uint32_t bid = blockIdx.x + pass_begin();
-    __shared__ float2 s_g[kAdamWarps][kAdamChunk];
-    __shared__ uint16_t s_i[kAdamWarps][kAdamChunk];
+    __shared__ float2 s_g[kAdamWarps][CHUNK];
+    __shared__ uint16_t s_i[kAdamWarps][CHUNK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (bid >= kAdamWBlocks) {
-        adam_table(t, a, (bid - kAdamWBlocks) * kAdamWarps + w, (gridDim.x - kAdamWBlocks) * kAdamWarps, s_g[w],
+        adam_table<CHUNK>(t, a, (bid - kAdamWBlocks) * kAdamWarps + w, (gridDim.x - kAdamWBlocks) * kAdamWarps, s_g[w],
                    s_i[w]);
         return;
     }
@@ -1676,17 +1680,19 @@ static gi_status adam_step(gi_nrc_s *nrc, int parts, cudaStream_t s) {
     at.grad = nrc->grad;
     at.tab16 = nrc->tab16;
     at.log2_table = nrc->cfg.log2_table;
+    const uint32_t resident = (uint32_t)nrc->sms * kAdamBlocksPerSm * kAdamWarps;
+    const uint32_t chunk = ((uint64_t)kL << nrc->cfg.log2_table) <= 128ull * resident ? 64u : 256u;
     at.chunk0[0] = 0;
     for (int l = 0; l < kL; ++l) {
         // a dense level's samples reach its first 6 (R + 1)^3 entries; gradients the caller wrote, all
         const uint64_t V = (uint64_t)nrc->geo.lv.res[l] + 1u;
         const uint64_t used = nrc->geo.lv.dense[l] && !nrc->grads_set ? 6u * V * V * V : nrc->T;
-        at.chunk0[l + 1] = at.chunk0[l] + (uint32_t)((used + kAdamChunk - 1) / kAdamChunk);
+        at.chunk0[l + 1] = at.chunk0[l] + (uint32_t)((used + chunk - 1) / chunk);
     }
     nrc->grads_set = false;
     const AdamWeightArgs aw = {nrc->w, nrc->wm, nrc->wv, nrc->wg, nrc->wimg, nrc->wpart, parts, nrc->stats};
     const unsigned blocks = std::min<uint32_t>((at.chunk0[kL] + kAdamWarps - 1) / kAdamWarps, (uint32_t)nrc->sms * kAdamBlocksPerSm);
-    launch(k_nrc_adam, kAdamWBlocks + blocks, 32 * kAdamWarps, 0, s, at, aw, a);
+    launch(chunk == 64u ? k_nrc_adam<64> : k_nrc_adam<256>, kAdamWBlocks + blocks, 32 * kAdamWarps, 0, s, at, aw, a);
     return cuda_status(cudaGetLastError(), "k_nrc_adam launch");
 }
 

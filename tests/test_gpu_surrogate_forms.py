@@ -81,3 +81,32 @@ def test_answers_of_a_view_equal_the_inference_of_their_points(n):
 def test_answers_in_groups_of_16_levels_equal_the_inference_of_their_points():
     # 741,000 answers: their groups of 16 levels are four items a warp, no longer run than shorter groups'
     test_answers_of_a_view_equal_the_inference_of_their_points(780_003)
+
+
+@pytest.mark.parametrize("log2", [13, 16])
+def test_adam_steps_the_listed_entries_of_either_chunk(log2):
+    # 64 entries a warp for small tables, 256 for others; a first step moves a touched entry by lr g / (|g| + eps)
+    # (float32: half an ulp of |p| < 1, and 2^-20 of the step), the others not at all
+    lr, eps, T = 1e-2, 1e-15, 1 << log2
+    rng = np.random.default_rng(7)
+    table, w1, w2, w3 = SI.params(3, log2)
+    grad = np.zeros(table.shape, np.float32)
+    hit = rng.random((16, T)) < 0.1
+    hit[3] = True
+    hit[5], hit[6] = False, np.arange(T) % 64 == 63
+    grad[hit] = rng.normal(size=(int(hit.sum()), 2)).astype(np.float32)
+    cfg = gi.make_nrc_config(*SI.CORNELL_AABB, log2_table=log2, resolutions=SI.SMALL_RESOLUTIONS, lr=lr, adam_eps=eps,
+                             max_records=128, max_queries=128)
+    nrc = gi.gi_nrc_create(cfg)
+    try:
+        gi.gi_nrc_set_params(nrc, table, w1, w2, w3)
+        gi.gi_nrc_set_gradients(nrc, grad, np.zeros_like(w1), np.zeros_like(w2), np.zeros_like(w3))
+        gi.gi_nrc_adam(nrc)
+        got = gi.gi_nrc_get_params(nrc, log2)[0]
+        g = grad.astype(np.float64)
+        want = table - lr * g / (np.abs(g) + eps)
+        assert np.array_equal(got[~hit], table[~hit])
+        assert np.abs(got - want).max() < 2.0 ** -24 * np.abs(want).max() + 2.0 ** -20 * lr
+        assert not np.any(gi.gi_nrc_get_gradients(nrc, log2)[0])
+    finally:
+        gi.gi_nrc_destroy(nrc)
