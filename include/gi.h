@@ -771,14 +771,15 @@ gi_status gi_cell_means_noalloc(const gi_hits *hits, const gi_view *view, float 
 /* ---------------------------------------------------------------- diagnostics
  * Not a step of the path.  gi_cache_update ends, per hit record (GI_MERGE_NONE), in L2
  * operations on the cell's 32-byte accumulator (Section 2.2.1's accumulation in 64-bit fixed
- * point): in the list form (GI_FIRST_TOUCH_LIST) three 64-bit additions of the sums and one
- * returning addition of the count, whose old value flags the first touch; in the bitmap
- * form (GI_FIRST_TOUCH_BITMAP, and AUTO) the four additions as one 32-byte request and a
- * non-returning set of the slot's bit.  gi_diag_update_atomics issues
- * those operations of the given form for n slot ids (records with slot_ids[i] >= 2^log2_slots are
- * skipped; one addition per record, as the update without merge) and nothing else: no record
- * stream, key, probe or slot-id store.  Timed beside gi_cache_update on the same frame's slot ids
- * it gives the floor of the update's accumulation on this GPU.
+ * point): the sums and the count added by four lanes as one 32-byte request.  In the list form
+ * (GI_FIRST_TOUCH_LIST) the count's addition returns its old value, which flags the first touch; in
+ * the bitmap form (GI_FIRST_TOUCH_BITMAP, and AUTO) nothing returns and the slot's bit is set.
+ * gi_diag_update_atomics issues those operations of the given form for n slot ids (records with
+ * slot_ids[i] >= 2^log2_slots are skipped; one addition per record, as the update without merge), by
+ * slot, and nothing else: no record stream, key, probe or slot-id store.  Timed beside gi_cache_update
+ * on the same frame's slot ids it gives the floor of the accumulation of a table in the list form, or
+ * of less than 2^21 slots in the bitmap form, on this GPU (larger bitmap tables add into the shorter
+ * span of the recently touched cells' accumulators and set a bit only where it is clear).
  *   slot_ids       device uint32[n] (4-byte aligned), e.g. the slot_ids_out of an update
  *   first_touch    the form: GI_FIRST_TOUCH_LIST, GI_FIRST_TOUCH_BITMAP or AUTO (the bitmap)
  *   scratch        device, caller-owned, zeroed by the caller, 32-byte aligned: 2^log2_slots

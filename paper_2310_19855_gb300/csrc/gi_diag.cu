@@ -1,12 +1,11 @@
 // Diagnostics, not a step of the path: the L2 floor of the cache update's accumulation.
 //
 // gi_cache_update ends, per hit record (the default GI_MERGE_NONE form), in L2 operations on the
-// cell's 32-byte accumulator.  List form: three 64-bit additions (the fixed-point sums) and one returning
-// addition of the count, whose old value flags the first touch.  Bitmap form: the sums and count added
-// by four lanes of the warp as one 32-byte request (warp_add_accum) and a non-returning set of the
-// slot's bit.  k_diag_atomics issues these operations for a frame's slot ids, with nothing else
-// (no record stream, key, probe or slot-id store) and by slot, so its time is the floor of the
-// accumulation of a table without dense accumulators on this GPU.
+// cell's 32-byte accumulator: the sums and count added by four lanes of the warp as one 32-byte request
+// (warp_add_accum).  List form: the count's addition returns, and its old value flags the first touch.
+// Bitmap form: a non-returning set of the slot's bit.  k_diag_atomics issues these operations for a
+// frame's slot ids, with nothing else (no record stream, key, probe or slot-id store) and by slot, so its
+// time is the floor of the accumulation of a table without dense accumulators on this GPU.
 #include "gi_cache_dev.cuh"
 
 namespace gi {
@@ -16,36 +15,26 @@ __global__ void __launch_bounds__(kUpdThreads, 8) k_diag_atomics(const uint32_t 
                                                                   uint32_t slots, Accum *acc, uint32_t *bitmap,
                                                                   uint32_t *first_out) {
     __shared__ __align__(32) unsigned long long s_red[kUpdThreads][4];
-    __shared__ uint32_t s_first;
+    __shared__ uint32_t s_touch[BITMAP ? 1 : kUpdBlockRecords], s_first;
     if (threadIdx.x == 0) s_first = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const unsigned long long stride = (unsigned long long)gridDim.x * kUpdThreads;
-    uint32_t first = 0;
     for (unsigned long long base = (unsigned long long)blockIdx.x * kUpdThreads; base < n; base += stride) {
         const unsigned long long i = base + threadIdx.x;
         const uint32_t s = i < n ? __ldcs(slot_ids + i) : GI_SLOT_NONE;
         const bool hit = s < slots;
-        if (BITMAP) {
-            if (hit) {
-                s_red[threadIdx.x][0] = 1ull;
-                s_red[threadIdx.x][1] = 2ull;
-                s_red[threadIdx.x][2] = 3ull;
-                s_red[threadIdx.x][3] = 1ull;
-                atomicOr(bitmap + (s >> 5), 1u << (s & 31u));
-            }
-            warp_add_accum(acc, nullptr, hit ? s : GI_SLOT_NONE, &s_red[threadIdx.x & ~31u][0], lane);
-        } else if (hit) {
-            Accum *a = acc + s;
-            atomicAdd(&a->sum[0], 1ull);
-            atomicAdd(&a->sum[1], 2ull);
-            atomicAdd(&a->sum[2], 3ull);
-            if (atomicAdd(&a->count, 1u) == 0u) ++first;
+        if (hit) {
+            s_red[threadIdx.x][0] = 1ull;
+            s_red[threadIdx.x][1] = 2ull;
+            s_red[threadIdx.x][2] = 3ull;
+            s_red[threadIdx.x][3] = 1ull;
+            if (BITMAP) atomicOr(bitmap + (s >> 5), 1u << (s & 31u));
         }
+        warp_add_accum<!BITMAP>(acc, nullptr, hit ? s : GI_SLOT_NONE, &s_red[threadIdx.x & ~31u][0], lane, s_touch,
+                                &s_first);
     }
     if (BITMAP) return;
-    first = __reduce_add_sync(kFull, first);
-    if (lane == 0 && first) atomicAdd(&s_first, first);
     __syncthreads();
     if (threadIdx.x == 0 && s_first) atomicAdd(first_out, s_first);
 }
