@@ -112,8 +112,9 @@ typedef void *gi_stream_t; /* cudaStream_t */
  *                   are the same).  GI_MERGE_WARP: the hits of a warp (32 consecutive records) that
  *                   name the same cell are merged first (__match_any_sync), so one of them probes
  *                   and accumulates for all.  Results are identical; the merge pays only where
- *                   consecutive records share cells.  Ignored by tile caches and by
- *                   gi_batch_frame, whose update never merges.
+ *                   consecutive records share cells, and is left out in the warps that hold more
+ *                   than half as many cells as hits.  Ignored by tile caches, which always merge
+ *                   by that rule, and by gi_batch_frame, whose update never merges.
  */
 typedef struct gi_cache_config {
     uint32_t log2_slots;
@@ -252,10 +253,12 @@ uint32_t gi_version(void);
 /*
  * Create a cache (Section 2.2.1): allocates the slot table (fingerprints,
  * 32-byte fixed-point accumulators, resolved radiance), a spare table for
- * compaction (from 2^21 slots on the second set of accumulators serves recently touched cells
- * instead, with 4 bytes of stamp per slot and table), the record of touched slots (a bitmap of one
- * bit per slot, or a touch list of 4 bytes per slot in the list form) and counters, on the
- * current CUDA device.  The library owns this memory until gi_cache_destroy.
+ * compaction, the record of touched slots (a bitmap of one bit per slot, or a touch list of 4 bytes
+ * per slot in the list form) and counters, on the current CUDA device.  Bitmap-form tables of 2^21
+ * slots and more have one set of accumulators by slot and one of 65/64 as many for the recently
+ * touched cells in place of the spare table's, 16 bytes of rank word per 32 slots in place of the
+ * bitmap, one bit of cold mark per slot and table, and with GI_RESOLVED_F16 4 bytes of stamp per slot
+ * and table.  The library owns this memory until gi_cache_destroy.
  * Synchronous.
  * Errors: GI_ERR_INVALID_ARG (cfg out of range), GI_ERR_OOM, GI_ERR_CUDA.
  */

@@ -108,12 +108,12 @@ struct Geometry {
     uint32_t log2_table;
 };
 
-enum EncMode { kEncPoints = 0, kEncSampled = 1, kEncQueries = 2 };
+enum EncMode { kEncPoints = 0, kEncSampled = 1 };  // of k_nrc_encode
 
 struct EncArgs {
     Geometry geo;
     const __half2 *tab16;
-    // points (mode kEncPoints) or records (modes kEncSampled, kEncQueries)
+    // points (kEncPoints) or records (kEncSampled, k_nrc_encode_queries)
     const float *pos[3];
     const float *nrm[3];
     const float *len;          // records: ray length (hit test)
@@ -124,7 +124,7 @@ struct EncArgs {
     uint32_t n_records, seed, offset;
     const uint32_t *slot_ids;
     CacheView cv;
-    // kEncQueries
+    // k_nrc_encode_queries
     const uint32_t *qidx;
     const uint32_t *qcount;
     // outputs
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kEncThreads) k_nrc_encode(EncArgs a) {
     }
 }
 
-// The records a view leaves to the network (kEncQueries).  A warp takes 32 consecutive ones through a
+// The records a view leaves to the network.  A warp takes 32 consecutive ones through a
 // group of consecutive levels, one level at a time: its lanes' vertices then lie in one level's table,
 // close together where the records are (they come probe by probe), and each record's position and normal
 // are read once per group.  A block takes a contiguous run of such items, so that the records of an
