@@ -71,7 +71,8 @@ def test_shared_cells_get_the_sums_of_their_records(kw, cells):
 
 
 def test_one_tile_cell_costs_no_multiple_of_many():
-    # a million additions to one address, one after the other, take a millisecond; merged by warps 54 us
+    # a million additions to one address, one after the other, take a millisecond; merged by warps 54 us,
+    # in a thousand cells 41
     n = 1_000_000
     assert update_us(dict(log2_slots=16, tiles=True), gather(n, 1, 3)) < 6 * update_us(
-        dict(log2_slots=16, tiles=True), gather(n, 100_003, 3))
+        dict(log2_slots=16, tiles=True), gather(n, 1_009, 3))
