@@ -8,12 +8,15 @@
 // time is the floor of the accumulation of a table without dense accumulators on this GPU.
 #include "gi_cache_dev.cuh"
 
+#include <algorithm>
+
 namespace gi {
 
 template <bool BITMAP>
-__global__ void __launch_bounds__(kUpdThreads, 8) k_diag_atomics(const uint32_t *slot_ids, unsigned long long n,
-                                                                  uint32_t slots, Accum *acc, uint32_t *bitmap,
-                                                                  uint32_t *first_out) {
+__global__ void __launch_bounds__(kUpdThreads, BITMAP ? 8 : 6) k_diag_atomics(const uint32_t *slot_ids,
+                                                                             unsigned long long n, uint32_t slots,
+                                                                             Accum *acc, uint32_t *bitmap,
+                                                                             uint32_t *first_out) {
     __shared__ __align__(32) unsigned long long s_red[kUpdThreads][4];
     __shared__ uint32_t s_touch[BITMAP ? 1 : kUpdBlockRecords], s_first;
     if (threadIdx.x == 0) s_first = 0;
@@ -68,7 +71,12 @@ extern "C" gi_status gi_diag_update_atomics(const uint32_t *slot_ids, uint64_t n
     const uint32_t slots = 1u << log2_slots;
     Accum *acc = static_cast<Accum *>(scratch);
     uint32_t *bits = reinterpret_cast<uint32_t *>(acc + slots);
-    const unsigned blocks = (unsigned)((n + kUpdBlockRecords - 1) / kUpdBlockRecords);
+    // the update's grids: the resident blocks, in the list form more where those would list too many touches
+    const uint32_t full = (uint32_t)((n + kUpdThreads - 1) / kUpdThreads);
+    const uint32_t blocks =
+        bitmap ? (uint32_t)resident_grid(k_diag_atomics<true>, kUpdThreads, full)
+               : std::max<uint32_t>((uint32_t)((n + kUpdBlockRecords - 1) / kUpdBlockRecords),
+                                    (uint32_t)resident_grid(k_diag_atomics<false>, kUpdThreads, full));
     cudaStream_t st = (cudaStream_t)stream;
     if (bitmap)
         k_diag_atomics<true><<<blocks, kUpdThreads, 0, st>>>(slot_ids, (unsigned long long)n, slots, acc, bits, nullptr);
