@@ -73,11 +73,11 @@ UPDATE_HEADER = ("gi_internal.cuh", "namespace gi {", "struct ResolveArgs {")
 NRC_ADAM_SECTION = ("gi_nrc.cu", "// ---------------------------------------------------------------- gradient scatter and Adam",
                     "// ---------------------------------------------------------------- query selection")
 NCU_TRAFFIC = {
-    # k_update, boxes-1080p (5th launch): 158.88 MB read + 33.17 MB written
-    "2:update": {"bytes_per_launch": 192052224, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
-                 "source_sha": "530c436e01a8c6ee"},
-    # k_nrc_adam (table and weights), Cornell 1080p: 105.84 MB read + 14.32 MB written
-    "4:adam_table": {"bytes_per_launch": 120159744, "sources": (NRC_ADAM_SECTION,), "source_sha": "04fc4aad2b956f33"},
+    # k_update, boxes-1080p (5th launch): 158.91 MB read + 33.19 MB written
+    "2:update": {"bytes_per_launch": 192099072, "sources": (UPDATE_SECTION, "gi_cache_dev.cuh", UPDATE_HEADER),
+                 "source_sha": "1328fddb83fad64f"},
+    # k_nrc_adam (table and weights), Cornell 1080p: 105.84 MB read + 14.23 MB written
+    "4:adam_table": {"bytes_per_launch": 120066560, "sources": (NRC_ADAM_SECTION,), "source_sha": "23e8805c31b8aecd"},
 }
 
 
