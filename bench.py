@@ -1750,6 +1750,13 @@ def other_configs(args, rank, world, local_rank):
     return out
 
 
+def with_summaries(line, blocks):
+    """The line with a summary of each other configuration's block: the blocks themselves go to the error
+    stream, so that the line stays short enough (about 6 KB) for a reader that keeps the output's end."""
+    short = {n: {k: b[k] for k in ("value", "unit", "steps", "ms_per_step") if k in b} for n, b in blocks.items()}
+    return dict(line, configs=short)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1764,7 +1771,8 @@ def main():
                          "configuration's 128); configuration 3: training rounds of the per-view networks "
                          "(default 2048); block 4-far: frames of online training (default 2048)")
     ap.add_argument("--no-other-configs", action="store_true",
-                    help="configuration 2: skip the compact runs of configurations 3-7 added to its line")
+                    help="configuration 2: skip the compact runs of configurations 3-7 (one JSON line each on the "
+                         "error stream, summaries in the output line)")
     ap.add_argument("--config", type=int, default=2, choices=[2, 3, 4, 5, 6, 7],
                     help="2: boxes at 1080p (default); 3: 16 batched views; 4: Cornell box at 1080p with the "
                          "learned surrogate; 5: boxes at 4K, 2^24 slots, FP16 resolved radiance; 6: boxes at "
@@ -1787,7 +1795,10 @@ def main():
     try:
         line = run_config(CONFIG, args, rank, world, local_rank)
         if line is not None and CONFIG == 2 and world == 1 and not args.no_other_configs:
-            line["configs"] = other_configs(args, rank, world, local_rank)
+            blocks = other_configs(args, rank, world, local_rank)
+            for name, block in blocks.items():
+                print(json.dumps({"configuration": name, **block}), file=sys.stderr, flush=True)
+            line = with_summaries(line, blocks)
         if line is not None:
             print(json.dumps(line), flush=True)
     finally:

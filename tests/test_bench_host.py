@@ -44,3 +44,10 @@ def test_comment_edits_keep_the_hash_and_code_edits_change_it(tmp_path, monkeypa
     # a change outside the section leaves the update's record alone
     p.write_text(text + "\n// trailing note\nstatic int unrelated_symbol = 0;\n")
     assert bench._source_sha(srcs) == h0
+
+
+def test_the_output_line_holds_summaries_of_the_other_configurations():
+    block = {"value": 1.5, "unit": "x", "steps": 3, "ms_per_step": 0.25, "pass_ms": {"update": 0.1}, "e2e": {"value": 2}}
+    line = bench.with_summaries({"value": 9}, {"5": block, "3": dict(block, value=2.5)})
+    assert line["value"] == 9 and set(line["configs"]) == {"5", "3"}
+    assert line["configs"]["3"] == {"value": 2.5, "unit": "x", "steps": 3, "ms_per_step": 0.25}
