@@ -232,23 +232,26 @@ __global__ void __launch_bounds__(1024) k_mip_tail(uint32_t *mask, MipInfo mi) {
 
 // ---------------------------------------------------------------- probe irradiance
 
-// Plain loads, as the slot ids of the general form below: the compiler orders them more freely than the
-// cache-operator loads.  128 rays per probe at 641 x 359 took 18.3 us with those, 10.9 so; 256 rays at
-// 1080p 45.0 and 41.4.
+// PLAIN: plain loads, which the compiler orders more freely than the cache-operator loads (as the slot ids of
+// the general form below): 128 rays per probe at 641 x 359 took 18.3 us with those, 10.9 so; 256 rays at 1080p
+// 45.0 and 41.4; 64 rays 17.2 and 16.9, at 4K with float16 storage 114 and 78.  The gathers of the atlas and
+// the batched pass of 64 rays keep the others (16 views: 187 us against 201 with plain loads).
+template <bool PLAIN>
 __device__ __forceinline__ float3 fetch_resolved(const void *r, uint32_t stride, int f16, uint32_t s) {
     r = static_cast<const char *>(r) + (size_t)s * stride;
     if (f16) {
-        const ushort4 h = ld(reinterpret_cast<const ushort4 *>(r));
+        const ushort4 h = PLAIN ? ld(reinterpret_cast<const ushort4 *>(r)) : __ldca(reinterpret_cast<const ushort4 *>(r));
         return make_float3(__half2float(__ushort_as_half(h.x)), __half2float(__ushort_as_half(h.y)),
                            __half2float(__ushort_as_half(h.z)));
     }
-    const float4 v = ld(reinterpret_cast<const float4 *>(r));
+    const float4 v = PLAIN ? ld(reinterpret_cast<const float4 *>(r)) : __ldca(reinterpret_cast<const float4 *>(r));
     return make_float3(v.x, v.y, v.z);
 }
 
+template <bool PLAIN>
 __device__ __forceinline__ bool ray_sample(const IntegrateArgs &a, uint32_t s, float3 &r) {
     if (s < a.slots) {
-        r = fetch_resolved(a.resolved, a.res_stride, a.f16, s);
+        r = fetch_resolved<PLAIN>(a.resolved, a.res_stride, a.f16, s);
         return true;
     }
     r = make_float3(a.env[0], a.env[1], a.env[2]);
@@ -283,7 +286,7 @@ __device__ __forceinline__ void gather_cells(const IntegrateArgs &a, uint32_t p,
         if (k != (uint32_t)lane) ray = load_rays(a, (size_t)p * a.rpp + k);
         // rays k and k + 32 sample cells lane and lane + 32; both gathers in flight together
         float3 r0, r1;
-        const bool h0 = ray_sample(a, ray.s0, r0), h1 = ray_sample(a, ray.s1, r1);
+        const bool h0 = ray_sample<false>(a, ray.s0, r0), h1 = ray_sample<false>(a, ray.s1, r1);
         if (h0) {
             acc[0][0] += r0.x; acc[0][1] += r0.y; acc[0][2] += r0.z; cnt[0] += 1.0f;
         }
@@ -384,7 +387,7 @@ __device__ __forceinline__ void load_moment_table(float *s_mom) {
     }
 }
 
-template <bool SURR, bool RPC1>
+template <bool SURR, bool RPC1, bool PLAIN>
 __device__ __forceinline__ void integrate_quad(const IntegrateArgs &a, uint32_t p, bool valid, const float *s_mom) {
     const int h = threadIdx.x & 3;
     float4 n4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -433,7 +436,7 @@ __device__ __forceinline__ void integrate_quad(const IntegrateArgs &a, uint32_t 
                 float3 r[kIntPass];
                 bool hs[kIntPass];
 #pragma unroll
-                for (int i = 0; i < kIntPass; ++i) hs[i] = ray_sample(a, sl[i], r[i]);
+                for (int i = 0; i < kIntPass; ++i) hs[i] = ray_sample<PLAIN>(a, sl[i], r[i]);
                 if (SURR) {
                     // records rec0 + i, rec0 = (p rpp + 64 j + 16 h + i0): bits 16 (h & 1) + i0 + i of
                     // the answer word of the 32 records starting at the probe's 64 j + 32 (h >> 1)
@@ -518,10 +521,10 @@ __device__ __forceinline__ void integrate_quad(const IntegrateArgs &a, uint32_t 
 // blk: block of kIntThreads / 4 probes (the batched pass passes the view-local block).  RPC1: 64
 // rays per probe (one per cell), a kernel of its own so that the general form's registers do not
 // weigh on it.
-template <bool SURR, bool RPC1>
+template <bool SURR, bool RPC1, bool PLAIN = true>
 __device__ __forceinline__ void integrate_body(const IntegrateArgs &a, uint32_t blk, const float *s_mom) {
     const uint32_t p = blk * (blockDim.x >> 2) + (threadIdx.x >> 2);
-    integrate_quad<SURR, RPC1>(a, p, p < a.probes, s_mom);
+    integrate_quad<SURR, RPC1, PLAIN>(a, p, p < a.probes, s_mom);
 }
 
 template <bool RPC1>
@@ -1336,7 +1339,7 @@ __global__ void __launch_bounds__(128, 4) k_integrate_batched(const IntegrateArg
     __shared__ IntegrateArgs sa;
     __shared__ __align__(16) float s_mom[64 * kMomStride];
     load_moment_table<true>(s_mom);
-    GI_BATCHED_ITEMS(prefix, nviews, sa, args, (integrate_body<false, RPC1>(sa, item, s_mom)));
+    GI_BATCHED_ITEMS(prefix, nviews, sa, args, (integrate_body<false, RPC1, !RPC1>(sa, item, s_mom)));
 }
 
 __global__ void __launch_bounds__(32 * kInterpWarps, kInterpBlocksPerSm) k_interpolate_batched(const InterpArgs *args, const uint32_t *prefix,
