@@ -14,7 +14,7 @@
 // accumulations over more memory than the L2 holds, and their cost follows that span (2.07 M
 // random additions of 32 bytes: 27 us over 2^20 slots, 53 us over 2^22, 80 us over 2^24, 86 us over
 // 2^25).  They therefore keep, beside `accum`:
-//   dense    Accum[N]        accumulators of the cells touched lately, side by side
+//   dense    Accum[65/64 N]  accumulators of the cells touched lately, side by side
 //   rank     RankWord[N/32]  which slots those are, the first one's place, the touched bits
 //   cold     u32[N/32]       the cold marks
 // and the stamps in the resolved float4's w, or with float16 storage in an array u32[N] (accum's stamp
@@ -307,10 +307,10 @@ static inline int list_update_blocks(unsigned long long n, uint32_t resident) {
 // when a thread walked its own word's bits 4 at a time with 3 blocks per SM: a word holds 0 to 32
 // touched slots, so those threads' chains were as uneven as their words.)
 // Large tables start at 2^21 slots (64 MB of accumulators, half of the L2).  At 2^22 the frame's update
-// fell from 62 to 55 us and its resolve stayed at 34 us; at 2^24 the update fell from 370 to 281 us and
-// the resolve from 135 to 97 us (both 1 ray a cell, 1080p and 4K); at 2^21 the cache's calls on 777777
-// records fell from 71.2 to 66.0 us and 16 views of 2^20 and 2^21 slots from 1291 to 1248 us.  At 2^20 the rank
-// loads cost what the shorter span gives (the same calls at 1249 us).
+// fell from 62 to 55 us and its resolve from 34 to 25; at 2^24 the update from 370 to 264 us and the resolve
+// from 135 to 94 (both 1 ray a cell, 1080p and 4K); at 2^21 the cache's calls on 777,777 records take 65 us
+// and 72 by slot, 16 views of 2^20 and 2^21 slots 1228 and 1280 us.  At 2^20 slots the rank words cost what the
+// shorter span gives: update and resolve of 777,777 records 28.8 and 30.8 us, of 100,000 14.9 and 12.8.
 constexpr uint32_t kDenseLog2Slots = 21, kDenseAge = 8;
 constexpr int kResListUnroll = 2, kResListBlocksPerSm = 4;
 constexpr int kResBmUnroll = 2, kResBmBlocksPerSm = 4, kResBmWords = 16;
